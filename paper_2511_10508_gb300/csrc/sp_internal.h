@@ -88,8 +88,8 @@ inline int steps_per_launch(int dims, int dtype, int model, int requested) {
 }
 
 // 3D FP64 27-point Allen-Cahn, Cahn-Hilliard (two passes through `mu`, N
-// doubles) and Gray-Scott with x-pair sums shared between y neighbours: kernel
-// family 0 of these grids.  Family 2 is then the z-streaming kernel with plane
+// doubles), Gray-Scott and Model C with x-pair sums shared between y neighbours:
+// kernel family 0 of these grids.  Family 2 (not for Model C) is then the z-streaming kernel with plane
 // sums in registers (step3d_zreg_kernel, family 0 of launch_step_f64), family 1
 // the accessor-based plane ring.
 constexpr int kZregFamily = 2;
@@ -104,7 +104,7 @@ inline bool twopass_applies(int dims, int dtype, int stencil, int model) {
 }
 inline bool planes27_applies(int dims, int dtype, int stencil, int model) {
     return dims == 3 && dtype == SP_F64 && stencil == SP_LAP_27 &&
-           (model == SP_ALLEN_CAHN || model == SP_CAHN_HILLIARD || model == SP_GRAY_SCOTT);
+           (model == SP_ALLEN_CAHN || model == SP_CAHN_HILLIARD || model == SP_GRAY_SCOTT || model == SP_MODEL_C);
 }
 
 // Tensor-map (TMA) plane loads (sp_tma.cu): kernel family kTmaFamily of 3D

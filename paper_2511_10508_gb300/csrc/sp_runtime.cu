@@ -500,7 +500,8 @@ static std::vector<TuneChoice> tune_candidates(const sp_sim *s) {
         if (s->dims == 3 && s->dtype != SP_F64 && s->model != SP_MODEL_C && s->nx % (int)(16 / s->esize) == 0 &&
             tma_available())
             c.push_back({1, kTmaFamily});
-        if (planes27_applies(s->dims, s->dtype, s->stencil, s->model)) c.push_back({1, kZregFamily});
+        if (planes27_applies(s->dims, s->dtype, s->stencil, s->model) && s->model != SP_MODEL_C)
+            c.push_back({1, kZregFamily});
         if (s->dims == 3 && steps_per_launch_3d(s->dtype, s->model, s->nx, 2) == 2) {
             c.push_back({2, 0});  // two steps per pass, 8 rows
             c.push_back({2, 1});  // 16 rows

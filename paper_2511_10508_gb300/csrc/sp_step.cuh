@@ -1135,8 +1135,10 @@ __global__ void __launch_bounds__(NT) step3d_zreg_kernel(StepArgs a, int tiles_x
 // point; mode 1: the update from mu and the centre phi), so mu is evaluated
 // once per point rather than on a halo ring as well; the buffer's HBM traffic
 // (16 bytes per point) is cheap next to the FP64 work on this part.  Allen-Cahn
-// (mode 2) and Gray-Scott (mode 3) take one pass.  Same operations in the same
-// order as every other family, so the results are identical bit for bit.
+// (mode 2), Gray-Scott (mode 3) and Model C (mode 4: phi and the density's chemical
+// potential, formed once per loaded point, are streamed; rho itself is read at the
+// output points) take one pass.  Tiles of 32 x 32, or 32 x 16 where the grid's edges
+// waste too much of the larger (small_tile).  Same operations in the same order as every other family, so the results are identical bit for bit.
 // The default for these grids; measured on GB300 against step3d_zreg_kernel:
 // Cahn-Hilliard 1024^3 17.5 vs 13.6 GLUPS, Allen-Cahn 512^3 29.6 vs 27.0,
 // Gray-Scott 512^3 14.9 vs 13.3.
@@ -1148,10 +1150,10 @@ struct Planes27Args {
     StepConsts k;
 };
 
-template <int MODE>
+template <int MODE, int TY_>
 struct Planes27Shape {
-    static constexpr int NF = (MODE == 3) ? 2 : 1;
-    static constexpr int TX = 32, TY = 32, NT = 256;
+    static constexpr int NF = (MODE >= 3) ? 2 : 1;
+    static constexpr int TX = 32, TY = TY_, NT = 8 * TY;
     static constexpr int WIN = TX + 2, HIN = TY + 2, AIN = WIN * HIN;
     static constexpr int AP = HIN * TX;                // pair sums of rows -1 .. TY
     static constexpr int EPT = (AIN + NT - 1) / NT;    // loaded cells per thread per field
@@ -1159,10 +1161,10 @@ struct Planes27Shape {
     static constexpr size_t smem_bytes = sizeof(double) * ((size_t)2 * NF * AIN + (size_t)NF * AP);
 };
 
-template <int MODE>
-__global__ void __launch_bounds__(256, MODE == 3 ? 1 : 2)
+template <int MODE, int TY_>
+__global__ void __launch_bounds__(8 * TY_, (MODE >= 3 ? 1 : 2) * 32 / TY_)
     planes27_kernel(Planes27Args a, int tiles_x, long long planes_per_cta, long long total) {
-    typedef Planes27Shape<MODE> Sh;
+    typedef Planes27Shape<MODE, TY_> Sh;
     constexpr int NF = Sh::NF, TX = Sh::TX, TY = Sh::TY, NT = Sh::NT, WIN = Sh::WIN, AIN = Sh::AIN, AP = Sh::AP;
     constexpr int EPT = Sh::EPT, EOUT = Sh::EOUT, OSTEP = Sh::OSTEP;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1213,7 +1215,9 @@ __global__ void __launch_bounds__(256, MODE == 3 ? 1 : 2)
             for (int f = 0; f < NF; ++f)
 #pragma unroll
                 for (int e = 0; e < EPT; ++e)
-                    if (loff[e] >= 0) buf[(size_t)f * AIN + t + e * NT] = pf[f][e];
+                    if (loff[e] >= 0)
+                        buf[(size_t)f * AIN + t + e * NT] =
+                            (MODE == 4 && f == 1) ? mc_mu<double>(pf[0][e], pf[NF - 1][e], k) : pf[f][e];
             if (j + 1 < nplanes) fetch(z0 + j);
             __syncthreads();
 #pragma unroll
@@ -1255,7 +1259,8 @@ __global__ void __launch_bounds__(256, MODE == 3 ? 1 : 2)
                         a.out[0][o] = ac_update<double>(fc[0], S[0], k);
                     } else {
                         double un, vn;
-                        gs_update<double>(fc[0], fc[1], S[0], S[1], k, un, vn);
+                        if constexpr (MODE == 3) gs_update<double>(fc[0], fc[NF - 1], S[0], S[NF - 1], k, un, vn);
+                        else mc_update<double>(fc[0], a.in[1][o], S[0], S[NF - 1], k, un, vn);
                         a.out[0][o] = un;
                         a.out[1][o] = vn;
                     }
@@ -1278,10 +1283,10 @@ __global__ void __launch_bounds__(256, MODE == 3 ? 1 : 2)
 // S + 1): the fused kernel also evaluates mu on a halo ring of the tile.  The
 // default for these grids; measured on GB300 at 1024^3 against the fused
 // kernel: 7-point 29.6 vs 27.2 GLUPS, 13-point 17.7 vs 14.3.
-template <int ST>
+template <int ST, int TY_>
 struct Ring2PassShape {
     static constexpr int R = StencilInfo<ST>::r;
-    static constexpr int TX = 32, TY = 32, NT = 256;
+    static constexpr int TX = 32, TY = TY_, NT = 8 * TY;
     static constexpr int WIN = TX + 2 * R, HIN = TY + 2 * R, AIN = WIN * HIN;
     static constexpr int D = 2 * R + 2;
     static constexpr int EPT = (AIN + NT - 1) / NT;
@@ -1289,10 +1294,10 @@ struct Ring2PassShape {
     static constexpr size_t smem_bytes = sizeof(double) * (size_t)D * AIN;
 };
 
-template <int ST, int MODE>
-__global__ void __launch_bounds__(256, 2)
+template <int ST, int MODE, int TY_>
+__global__ void __launch_bounds__(8 * TY_, 64 / TY_)
     ring2pass_kernel(Planes27Args a, int tiles_x, long long planes_per_cta, long long total) {
-    typedef Ring2PassShape<ST> Sh;
+    typedef Ring2PassShape<ST, TY_> Sh;
     constexpr int R = Sh::R, TX = Sh::TX, NT = Sh::NT, WIN = Sh::WIN, AIN = Sh::AIN, D = Sh::D;
     constexpr int EPT = Sh::EPT, EOUT = Sh::EOUT, OSTEP = Sh::OSTEP;
     extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -38,6 +38,12 @@ cudaError_t launch_planes27_f64(int model, const StepArgs &a, void *mu, cudaStre
         p.out[0] = out0;
         p.out[1] = out1;
         return launch_planes27_mode<3>(p, s, n_sm);
+    case MC:
+        p.in[0] = in0;
+        p.in[1] = in1;
+        p.out[0] = out0;
+        p.out[1] = out1;
+        return launch_planes27_mode<4>(p, s, n_sm);
     default:
         return cudaErrorInvalidValue;
     }

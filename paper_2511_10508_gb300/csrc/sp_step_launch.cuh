@@ -15,27 +15,49 @@
 
 namespace sp {
 
-// 3D tiles (x, y) per storage type and stencil radius.
-template <typename T> struct Tiles;
-template <> struct Tiles<double> {
-    template <int r> struct T3 { static constexpr int TX = (r == 1) ? 64 : 32, TY = 32, NT = 256; };
-};
-template <> struct Tiles<float> {
-    template <int r> struct T3 { static constexpr int TX = 64, TY = 16, NT = 256; };
-};
-template <> struct Tiles<bf16> {
-    template <int r> struct T3 { static constexpr int TX = 64, TY = 16, NT = 256; };
-};
+// 3D FP64 tiles (x, y) per stencil radius, and the small tile for grids that the large
+// one covers badly.
+template <int r> struct Tiles64 { static constexpr int TX = (r == 1) ? 64 : 32, TY = 32, NT = 256; };
+constexpr int kSmallTX = 32, kSmallTY = 16, kSmallNT = 128;
 
-constexpr int kMinRun = 32;
+// The small tile wins where the large one's ragged edges cost more than a tenth in
+// points (both evaluate whole tiles), e.g. 71 x 35: 3 x 2 tiles of 32 x 32 against 3 x 3
+// of 32 x 16.  On whole tiles the large one reads fewer halo cells per point.
+inline bool small_tile(int nx, int ny, int TX, int TY) {
+    auto area = [&](int tx, int ty) {
+        return (double)((nx + tx - 1) / tx) * tx * ((double)((ny + ty - 1) / ty) * ty);
+    };
+    return area(kSmallTX, kSmallTY) < 0.9 * area(TX, TY);
+}
+
+constexpr int kMinRun = 32;  // 2D warp strips: rows per CTA at least
 constexpr size_t kMaxSmemPerCta = 227 * 1024;  // opt-in maximum of dynamic shared memory per CTA
 
-// Persistent grids: one resident wave of CTAs (SMs x occupancy), each owning an
-// equal share of the flattened (tile, slow-axis) work, but at least kMinRun
-// slices per CTA so that the halo slices of each segment stay a small fraction.
-inline long long persistent_ctas(long long total_slices, int ctas_per_sm, int n_sm) {
-    const long long wave = (long long)n_sm * std::max(ctas_per_sm, 1);
-    return std::max(1LL, std::min(wave, total_slices / kMinRun));
+// Planes per CTA of a persistent 3D kernel whose CTAs own equal contiguous runs of
+// the flattened (tile, z) space; at most one resident wave (n_sm x occ CTAs).  A run
+// of p planes costs p + halo planes, halo standing for the planes it only warms its
+// rings with, once more where runs cross from one tile into the next.  With q CTAs on
+// the fullest SM the kernel takes about q + 1 runs: the FP64 pipe is shared, but the
+// barriers and loads of one run are not hidden.  Grids that fill the wave with long runs keep p =
+// total / wave; small ones are spread over all SMs down to single planes (64^3 FP64
+// Gray-Scott 7-point: 417 us per step with runs of at least 32 planes, 17 us now;
+// 32^3 Cahn-Hilliard 179 -> 11.5 us; 129 x 32 x 208 Cahn-Hilliard 189 -> 47 us, where
+// the balance of q against p decides between runs of 3 (53 us) and 4 planes).
+inline long long planes_per_cta(long long tiles, int nz, double halo, int occ, int n_sm) {
+    const long long total = tiles * nz, wave = (long long)n_sm * std::max(occ, 1);
+    const long long p0 = (total + wave - 1) / wave;
+    long long best = p0;
+    double best_cost = 0;
+    for (long long p = p0; p <= std::min(total, 4 * p0 + 8); ++p) {
+        const long long ctas = (total + p - 1) / p, q = (ctas + n_sm - 1) / n_sm;
+        const double cost = (q + 1.0) * (p + (nz % p ? 2 : 1) * halo);
+        if (p == p0 || cost < best_cost * 0.999) {
+            best = p;
+            best_cost = cost;
+        }
+        if (q == 1) break;  // longer runs on fewer SMs only take longer
+    }
+    return best;
 }
 
 // Launch with programmatic stream serialisation (the kernel calls pdl_enter()
@@ -138,18 +160,17 @@ cudaError_t launch_zreg(const StepArgs &a, cudaStream_t s, int n_sm) {
         return o;
     }();
     const int tx = (a.nx + TX - 1) / TX, ty = (a.ny + TY - 1) / TY;
-    const long long ctas = persistent_ctas((long long)tx * ty * a.nz, occ, n_sm);
-    const long long planes = ((long long)tx * ty * a.nz + ctas - 1) / ctas;
+    const long long planes = planes_per_cta((long long)tx * ty, a.nz, 1.0, occ, n_sm);
     kern<<<(unsigned)(((long long)tx * ty * a.nz + planes - 1) / planes), NT, Sh::smem_bytes, s>>>(a, tx, ty, planes);
     return cudaGetLastError();
 }
 
 // FP64 27-point with shared pair sums: one pass per mode (Cahn-Hilliard: mode 0
 // then mode 1 through the mu buffer).
-template <int MODE>
-cudaError_t launch_planes27_mode(const Planes27Args &a, cudaStream_t s, int n_sm) {
-    typedef Planes27Shape<MODE> Sh;
-    auto kern = planes27_kernel<MODE>;
+template <int MODE, int TY>
+cudaError_t launch_planes27_tile(const Planes27Args &a, cudaStream_t s, int n_sm) {
+    typedef Planes27Shape<MODE, TY> Sh;
+    auto kern = planes27_kernel<MODE, TY>;
     static const int occ = [&] {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::smem_bytes);
         int o = 1;
@@ -158,16 +179,20 @@ cudaError_t launch_planes27_mode(const Planes27Args &a, cudaStream_t s, int n_sm
     }();
     const int tx = (a.nx + Sh::TX - 1) / Sh::TX, ty = (a.ny + Sh::TY - 1) / Sh::TY;
     const long long total = (long long)tx * ty * a.nz;
-    const long long ctas = persistent_ctas(total, occ, n_sm);
-    const long long planes = (total + ctas - 1) / ctas;
+    const long long planes = planes_per_cta((long long)tx * ty, a.nz, 1.0, occ, n_sm);
     kern<<<(unsigned)((total + planes - 1) / planes), Sh::NT, Sh::smem_bytes, s>>>(a, tx, planes, total);
     return cudaGetLastError();
 }
+template <int MODE>
+cudaError_t launch_planes27_mode(const Planes27Args &a, cudaStream_t s, int n_sm) {
+    return small_tile(a.nx, a.ny, 32, 32) ? launch_planes27_tile<MODE, 16>(a, s, n_sm)
+                                          : launch_planes27_tile<MODE, 32>(a, s, n_sm);
+}
 
-template <int ST, int MODE>
-cudaError_t launch_ring2pass_mode(const Planes27Args &a, cudaStream_t s, int n_sm) {
-    typedef Ring2PassShape<ST> Sh;
-    auto kern = ring2pass_kernel<ST, MODE>;
+template <int ST, int MODE, int TY>
+cudaError_t launch_ring2pass_tile(const Planes27Args &a, cudaStream_t s, int n_sm) {
+    typedef Ring2PassShape<ST, TY> Sh;
+    auto kern = ring2pass_kernel<ST, MODE, TY>;
     static const int occ = [&] {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::smem_bytes);
         int o = 1;
@@ -176,9 +201,30 @@ cudaError_t launch_ring2pass_mode(const Planes27Args &a, cudaStream_t s, int n_s
     }();
     const int tx = (a.nx + Sh::TX - 1) / Sh::TX, ty = (a.ny + Sh::TY - 1) / Sh::TY;
     const long long total = (long long)tx * ty * a.nz;
-    const long long ctas = persistent_ctas(total, occ, n_sm);
-    const long long planes = (total + ctas - 1) / ctas;
+    const long long planes = planes_per_cta((long long)tx * ty, a.nz, 0.7 * Sh::R, occ, n_sm);
     kern<<<(unsigned)((total + planes - 1) / planes), Sh::NT, Sh::smem_bytes, s>>>(a, tx, planes, total);
+    return cudaGetLastError();
+}
+template <int ST, int MODE>
+cudaError_t launch_ring2pass_mode(const Planes27Args &a, cudaStream_t s, int n_sm) {
+    return small_tile(a.nx, a.ny, 32, 32) ? launch_ring2pass_tile<ST, MODE, 16>(a, s, n_sm)
+                                          : launch_ring2pass_tile<ST, MODE, 32>(a, s, n_sm);
+}
+
+// 3D FP64, accessor-based plane ring.
+template <int MODEL, int ST, int TX, int TY, int NT>
+cudaError_t launch_step3d_tile(const StepArgs &a, cudaStream_t s, int n_sm) {
+    typedef Step3dShape<MODEL, ST, double, TX, TY, NT> Sh;
+    auto kern = step3d_kernel<MODEL, ST, double, TX, TY, NT>;
+    static const int occ = [&] {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::smem_bytes);
+        int o = 1;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, NT, Sh::smem_bytes);
+        return o;
+    }();
+    const int tx = (a.nx + TX - 1) / TX, ty = (a.ny + TY - 1) / TY;
+    const long long planes = planes_per_cta((long long)tx * ty, a.nz, 0.7 * Sh::RIN, occ, n_sm);
+    kern<<<(unsigned)(((long long)tx * ty * a.nz + planes - 1) / planes), NT, Sh::smem_bytes, s>>>(a, tx, ty, planes);
     return cudaGetLastError();
 }
 
@@ -355,28 +401,17 @@ cudaError_t launch_step_t(const StepArgs &a, cudaStream_t s, int n_sm, int k) {
             return o;
         }();
         const int tx = (a.nx + Sh::TX - 1) / Sh::TX, ty = (a.ny + Sh::TY - 1) / Sh::TY;
-        const long long ctas = persistent_ctas((long long)tx * ty * a.nz, occ, n_sm);
-        const long long planes = ((long long)tx * ty * a.nz + ctas - 1) / ctas;
+        const long long planes = planes_per_cta((long long)tx * ty, a.nz, Sh::R, occ, n_sm);
         kern<<<(unsigned)(((long long)tx * ty * a.nz + planes - 1) / planes), Sh::NT, Sh::smem_bytes, s>>>(
             a, tx, ty, planes);
     } else {
         if constexpr (MODEL != MC) {
             if (ST == L27 && g_step_variant == 0) return launch_zreg<MODEL, T>(a, s, n_sm);
         }
-        typedef typename Tiles<T>::template T3<StencilInfo<ST>::r> TT;
-        typedef Step3dShape<MODEL, ST, T, TT::TX, TT::TY, TT::NT> Sh;
-        auto kern = step3d_kernel<MODEL, ST, T, TT::TX, TT::TY, TT::NT>;
-        static const int occ = [&] {
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::smem_bytes);
-            int o = 1;
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, TT::NT, Sh::smem_bytes);
-            return o;
-        }();
-        const int tx = (a.nx + TT::TX - 1) / TT::TX, ty = (a.ny + TT::TY - 1) / TT::TY;
-        const long long ctas = persistent_ctas((long long)tx * ty * a.nz, occ, n_sm);
-        const long long planes = ((long long)tx * ty * a.nz + ctas - 1) / ctas;
-        kern<<<(unsigned)(((long long)tx * ty * a.nz + planes - 1) / planes), TT::NT, Sh::smem_bytes, s>>>(
-            a, tx, ty, planes);
+        typedef Tiles64<StencilInfo<ST>::r> TT;
+        if (small_tile(a.nx, a.ny, TT::TX, TT::TY))
+            return launch_step3d_tile<MODEL, ST, kSmallTX, kSmallTY, kSmallNT>(a, s, n_sm);
+        return launch_step3d_tile<MODEL, ST, TT::TX, TT::TY, TT::NT>(a, s, n_sm);
     }
     return cudaGetLastError();
 }
