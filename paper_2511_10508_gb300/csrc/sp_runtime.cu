@@ -385,7 +385,7 @@ extern "C" int sp_create(int model, int dims, const int64_t shape[3], double h, 
         return fail(SP_ECUDA, "initial condition: %s", cudaGetErrorString(e));
     }
     if (prm.scheme == SP_SCHEME_SPECTRAL) {
-        int rc = spectral_create(s->dtype, dims, s->nx, s->ny, s->nz, &s->spec);
+        int rc = spectral_create(s->dtype, dims, s->nx, s->ny, s->nz, h, &s->spec);
         if (rc == SP_OK) rc = spectral_load(s->spec, s->f[0][0], s->stream);
         if (rc == SP_OK && cudaStreamSynchronize(s->stream) != cudaSuccess) rc = SP_ECUDA;
         if (rc != SP_OK) {
@@ -616,8 +616,8 @@ extern "C" int sp_step(sp_sim *s, int64_t nsteps, void *stream) {
                 if (int rc = spectral_load(s->spec, s->f[0][0], st)) return fail(rc, "%s", spectral_last_error());
                 s->spec_dirty = false;
             }
-            if (int rc = spectral_step(s->spec, s->model, s->f[0][0], s->f[1][0], s->h, s->dt, s->p.c1, s->p.c2,
-                                       s->p.kappa, st, s->n_sm, i + 1 < nsteps))
+            if (int rc = spectral_step(s->spec, s->model, s->f[0][0], s->dt, s->p.c1, s->p.c2, s->p.kappa, st,
+                                       i + 1 < nsteps))
                 return fail(rc, "spectral step: %s", spectral_last_error());
             s->steps += 1;
         }
