@@ -48,13 +48,17 @@ static bool factor_len(int n, FftLen *L) {
     L->pow2 = is_pow2(n) && n >= 32;
     L->lgn = 0;
     while ((1 << L->lgn) < n) ++L->lgn;
-    L->ls = (L->lgn + 1) / 2;
     L->nst = 0;
-    if (L->pow2) {  // radix 16, then as few stages as possible, of even radices
-        L->lgr[L->nst++] = 4;
-        for (int rest = L->lgn - 4; rest > 0; rest -= L->lgr[L->nst - 1]) {
-            const int left = (rest + 3) / 4;
-            L->lgr[L->nst++] = (rest + left - 1) / left;
+    if (L->pow2) {
+        for (int v = 0; v < 2; ++v) {  // radix V, then as few stages as possible, of even radices
+            FftStages &S = L->reg[v];
+            const int lgv = v == 0 ? 4 : 2;
+            S.nst = 0;
+            S.lgr[S.nst++] = lgv;
+            for (int rest = L->lgn - lgv; rest > 0 && S.nst < 8; rest -= S.lgr[S.nst - 1]) {
+                const int left = (rest + lgv - 1) / lgv;
+                S.lgr[S.nst++] = (rest + left - 1) / left;
+            }
         }
         return true;
     }
@@ -92,8 +96,9 @@ int spectral_create(int dtype, int dims, int nx, int ny, int nz, double h, Spect
             delete P;
             return SP_EINVAL;
         }
-    // twiddles exp(-2 pi i t / n) of each distinct side, in long double on the host, rounded
-    // once to the working precision; squared wavenumbers of each axis in FP64, rounded once
+    // twiddles of each distinct side (see FftStages, FftLen), in long double on the host,
+    // rounded once to the working precision; squared wavenumbers of each axis in FP64,
+    // rounded once
     std::vector<long double> re, im;
     std::vector<double> k2;
     const long double two_pi = 6.283185307179586476925286766559005768L;
@@ -109,23 +114,27 @@ int spectral_create(int dtype, int dims, int nx, int ny, int nz, double h, Spect
             const double k = (double)(two_pi / ((long double)L.n * (long double)h)) * (m < (L.n + 1) / 2 ? m : m - L.n);
             k2.push_back(k * k);
         }
-        int prev = -1;
+        int same = -1;
         for (int b = 0; b < a; ++b)
-            if (sides[b] == sides[a]) prev = b;
-        if (prev >= 0) {
-            L.tw_off = ls[prev]->tw_off;
-            L.lo_off = ls[prev]->lo_off;
-            L.hi_off = ls[prev]->hi_off;
+            if (sides[b] == sides[a]) same = b;
+        if (same >= 0) {
+            L.tw_off = ls[same]->tw_off;
+            for (int v = 0; v < 2; ++v) L.reg[v].tw_off = ls[same]->reg[v].tw_off;
             continue;
         }
         L.tw_off = (int)re.size();
-        for (int t = 0; t < L.n; ++t) root(t, L.n);
-        L.lo_off = L.hi_off = 0;
-        if (!L.pow2 || f64) continue;
-        L.lo_off = (int)re.size();
-        for (int t = 0; t < (1 << L.ls); ++t) root(t, L.n);
-        L.hi_off = (int)re.size();
-        for (int u = 0; u < (L.n >> L.ls); ++u) root((long long)u << L.ls, L.n);
+        if (!L.pow2)
+            for (int t = 0; t < L.n; ++t) root(t, L.n);
+        for (int v = 0; v < (L.pow2 ? 2 : 0); ++v) {
+            FftStages &S = L.reg[v];
+            S.tw_off = (int)re.size();
+            if (v == 1 && L.n > 1024) continue;  // never transformed with 4 points per thread
+            for (int i = 1, lgp = S.lgr[0]; i < S.nst; lgp += S.lgr[i++])
+                for (int l = 1; l <= S.lgr[i]; ++l)  // w^(R >> l) exp(-2 pi i m / 2^l)
+                    for (int m = 0; m < std::max(1, 1 << l >> 2); ++m)
+                        for (int k = 0; k < (1 << lgp); ++k)
+                            root(((long long)k << (S.lgr[i] - l)) + ((long long)m << (lgp + S.lgr[i] - l)), 1 << (lgp + S.lgr[i]));
+        }
     }
     const size_t rb = f64 ? sizeof(double) : sizeof(float), cb = 2 * rb;
     std::vector<unsigned char> host(re.size() * cb), host2(k2.size() * rb);

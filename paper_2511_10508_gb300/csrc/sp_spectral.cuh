@@ -10,17 +10,22 @@ namespace sp {
 constexpr int kFftMaxN = 8192;
 constexpr int kFftMaxStages = 16;
 
+// The stages of a register transform with V points per thread: radices 2^lgr[s], the
+// first one V.  tw_off: complex offset of the stages' twiddles in the plan's table, for
+// every later stage (radix R after radices of product p) R/2 rows of p entries:
+// w^(R >> l) exp(-2 pi i m / 2^l), w = exp(-2 pi i k / (R p)), k < p, for the levels l = 1 ..
+// log2 R and m < max(1, 2^(l-2)).
+struct FftStages {
+    int nst, lgr[8], tw_off;
+};
+
 // One transform length.  A power of two from 32 on is transformed in registers
-// (fft_regs): kFftV values per thread, radices 2^lgr[s], the first one 16.  Other
-// lengths take mixed-radix stages in shared memory (fft_lines): radices rad[s].
+// (fft_regs), other lengths by mixed-radix stages in shared memory (fft_lines).
 struct FftLen {
-    int n, pow2;           // pow2: the register transform
-    int lgn, nst;
-    int lgr[4];
-    int rad[kFftMaxStages];
-    int tw_off;            // complex offset of exp(-2 pi i t / n), t < n, in the plan's table
-    // the two-level table w(t) = lo[t mod 2^ls] hi[t >> ls] (FP32, powers of two)
-    int ls, lo_off, hi_off;
+    int n, pow2, lgn;      // pow2: the register transform
+    FftStages reg[2];      // 16 and 4 points per thread
+    int nst, rad[kFftMaxStages];
+    int tw_off;            // mixed: complex offset of exp(-2 pi i t / n), t < n, in the plan's table
     int k2_off;            // real offset of (2 pi freq(m) / (n h))^2, m < n, in the plan's wavenumber table
 };
 
@@ -77,21 +82,24 @@ template <typename C> __device__ __forceinline__ void butterfly(C &a, C &b, C t)
 
 // ============================================ powers of two, in registers ==
 //
-// A line of n points is held by T = n / 16 threads, 16 values each: thread t has
-// points t + j T, before and after a transform, so the loads and stores of lines are
+// A line of n points is held by T = n / V threads, V values each: thread t has points
+// t + j T, before and after a transform, so the loads and stores of lines are
 // coalesced, the Fourier update and the cube run on registers, and a forward
 // transform is followed by an inverse one without a pass through memory.  The stages
-// are those of a Stockham transform of radices 16, .. (first 16, then 16, 8, 4 or 2);
-// between two stages the values change threads through one shared-memory buffer.
+// are those of a Stockham transform, the first of radix V; between two stages the
+// values change threads through one shared-memory buffer.
 // Radix-R butterflies are decimation in time with the stage's twiddles merged into
 // every level as multiply-adds (after Goedecker, SIAM J. Sci. Comput. 18, 1997: six
 // per two points and level): 192 operations and 8 distinct twiddles for 16 points
 // where separate twiddles take 228 and 15; the first stage, whose twiddles are
-// constants, takes 148.
+// constants, takes 148.  The twiddles come from tables in the order in which the
+// threads need them, through L1 (computing them from a two-level table in shared
+// memory took a quarter of the FP32 instructions).
 // The inverse is the forward transform of values with real and imaginary part
 // exchanged.  Every transform here therefore runs the same code.
-
-constexpr int kFftV = 16;
+// V = 16 for throughput.  V = 4 where V = 16 would leave fewer than four warps per SM
+// (a single FP64 warp gets a quarter of the SM's FP64 rate, and short code matters when
+// every instruction is fetched for one warp).
 
 __host__ __device__ constexpr int bit_reverse(int m, int lg) {
     int r = 0;
@@ -107,13 +115,13 @@ template <typename C> __device__ __forceinline__ C root16(int m) {
     return m == 0 ? C{R(1), R(0)} : m == 1 ? C{R(c1), R(-s1)} : m == 2 ? C{R(h), R(-h)} : C{R(s1), R(-c1)};
 }
 
-// R-point butterflies of the values u[q + j Q] (Q = kFftV / R), q < Q; output m of
-// butterfly q is left at u[q + bit_reverse(m) Q].  TW: with twiddles, T(q, s, m) the
-// factor w^(R >> s) exp(-2 pi i m / 2^s) of level s (m < max(1, 2^(s-2)); the other
-// half of a level is those times -i).
-template <int LGR, bool TW, typename C, typename TwF>
-__device__ __forceinline__ void dit(C (&u)[kFftV], const TwF &tw) {
-    constexpr int R = 1 << LGR, Q = kFftV / R;
+// R-point butterflies of the values u[q + j Q] (Q = V / R), q < Q; output m of
+// butterfly q is left at u[q + bit_reverse(m) Q].  TW: with twiddles, tw(q, row) the
+// factor of level s and m in row (s < 3 ? s - 1 : 2^(s-2) + m) of the stage's table (m <
+// max(1, 2^(s-2)); the other half of a level is those times -i).
+template <int LGR, bool TW, int V, typename C, typename TwF>
+__device__ __forceinline__ void dit(C (&u)[V], const TwF &tw) {
+    constexpr int R = 1 << LGR, Q = V / R;
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
 #pragma unroll
@@ -122,7 +130,7 @@ __device__ __forceinline__ void dit(C (&u)[kFftV], const TwF &tw) {
 #pragma unroll
             for (int mt = 0; mt < nt; ++mt) {
                 C t{1, 0};
-                if constexpr (TW) t = tw(q, s, mt);
+                if constexpr (TW) t = tw(q, s < 3 ? s - 1 : nt + mt);
                 else t = root16<C>(mt << (4 - s > 0 ? 4 - s : 0));
 #pragma unroll
                 for (int rot = 0; rot < (nm < 2 ? 1 : 2); ++rot) {
@@ -145,22 +153,12 @@ __device__ __forceinline__ void dit(C (&u)[kFftV], const TwF &tw) {
     }
 }
 
-// Shared-memory slot of point i of a line: from 256 points on one empty slot after
-// every 16 (the first stage's stores, 16 points apart, and all loads are then free of
-// bank conflicts).  sh is 4 or 31; slot(a + b) = slot(a) + slot(b) for b a multiple
-// of 16 or sh = 31.
+// Shared-memory slot of point i of a line: for 256 points and more (V = 16) one empty
+// slot after every 16 (the first stage's stores, 16 points apart, and all loads are then
+// free of bank conflicts).  sh is 4 or 31; slot(a + b) = slot(a) + slot(b) for b a
+// multiple of 16 or sh = 31.
 __device__ __forceinline__ int slot_of(int i, int sh) { return i + (i >> sh); }
-__host__ __device__ __forceinline__ int pad_shift(int n) { return n >= 256 ? 4 : 31; }
-
-template <typename C> struct Twiddles {
-    const C *tab;          // full table (FP64: read through L1)
-    const C *lo, *hi;      // two-level table in shared memory (FP32)
-    int ls;
-    __device__ __forceinline__ C at(int i) const {
-        if constexpr (sizeof(C) == 16) return __ldg(tab + i);
-        else return cmul(lo[slot_of(i & ((1 << ls) - 1), 4)], hi[i >> ls]);
-    }
-};
+template <int V> __host__ __device__ __forceinline__ int pad_shift(int n) { return V == 16 && n >= 256 ? 4 : 31; }
 
 // the position of this thread in its line and the synchronisation of a line's threads
 struct LineThread {
@@ -172,30 +170,19 @@ struct LineThread {
     }
 };
 
-// twiddled stage of radix 2^LGR after radices of product 2^lgp
-template <int LGR, typename C>
-__device__ __forceinline__ void twiddled_stage(C (&u)[kFftV], const Twiddles<C> &W, int t, int lgT, int lgn, int lgp) {
-    constexpr int R = 1 << LGR;
-    const int lgstep = lgn - lgp - LGR, n = 1 << lgn;
-    // the level factors of butterfly q: w = exp(-2 pi i k / (R p)), k = (t + q T) mod p
-    auto tw = [&](int q, int s, int mt) -> C {
+// twiddled stage of radix 2^LGR after radices of product 2^lgp; tw: the stage's table
+template <int LGR, int V, typename C>
+__device__ __forceinline__ void twiddled_stage(C (&u)[V], const C *tw, int t, int lgT, int lgp) {
+    dit<LGR, true>(u, [&](int q, int row) -> C {
         const int k = (t + (q << lgT)) & ((1 << lgp) - 1);
-        const int e = k << lgstep;
-        if constexpr (sizeof(C) == 16) {
-            return W.at(e * (R >> s) + ((mt << lgn) >> s));
-        } else {
-            const C w = W.at(e * (R >> s));
-            return mt == 0 ? w : cmul(w, root16<C>(mt << (4 - s > 0 ? 4 - s : 0)));
-        }
-    };
-    (void)n;
-    dit<LGR, true>(u, tw);
+        return __ldg(tw + k + (row << lgp));
+    });
 }
 
 // outputs of a radix-2^LGR stage to their sorted places in buf
-template <int LGR, typename C>
-__device__ __forceinline__ void scatter(const C (&u)[kFftV], C *buf, int t, int lgT, int lgp, int sh) {
-    constexpr int R = 1 << LGR, Q = kFftV / R;
+template <int LGR, int V, typename C>
+__device__ __forceinline__ void scatter(const C (&u)[V], C *buf, int t, int lgT, int lgp, int sh) {
+    constexpr int R = 1 << LGR, Q = V / R;
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
         const int b = t + (q << lgT), k = b & ((1 << lgp) - 1);
@@ -206,45 +193,50 @@ __device__ __forceinline__ void scatter(const C (&u)[kFftV], C *buf, int t, int 
 }
 
 // natural order of the last stage's outputs (registers renamed)
-template <int LGR, typename C> __device__ __forceinline__ void unscramble(C (&u)[kFftV]) {
-    constexpr int R = 1 << LGR, Q = kFftV / R;
-    C v[kFftV];
+template <int LGR, int V, typename C> __device__ __forceinline__ void unscramble(C (&u)[V]) {
+    constexpr int R = 1 << LGR, Q = V / R;
+    C v[V];
 #pragma unroll
     for (int q = 0; q < Q; ++q)
 #pragma unroll
         for (int m = 0; m < R; ++m) v[q + m * Q] = u[q + bit_reverse(m, LGR) * Q];
 #pragma unroll
-    for (int j = 0; j < kFftV; ++j) u[j] = v[j];
+    for (int j = 0; j < V; ++j) u[j] = v[j];
 }
 
 // Forward transform (unnormalised) of the line whose points t + j T this thread holds.
 // buf: the line's buffer, free for use once the line's threads have synchronised.
-template <typename C>
-__device__ __forceinline__ void fft_regs(C (&u)[kFftV], C *buf, const FftLen &L, const Twiddles<C> &W,
-                                         const LineThread &lt) {
-    const int t = lt.t, lgT = lt.lgT, sh = pad_shift(L.n);
+template <int V, typename C>
+__device__ __forceinline__ void fft_regs(C (&u)[V], C *buf, const FftLen &L, const C *tw_all, const LineThread &lt) {
+    constexpr int LGV = V == 16 ? 4 : 2;
+    const FftStages &S = L.reg[V == 16 ? 0 : 1];
+    const int t = lt.t, lgT = lt.lgT, sh = pad_shift<V>(L.n);
     const int rd = slot_of(t, sh), rinc = slot_of(1 << lgT, sh);
-    dit<4, false>(u, [](int, int, int) { return C{1, 0}; });
+    const C *tw = tw_all + S.tw_off;
+    dit<LGV, false>(u, [](int, int) { return C{1, 0}; });
     lt.sync();
 #pragma unroll
-    for (int m = 0; m < kFftV; ++m) buf[slot_of(t << 4, sh) + m] = u[bit_reverse(m, 4)];
-    int lgp = 4;
+    for (int m = 0; m < V; ++m) buf[slot_of(t << LGV, sh) + m] = u[bit_reverse(m, LGV)];
+    int lgp = LGV;
 #pragma unroll 1
-    for (int s = 1; s < L.nst; ++s) {
+    for (int s = 1; s < S.nst; ++s) {
         lt.sync();
 #pragma unroll
-        for (int j = 0; j < kFftV; ++j) u[j] = buf[rd + j * rinc];
-        const bool last = s + 1 == L.nst;
-        switch (L.lgr[s]) {
-#define SP_STAGE(LG)                                          \
-    case LG:                                                  \
-        twiddled_stage<LG>(u, W, t, lgT, L.lgn, lgp);         \
-        if (!last) {                                          \
-            lt.sync();                                        \
-            scatter<LG>(u, buf, t, lgT, lgp, sh);             \
-        } else {                                              \
-            unscramble<LG>(u);                                \
-        }                                                     \
+        for (int j = 0; j < V; ++j) u[j] = buf[rd + j * rinc];
+        const bool last = s + 1 == S.nst;
+        const int lgr = S.lgr[s];
+        switch (lgr) {
+#define SP_STAGE(LG)                                    \
+    case LG:                                            \
+        if constexpr (LG <= LGV) {                      \
+            twiddled_stage<LG>(u, tw, t, lgT, lgp);     \
+            if (!last) {                                \
+                lt.sync();                              \
+                scatter<LG>(u, buf, t, lgT, lgp, sh);   \
+            } else {                                    \
+                unscramble<LG>(u);                      \
+            }                                           \
+        }                                               \
         break;
             SP_STAGE(4)
             SP_STAGE(3)
@@ -252,7 +244,8 @@ __device__ __forceinline__ void fft_regs(C (&u)[kFftV], C *buf, const FftLen &L,
             SP_STAGE(1)
 #undef SP_STAGE
         }
-        lgp += L.lgr[s];
+        tw += (size_t)1 << (lgp + lgr - 1);
+        lgp += lgr;
     }
 }
 
@@ -283,27 +276,9 @@ struct PassGeom {
     int ny, nz, nxh, nrows;
 };
 
-template <typename R> __device__ __forceinline__ Twiddles<typename Cplx<R>::type> load_tw(
-    const FftLen &L, const typename Cplx<R>::type *tw, typename Cplx<R>::type *dst) {
-    typedef typename Cplx<R>::type C;
-    Twiddles<C> W{tw + L.tw_off, nullptr, nullptr, L.ls};
-    if constexpr (sizeof(R) == 4) {
-        const int nlo = 1 << L.ls, nhi = L.n >> L.ls;
-        C *h = dst + slot_of(nlo, 4) + 1;
-        for (int i = threadIdx.x; i < nlo + nhi; i += blockDim.x) {
-            if (i < nlo) dst[slot_of(i, 4)] = tw[L.lo_off + i];
-            else h[i - nlo] = tw[L.hi_off + i - nlo];
-        }
-        W.lo = dst;
-        W.hi = h;
-        __syncthreads();
-    }
-    return W;
-}
-
-// this thread's line within the CTA and its place in it
-__device__ __forceinline__ int line_thread(const FftLen &L, const PassGeom &g, LineThread &lt) {
-    lt.lgT = L.lgn - 4;
+// this thread's line within the CTA and its place in it (V points per thread)
+template <int V> __device__ __forceinline__ int line_thread(const FftLen &L, const PassGeom &g, LineThread &lt) {
+    lt.lgT = L.lgn - (V == 16 ? 4 : 2);
     const int I = 1 << g.lgI, lo = threadIdx.x & (I - 1), r = threadIdx.x >> g.lgI;
     lt.t = r & ((1 << lt.lgT) - 1);
     lt.warp_local = lt.lgT + g.lgI <= 5;
@@ -316,18 +291,17 @@ template <typename R> struct FftBounds {
     static constexpr int NT = sizeof(R) == 8 ? 256 : 512, MINB = 2;
 };
 
-template <typename R, int MODE>
+template <typename R, int MODE, int V>
 __global__ void __launch_bounds__(FftBounds<R>::NT, FftBounds<R>::MINB)
     rows_regs_kernel(R *f, typename Cplx<R>::type *Z, PassGeom g, R coef, FftLen L, const typename Cplx<R>::type *tw) {
     typedef typename Cplx<R>::type C;
-    constexpr int V = kFftV, H = V / 2;
+    constexpr int H = V / 2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C *bufs = reinterpret_cast<C *>(smem_raw);
-    const Twiddles<C> W = load_tw<R>(L, tw, bufs + g.G * g.LS);
+    pdl_enter();
     LineThread lt;
-    const int l = line_thread(L, g, lt);
-    C *buf = bufs + l * g.LS;
-    const int n = L.n, sh = pad_shift(n), T = 1 << lt.lgT, t = lt.t;
+    const int l = line_thread<V>(L, g, lt);
+    C *buf = reinterpret_cast<C *>(smem_raw) + l * g.LS;
+    const int n = L.n, sh = pad_shift<V>(n), T = 1 << lt.lgT, t = lt.t;
     const int pair = blockIdx.x * g.G + l;
     const bool on = pair < g.nlines;
     const int ra = 2 * pair;
@@ -335,7 +309,7 @@ __global__ void __launch_bounds__(FftBounds<R>::NT, FftBounds<R>::MINB)
     const size_t ro = (size_t)ra * n;
     C u[V];
     auto read_pair = [&](int k, C &A, C &B) {  // modes k of the two rows
-        const C *p = Z + (size_t)k * g.nrows + ra;
+        const C *p = Z + ((uint64_t)(uint32_t)k * (uint32_t)g.nrows + (uint32_t)ra);
         if (sizeof(R) == 4 && vec) {
             const float4 q = *reinterpret_cast<const float4 *>(p);
             A = C{(R)q.x, (R)q.y};
@@ -380,7 +354,7 @@ __global__ void __launch_bounds__(FftBounds<R>::NT, FftBounds<R>::MINB)
     }
 #pragma unroll 1
     for (int pass = 0; pass < (MODE == kRowInverseNext ? 2 : 1); ++pass) {
-        fft_regs(u, buf, L, W, lt);
+        fft_regs(u, buf, L, tw, lt);
         if ((MODE == kRowInverse || MODE == kRowInverseNext) && pass == 0) {
             if (on) {
 #pragma unroll
@@ -404,7 +378,7 @@ __global__ void __launch_bounds__(FftBounds<R>::NT, FftBounds<R>::MINB)
         if (on) {
             auto put = [&](int k, C zk, C zc) {
                 const C A{zk.x + zc.x, zk.y - zc.y}, B{zk.y + zc.y, zc.x - zk.x};
-                C *p = Z + (size_t)k * g.nrows + ra;
+                C *p = Z + ((uint64_t)(uint32_t)k * (uint32_t)g.nrows + (uint32_t)ra);
                 if (sizeof(R) == 4 && vec) {
                     *reinterpret_cast<float4 *>(p) = make_float4((float)A.x, (float)A.y, (float)B.x, (float)B.y);
                 } else {
@@ -422,20 +396,19 @@ __global__ void __launch_bounds__(FftBounds<R>::NT, FftBounds<R>::MINB)
     }
 }
 
-template <typename R, int MODE, int MODEL>
+template <typename R, int MODE, int MODEL, int V>
 __global__ void __launch_bounds__(FftBounds<R>::NT, FftBounds<R>::MINB)
     lines_regs_kernel(typename Cplx<R>::type *Z, typename Cplx<R>::type *uh, PassGeom g, FftLen L,
                       const typename Cplx<R>::type *tw, const R *kx2, const R *ky2, const R *kz2, SpecCoef<R> c) {
     typedef typename Cplx<R>::type C;
-    constexpr int V = kFftV;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C *bufs = reinterpret_cast<C *>(smem_raw);
-    const Twiddles<C> W = load_tw<R>(L, tw, bufs + g.G * g.LS);
+    pdl_enter();
     LineThread lt;
-    const int l = line_thread(L, g, lt);
-    C *buf = bufs + l * g.LS;
+    const int l = line_thread<V>(L, g, lt);
+    C *buf = reinterpret_cast<C *>(smem_raw) + l * g.LS;
     const int T = 1 << lt.lgT, t = lt.t;
-    size_t base, es;   // first point of the line, elements between its points
+    size_t base;       // first point of the line
+    uint32_t es;       // elements between its points (a line spans less than 2^31)
     R kb = 0;          // the squared wavenumber of the other axes
     const R *kl;       // and along the line
     bool on;
@@ -458,24 +431,24 @@ __global__ void __launch_bounds__(FftBounds<R>::NT, FftBounds<R>::MINB)
     if (on) {
 #pragma unroll
         for (int j = 0; j < V; ++j) {
-            const C v = Z[base + (size_t)(t + j * T) * es];
+            const C v = Z[base + (uint32_t)(t + j * T) * es];
             u[j] = MODE == kLineInverse ? swapped(v) : v;
         }
     }
 #pragma unroll 1
     for (int pass = 0; pass < (MODE == kLineUpdate ? 2 : 1); ++pass) {
-        fft_regs(u, buf, L, W, lt);
+        fft_regs(u, buf, L, tw, lt);
         if (MODE == kLineUpdate && pass == 0 && on) {
 #pragma unroll
             for (int j = 0; j < V; ++j) {
                 const int i = t + j * T;
-                u[j] = swapped(update_mode<R, MODEL>(uh + base + (size_t)i * es, u[j], kb + kl[i], c));
+                u[j] = swapped(update_mode<R, MODEL>(uh + base + (uint32_t)i * es, u[j], kb + kl[i], c));
             }
         }
     }
     if (on) {
 #pragma unroll
-        for (int j = 0; j < V; ++j) Z[base + (size_t)(t + j * T) * es] = MODE == kLineForward ? u[j] : swapped(u[j]);
+        for (int j = 0; j < V; ++j) Z[base + (uint32_t)(t + j * T) * es] = MODE == kLineForward ? u[j] : swapped(u[j]);
     }
 }
 
@@ -620,6 +593,7 @@ __global__ void __launch_bounds__(512) rows_mixed_kernel(R *f, typename Cplx<R>:
     typedef typename Cplx<R>::type C;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *buf = reinterpret_cast<C *>(smem_raw), *alt = buf + g.G * L.n;
+    pdl_enter();
     const int n = L.n, half = n / 2, pair0 = blockIdx.x * g.G, nl = min(g.G, g.nlines - pair0);
     if constexpr (MODE == kRowInverse || MODE == kRowInverseNext) {
         // both halves of the Hermitian extension from one read (parts exchanged)
@@ -669,6 +643,7 @@ __global__ void __launch_bounds__(512)
     typedef typename Cplx<R>::type C;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *buf = reinterpret_cast<C *>(smem_raw), *alt = buf + g.G * L.n;
+    pdl_enter();
     const int n = L.n;
     int nl, first, kx = 0;  // lines of this CTA; first line (contiguous) or first y (strided)
     size_t base;
@@ -727,9 +702,10 @@ inline int lines_per_cta(int most, int least, long long lines, int n_sm) {
     return std::max(G, least);
 }
 
-// geometry, threads and shared memory of a pass; lines that a CTA interleaves: 2^lgI
+// geometry, threads, points per thread (V; 0: mixed radices) and shared memory of a
+// pass; a CTA interleaves up to 2^lgI_max lines
 template <typename R>
-void pass_shape(const SpectralPlan *P, const FftLen &L, long long lines, int lgI_max, PassGeom &g, int &threads,
+void pass_shape(const SpectralPlan *P, const FftLen &L, long long lines, int lgI_max, PassGeom &g, int &threads, int &V,
                 size_t &smem) {
     constexpr size_t cb = 2 * sizeof(R);
     g.ny = P->ny;
@@ -737,23 +713,28 @@ void pass_shape(const SpectralPlan *P, const FftLen &L, long long lines, int lgI
     g.nxh = P->nxh;
     g.nrows = P->ny * P->nz;
     if (L.pow2) {
-        const int T = L.n / kFftV, most = std::max(1, (L.n >= 4096 ? FftBounds<R>::NT : 256) / T);
+        V = L.n <= 1024 && lines * (L.n / 16) < 4LL * 32 * P->n_sm ? 4 : 16;
+        const int T = L.n / V, most = std::max(1, (L.n >= 4096 ? FftBounds<R>::NT : 256) / T);
         g.G = lines_per_cta(most, std::max(1, 32 / T), lines, P->n_sm);
         g.lgI = 0;
         while (g.lgI < lgI_max && (2 << g.lgI) <= g.G) ++g.lgI;
         // lines of adjacent threads start in different banks
         const int phase = sizeof(R) == 8 ? 8 : 16, want = g.lgI ? std::max(1, phase >> g.lgI) : 0;
-        g.LS = L.n + (L.n >> pad_shift(L.n));
+        g.LS = L.n + (L.n >> (V == 16 ? pad_shift<16>(L.n) : pad_shift<4>(L.n)));
         while (g.lgI && g.LS % phase != want % phase) ++g.LS;
         threads = g.G * T;
-        smem = cb * ((size_t)g.G * g.LS + (sizeof(R) == 4 ? (1 << L.ls) + (1 << L.ls) / 16 + 1 + (L.n >> L.ls) : 0));
+        smem = cb * (size_t)g.G * g.LS;
     } else {
+        V = 0;
         const int T = (L.n + kMixV - 1) / kMixV;
         int most = std::max(1, 256 / T);
         while (most > 1 && 2 * cb * most * L.n > 48 * 1024) --most;
         g.G = lines_per_cta(most, 1, lines, P->n_sm);
         g.lgI = g.LS = 0;
-        threads = std::max(32, (g.G * T + 31) / 32 * 32);
+        // few lines: fewer points per thread, down to 2, while an SM has under 8 warps
+        int t = T;
+        while (g.G * t * 2 <= 256 && 2 * t * 2 <= L.n && lines * t < 8LL * 32 * P->n_sm) t *= 2;
+        threads = std::max(32, (g.G * t + 31) / 32 * 32);
         smem = 2 * cb * (size_t)g.G * L.n;
     }
 }
@@ -768,16 +749,16 @@ static cudaError_t rows_mode(const SpectralPlan *P, R *f, typename Cplx<R>::type
     typedef typename Cplx<R>::type C;
     PassGeom g{};
     int threads;
+    int V;
     size_t smem;
     g.nlines = (P->ny * P->nz + 1) / 2;
     // adjacent threads take two row pairs: a full 32-byte sector (FP32) of every mode
-    pass_shape<R>(P, P->lx, g.nlines, sizeof(R) == 4 ? 1 : 0, g, threads, smem);
+    pass_shape<R>(P, P->lx, g.nlines, sizeof(R) == 4 ? 1 : 0, g, threads, V, smem);
     const unsigned blocks = (unsigned)((g.nlines + g.G - 1) / g.G);
-    auto kern = P->lx.pow2 ? rows_regs_kernel<R, MODE> : rows_mixed_kernel<R, MODE>;
+    auto kern = V == 16 ? rows_regs_kernel<R, MODE, 16> : V == 4 ? rows_regs_kernel<R, MODE, 4> : rows_mixed_kernel<R, MODE>;
     const cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
-    kern<<<blocks, threads, smem, s>>>(f, Z, g, coef, P->lx, static_cast<const C *>(P->tw));
-    return cudaGetLastError();
+    return launch_pdl(kern, dim3(blocks), dim3(threads), smem, s, f, Z, g, coef, P->lx, static_cast<const C *>(P->tw));
 }
 
 template <typename R>
@@ -797,22 +778,24 @@ static cudaError_t lines_mode(const SpectralPlan *P, int axis, const SpecCoef<R>
     const FftLen &L = axis == 1 ? P->ly : P->lz;
     PassGeom g{};
     int threads;
+    int V;
     size_t smem;
     const long long lines = (long long)P->nxh * (axis == 1 ? P->nz : P->ny);
     g.nlines = (int)lines;
-    pass_shape<R>(P, L, lines, axis == 1 ? 0 : 4, g, threads, smem);
+    pass_shape<R>(P, L, lines, axis == 1 ? 0 : 4, g, threads, V, smem);
     unsigned blocks = (unsigned)((lines + g.G - 1) / g.G);
     if (axis == 2) {
         g.per_kx = (P->ny + g.G - 1) / g.G;
         blocks = (unsigned)(P->nxh * g.per_kx);
     }
-    auto kern = L.pow2 ? lines_regs_kernel<R, MODE, MODEL> : lines_mixed_kernel<R, MODE, MODEL>;
+    auto kern = V == 16 ? lines_regs_kernel<R, MODE, MODEL, 16>
+                : V == 4 ? lines_regs_kernel<R, MODE, MODEL, 4>
+                         : lines_mixed_kernel<R, MODE, MODEL>;
     const cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     const R *k2 = static_cast<const R *>(P->k2);
-    kern<<<blocks, threads, smem, s>>>(Z, static_cast<C *>(P->uh), g, L, static_cast<const C *>(P->tw),
-                                       k2 + P->lx.k2_off, k2 + P->ly.k2_off, k2 + P->lz.k2_off, c);
-    return cudaGetLastError();
+    return launch_pdl(kern, dim3(blocks), dim3(threads), smem, s, Z, static_cast<C *>(P->uh), g, L,
+                      static_cast<const C *>(P->tw), k2 + P->lx.k2_off, k2 + P->ly.k2_off, k2 + P->lz.k2_off, c);
 }
 
 template <typename R>
