@@ -7,9 +7,10 @@
 // tile's grid descriptor (model, stencil, sizes, buffers, coefficients) and
 // runs the same tile code as the single-grid kernels (2D: 128 x 32 tiles, 3D:
 // 32 x 16 x 8 boxes), so a grid's result does not depend on what else is
-// resident.  A scheduling quantum is Q time steps = Q launches per kind,
-// captured once into a CUDA graph and replayed while the set of resident grids
-// is unchanged; grids that finish inside a quantum skip the remaining steps.
+// resident.  Grids of kOwnLaunch points and more are stepped by the single-grid kernels
+// on streams beside the batched launches.  A scheduling quantum is Q time steps = Q
+// launches per kind, captured once into a CUDA graph (the kinds as parallel branches)
+// and replayed while the set of resident grids is unchanged; grids that finish inside a quantum skip the remaining steps.
 //
 // Host side: a scheduler thread admits pending requests by priority, in
 // arrival order within a priority (later requests may pass one that does not
@@ -50,20 +51,26 @@ struct TileDesc {
 
 constexpr int kB2X = 128, kB2Y = 32, kB3X = 32, kB3Y = 16, kB3Z = 8, kBatchNT = 256;
 
-template <typename T> constexpr size_t batch2d_smem() {
-    size_t m = 0;
-#define SP_M(MO, ST) m = std::max(m, Step2dTileShape<MO, ST, T, kB2X, kB2Y>::smem_bytes);
-    SP_M(AC, L5) SP_M(AC, L9BOX) SP_M(AC, L9X4) SP_M(CH, L5) SP_M(CH, L9BOX) SP_M(CH, L9X4)
-    SP_M(GS, L5) SP_M(GS, L9BOX) SP_M(GS, L9X4) SP_M(MC, L5) SP_M(MC, L9BOX) SP_M(MC, L9X4)
+// Shared memory of one tile / box of a model and stencil.  A launch takes the largest of
+// the grids resident in its kind, not of every instantiation: the 13-point Cahn-Hilliard
+// box needs 192 KB in FP64 and would leave one CTA per SM to every other model.
+template <typename T> size_t tile_smem(int model, int stencil) {
+    switch (model * 8 + stencil) {
+#define SP_M(MO, ST) case MO * 8 + ST: return Step2dTileShape<MO, ST, T, kB2X, kB2Y>::smem_bytes;
+#define SP_B(MO, ST) case MO * 8 + ST: return Step3dBoxShape<MO, ST, T, kB3X, kB3Y, kB3Z>::smem_bytes;
+        SP_M(AC, L5) SP_M(AC, L9BOX) SP_M(AC, L9X4) SP_M(CH, L5) SP_M(CH, L9BOX) SP_M(CH, L9X4)
+        SP_M(GS, L5) SP_M(GS, L9BOX) SP_M(GS, L9X4) SP_M(MC, L5) SP_M(MC, L9BOX) SP_M(MC, L9X4)
+        SP_B(AC, L7) SP_B(AC, L27) SP_B(AC, L13X4) SP_B(CH, L7) SP_B(CH, L27) SP_B(CH, L13X4)
+        SP_B(GS, L7) SP_B(GS, L27) SP_B(GS, L13X4) SP_B(MC, L7) SP_B(MC, L27) SP_B(MC, L13X4)
 #undef SP_M
-    return m;
+#undef SP_B
+    }
+    return 0;
 }
-template <typename T> constexpr size_t batch3d_smem() {
+template <typename T> size_t largest_smem(int dims) {
     size_t m = 0;
-#define SP_M(MO, ST) m = std::max(m, Step3dBoxShape<MO, ST, T, kB3X, kB3Y, kB3Z>::smem_bytes);
-    SP_M(AC, L7) SP_M(AC, L27) SP_M(AC, L13X4) SP_M(CH, L7) SP_M(CH, L27) SP_M(CH, L13X4)
-    SP_M(GS, L7) SP_M(GS, L27) SP_M(GS, L13X4) SP_M(MC, L7) SP_M(MC, L27) SP_M(MC, L13X4)
-#undef SP_M
+    for (int mo : {AC, CH, GS, MC})
+        for (int st = dims == 2 ? L5 : L7; st <= (dims == 2 ? L9X4 : L13X4); ++st) m = std::max(m, tile_smem<T>(mo, st));
     return m;
 }
 
@@ -117,29 +124,37 @@ static int kind_of(int dims, int dtype) { return (dims == 3 ? 2 : 0) + (dtype ==
 
 static cudaError_t set_batch_attributes() {
     cudaError_t e = cudaFuncSetAttribute(batch2d_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)batch2d_smem<double>());
+                                         (int)largest_smem<double>(2));
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(batch2d_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)batch2d_smem<float>());
+                                 (int)largest_smem<float>(2));
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(batch3d_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)batch3d_smem<double>());
+                                 (int)largest_smem<double>(3));
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(batch3d_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)batch3d_smem<float>());
+                                 (int)largest_smem<float>(3));
     return e;
 }
 
-static cudaError_t launch_batch(int kind, const GridDesc *grids, const TileDesc *tiles, int ntiles, int j,
+static cudaError_t launch_batch(int kind, const GridDesc *grids, const TileDesc *tiles, int ntiles, size_t smem, int j,
                                 cudaStream_t s) {
     switch (kind) {
-    case 0: batch2d_kernel<double><<<ntiles, kBatchNT, batch2d_smem<double>(), s>>>(grids, tiles, j); break;
-    case 1: batch2d_kernel<float><<<ntiles, kBatchNT, batch2d_smem<float>(), s>>>(grids, tiles, j); break;
-    case 2: batch3d_kernel<double><<<ntiles, kBatchNT, batch3d_smem<double>(), s>>>(grids, tiles, j); break;
-    default: batch3d_kernel<float><<<ntiles, kBatchNT, batch3d_smem<float>(), s>>>(grids, tiles, j); break;
+    case 0: batch2d_kernel<double><<<ntiles, kBatchNT, smem, s>>>(grids, tiles, j); break;
+    case 1: batch2d_kernel<float><<<ntiles, kBatchNT, smem, s>>>(grids, tiles, j); break;
+    case 2: batch3d_kernel<double><<<ntiles, kBatchNT, smem, s>>>(grids, tiles, j); break;
+    default: batch3d_kernel<float><<<ntiles, kBatchNT, smem, s>>>(grids, tiles, j); break;
     }
     return cudaGetLastError();
 }
+
+// A grid of a million points and more fills the GPU by itself: it is stepped by the
+// single-grid kernels (plane streaming, warp strips, fused steps; bit-identical to the
+// tiles), launched on a stream of its own beside the batched ones.  236^3 FP64 Gray-Scott:
+// 850 us per step in boxes, 610 alone.  Smaller grids share the batched launches, whose
+// cost they split.
+constexpr uint64_t kOwnLaunch = 1u << 20;
+constexpr int kOwnStreams = 4, kKinds = 4;
 
 }  // namespace sp
 
@@ -192,7 +207,10 @@ struct sp_server {
     int grids_cap = 0;
     TileDesc *d_tiles = nullptr;
     size_t tiles_cap = 0;
-    int kind_off[4] = {0, 0, 0, 0}, kind_n[4] = {0, 0, 0, 0};
+    int kind_off[kKinds] = {0, 0, 0, 0}, kind_n[kKinds] = {0, 0, 0, 0};
+    size_t kind_smem[kKinds] = {0, 0, 0, 0};
+    cudaStream_t side[kOwnStreams] = {nullptr, nullptr, nullptr, nullptr};  // own-launch grids; branches of a capture
+    cudaEvent_t fork = nullptr, join[kOwnStreams] = {nullptr, nullptr, nullptr, nullptr};
     double *d_partials = nullptr, *h_scalar = nullptr;
     int nred = 0;
     cudaGraphExec_t graph = nullptr;
@@ -236,10 +254,14 @@ static cudaError_t rebuild_tables(sp_server *S) {
         if (e == cudaSuccess) e = cudaMallocHost(&S->h_grids, sizeof(GridDesc) * S->grids_cap);
         if (e != cudaSuccess) return e;
     }
-    std::vector<TileDesc> tiles[4];
+    std::vector<TileDesc> tiles[kKinds];
+    for (int kd = 0; kd < kKinds; ++kd) S->kind_smem[kd] = 0;
     for (int g = 0; g < ng; ++g) {
         const Req *q = S->resident[g];
+        if (q->N >= kOwnLaunch) continue;
         const int kind = kind_of(q->r.dims, q->r.params.dtype);
+        S->kind_smem[kind] = std::max(S->kind_smem[kind], q->r.params.dtype == SP_F64 ? tile_smem<double>(q->r.model, q->stencil)
+                                                                                       : tile_smem<float>(q->r.model, q->stencil));
         if (q->r.dims == 2) {
             for (int y = 0; y < q->ny; y += kB2Y)
                 for (int x = 0; x < q->nx; x += kB2X) tiles[kind].push_back({g, x, y, 0});
@@ -250,7 +272,7 @@ static cudaError_t rebuild_tables(sp_server *S) {
         }
     }
     size_t total = 0;
-    for (int kd = 0; kd < 4; ++kd) {
+    for (int kd = 0; kd < kKinds; ++kd) {
         S->kind_off[kd] = (int)total;
         S->kind_n[kd] = (int)tiles[kd].size();
         total += tiles[kd].size();
@@ -263,7 +285,7 @@ static cudaError_t rebuild_tables(sp_server *S) {
     }
     std::vector<TileDesc> flat;
     flat.reserve(total);
-    for (int kd = 0; kd < 4; ++kd) flat.insert(flat.end(), tiles[kd].begin(), tiles[kd].end());
+    for (int kd = 0; kd < kKinds; ++kd) flat.insert(flat.end(), tiles[kd].begin(), tiles[kd].end());
     if (total) {
         cudaError_t e = cudaMemcpyAsync(S->d_tiles, flat.data(), sizeof(TileDesc) * total, cudaMemcpyHostToDevice,
                                         S->stream);
@@ -294,27 +316,93 @@ static cudaError_t upload_descriptors(sp_server *S, int Q) {
                            S->stream);
 }
 
-static cudaError_t run_quantum(sp_server *S, int Q) {
-    if (!S->graph_valid) {
-        if (S->graph) {
-            cudaGraphExecDestroy(S->graph);
-            S->graph = nullptr;
-        }
-        cudaGraph_t g = nullptr;
-        cudaError_t e = cudaStreamBeginCapture(S->stream, cudaStreamCaptureModeThreadLocal);
-        if (e != cudaSuccess) return e;
-        for (int j = 0; j < Q && e == cudaSuccess; ++j)
-            for (int kd = 0; kd < 4 && e == cudaSuccess; ++kd)
-                if (S->kind_n[kd] > 0)
-                    e = launch_batch(kd, S->d_grids, S->d_tiles + S->kind_off[kd], S->kind_n[kd], j, S->stream);
-        cudaError_t e2 = cudaStreamEndCapture(S->stream, &g);
-        if (e == cudaSuccess) e = e2;
-        if (e == cudaSuccess) e = cudaGraphInstantiate(&S->graph, g, 0);
-        if (g) cudaGraphDestroy(g);
-        if (e != cudaSuccess) return e;
-        S->graph_valid = true;
+// `from` waits for `to`'s work so far
+static cudaError_t chain(cudaStream_t from, cudaStream_t to, cudaEvent_t ev) {
+    const cudaError_t e = cudaEventRecord(ev, from);
+    return e != cudaSuccess ? e : cudaStreamWaitEvent(to, ev, 0);
+}
+
+// The batched launches of a quantum: Q launches per kind, the kinds (independent grids)
+// as parallel branches.
+static cudaError_t capture_quantum(sp_server *S, int Q) {
+    if (S->graph) {
+        cudaGraphExecDestroy(S->graph);
+        S->graph = nullptr;
     }
-    return cudaGraphLaunch(S->graph, S->stream);
+    cudaGraph_t g = nullptr;
+    cudaError_t e = cudaStreamBeginCapture(S->stream, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return e;
+    for (int kd = 0; kd < kKinds && e == cudaSuccess; ++kd) {
+        if (S->kind_n[kd] == 0) continue;
+        e = chain(S->stream, S->side[kd], S->fork);
+        for (int j = 0; j < Q && e == cudaSuccess; ++j)
+            e = launch_batch(kd, S->d_grids, S->d_tiles + S->kind_off[kd], S->kind_n[kd], S->kind_smem[kd], j, S->side[kd]);
+    }
+    for (int kd = 0; kd < kKinds; ++kd)  // also after an error, so that the capture can end
+        if (S->kind_n[kd] > 0) {
+            const cudaError_t e1 = chain(S->side[kd], S->stream, S->join[kd]);
+            if (e == cudaSuccess) e = e1;
+        }
+    const cudaError_t e2 = cudaStreamEndCapture(S->stream, &g);
+    if (e == cudaSuccess) e = e2;
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&S->graph, g, 0);
+    if (g) cudaGraphDestroy(g);
+    S->graph_valid = e == cudaSuccess;
+    return e;
+}
+
+// `steps` steps of one large grid from the level `parity` on; on return `parity` is the
+// current level.  One launch takes the library's default number of steps.
+static cudaError_t own_steps(const sp_server *S, const Req *q, int &parity, int steps, cudaStream_t s) {
+    const int spl = q->r.dims == 2 ? steps_per_launch(2, q->r.params.dtype, q->r.model, 0) : 1;
+    StepArgs a;
+    a.nx = q->nx;
+    a.ny = q->ny;
+    a.nz = q->nz;
+    a.k = q->k;
+    a.kf = to_float(q->k);
+    for (int j = 0; j < steps;) {
+        const int k = steps - j >= spl ? spl : 1, f1 = q->nf > 1 ? 1 : 0;
+        a.in0 = q->buf[parity][0];
+        a.in1 = q->buf[parity][f1];
+        a.out0 = q->buf[parity ^ 1][0];
+        a.out1 = q->buf[parity ^ 1][f1];
+        // (Cahn-Hilliard's two-pass kernels would need a buffer that admission does not count)
+        const bool pairs = q->r.model != SP_CAHN_HILLIARD &&
+                           planes27_applies(q->r.dims, q->r.params.dtype, q->stencil, q->r.model);
+        const cudaError_t e = pairs ? launch_planes27_f64(q->r.model, a, nullptr, s, S->n_sm)
+                              : q->r.params.dtype == SP_F64
+                                  ? launch_step_f64(q->r.model, q->stencil, a, s, S->n_sm, k)
+                                  : launch_step_f32(q->r.model, q->stencil, a, s, S->n_sm, k);
+        if (e != cudaSuccess) return e;
+        parity ^= 1;  // one launch swaps the levels
+        j += k;
+    }
+    return cudaSuccess;
+}
+
+// One quantum of every resident grid: the large ones on side streams, the batched graph
+// beside them, all joined into the server's stream.
+static cudaError_t run_quantum(sp_server *S, int Q) {
+    bool batch = false, used[kOwnStreams] = {};
+    for (int kd = 0; kd < kKinds; ++kd) batch = batch || S->kind_n[kd] > 0;
+    cudaError_t e = batch && !S->graph_valid ? capture_quantum(S, Q) : cudaSuccess;
+    if (e == cudaSuccess) e = cudaEventRecord(S->fork, S->stream);
+    if (e == cudaSuccess && batch) e = cudaGraphLaunch(S->graph, S->stream);
+    int next = 0;
+    for (Req *q : S->resident) {
+        if (q->N < kOwnLaunch || e != cudaSuccess) continue;
+        const int b = next++ % kOwnStreams;
+        if (!used[b]) e = cudaStreamWaitEvent(S->side[b], S->fork, 0);
+        used[b] = true;
+        if (e == cudaSuccess) e = own_steps(S, q, q->parity, (int)std::min<int64_t>(Q, q->steps_left), S->side[b]);
+    }
+    for (int b = 0; b < kOwnStreams; ++b)
+        if (used[b]) {
+            const cudaError_t e1 = chain(S->side[b], S->stream, S->join[b]);
+            if (e == cudaSuccess) e = e1;
+        }
+    return e;
 }
 
 static void finish_locked(sp_server *S, Req *q, int status) {
@@ -457,7 +545,7 @@ static void scheduler(sp_server *S) {
             const int64_t adv = std::min<int64_t>(Q, q->steps_left);
             q->steps_left -= adv;
             q->steps_done += adv;
-            q->parity ^= (int)(adv & 1);
+            if (q->N < kOwnLaunch) q->parity ^= (int)(adv & 1);  // own launches keep it themselves
             S->lups += (double)q->N * (double)adv;
             if (e != cudaSuccess || q->steps_left == 0) done.push_back(q);
             else keep.push_back(q);
@@ -496,6 +584,14 @@ extern "C" int sp_admission_order(int n, const size_t bytes[], const int priorit
     return na;
 }
 
+static void destroy_side(sp_server *S) {
+    for (int b = 0; b < kOwnStreams; ++b) {
+        if (S->side[b]) cudaStreamDestroy(S->side[b]);
+        if (S->join[b]) cudaEventDestroy(S->join[b]);
+    }
+    if (S->fork) cudaEventDestroy(S->fork);
+}
+
 extern "C" int sp_server_create(size_t hbm_budget_bytes, int max_slots, int quantum_steps, sp_server **out) {
     if (!out) return SP_EINVAL;
     *out = nullptr;
@@ -510,6 +606,11 @@ extern "C" int sp_server_create(size_t hbm_budget_bytes, int max_slots, int quan
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&S->n_sm, cudaDevAttrMultiProcessorCount, S->device);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&S->stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&S->ev, cudaEventBlockingSync | cudaEventDisableTiming);
+    for (int b = 0; b < kOwnStreams; ++b) {
+        if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&S->side[b], cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&S->join[b], cudaEventDisableTiming);
+    }
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&S->fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = set_batch_attributes();
     if (e == cudaSuccess) {
         S->nred = 2 * S->n_sm * kReduceBlocksPerSM;
@@ -520,6 +621,7 @@ extern "C" int sp_server_create(size_t hbm_budget_bytes, int max_slots, int quan
         cudaGetLastError();
         if (S->stream) cudaStreamDestroy(S->stream);
         if (S->ev) cudaEventDestroy(S->ev);
+        destroy_side(S);
         if (S->d_partials) cudaFree(S->d_partials);
         delete S;
         return SP_ECUDA;
@@ -660,6 +762,7 @@ extern "C" int sp_server_destroy(sp_server *S) {
     if (S->d_partials) cudaFree(S->d_partials);
     if (S->h_scalar) cudaFreeHost(S->h_scalar);
     if (S->ev) cudaEventDestroy(S->ev);
+    destroy_side(S);
     if (S->stream) cudaStreamDestroy(S->stream);
     delete S;
     return SP_OK;

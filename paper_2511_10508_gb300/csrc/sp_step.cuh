@@ -1137,8 +1137,8 @@ __global__ void __launch_bounds__(NT) step3d_zreg_kernel(StepArgs a, int tiles_x
 // (16 bytes per point) is cheap next to the FP64 work on this part.  Allen-Cahn
 // (mode 2), Gray-Scott (mode 3) and Model C (mode 4: phi and the density's chemical
 // potential, formed once per loaded point, are streamed; rho itself is read at the
-// output points) take one pass.  Tiles of 32 x 32, or 32 x 16 where the grid's edges
-// waste too much of the larger (small_tile).  Same operations in the same order as every other family, so the results are identical bit for bit.
+// output points) take one pass.  Same operations in the same order as every other
+// family, so the results are identical bit for bit.
 // The default for these grids; measured on GB300 against step3d_zreg_kernel:
 // Cahn-Hilliard 1024^3 17.5 vs 13.6 GLUPS, Allen-Cahn 512^3 29.6 vs 27.0,
 // Gray-Scott 512^3 14.9 vs 13.3.
@@ -1150,10 +1150,10 @@ struct Planes27Args {
     StepConsts k;
 };
 
-template <int MODE, int TY_>
+template <int MODE>
 struct Planes27Shape {
     static constexpr int NF = (MODE >= 3) ? 2 : 1;
-    static constexpr int TX = 32, TY = TY_, NT = 8 * TY;
+    static constexpr int TX = 32, TY = 16, NT = 128;
     static constexpr int WIN = TX + 2, HIN = TY + 2, AIN = WIN * HIN;
     static constexpr int AP = HIN * TX;                // pair sums of rows -1 .. TY
     static constexpr int EPT = (AIN + NT - 1) / NT;    // loaded cells per thread per field
@@ -1161,10 +1161,10 @@ struct Planes27Shape {
     static constexpr size_t smem_bytes = sizeof(double) * ((size_t)2 * NF * AIN + (size_t)NF * AP);
 };
 
-template <int MODE, int TY_>
-__global__ void __launch_bounds__(8 * TY_, (MODE >= 3 ? 1 : 2) * 32 / TY_)
+template <int MODE>
+__global__ void __launch_bounds__(128, MODE >= 3 ? 2 : 4)
     planes27_kernel(Planes27Args a, int tiles_x, long long planes_per_cta, long long total) {
-    typedef Planes27Shape<MODE, TY_> Sh;
+    typedef Planes27Shape<MODE> Sh;
     constexpr int NF = Sh::NF, TX = Sh::TX, TY = Sh::TY, NT = Sh::NT, WIN = Sh::WIN, AIN = Sh::AIN, AP = Sh::AP;
     constexpr int EPT = Sh::EPT, EOUT = Sh::EOUT, OSTEP = Sh::OSTEP;
     extern __shared__ __align__(16) unsigned char smem_raw[];

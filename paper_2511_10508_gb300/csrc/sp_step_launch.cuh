@@ -15,19 +15,19 @@
 
 namespace sp {
 
-// 3D FP64 tiles (x, y) per stencil radius, and the small tile for grids that the large
-// one covers badly.
-template <int r> struct Tiles64 { static constexpr int TX = (r == 1) ? 64 : 32, TY = 32, NT = 256; };
-constexpr int kSmallTX = 32, kSmallTY = 16, kSmallNT = 128;
-
-// The small tile wins where the large one's ragged edges cost more than a tenth in
-// points (both evaluate whole tiles), e.g. 71 x 35: 3 x 2 tiles of 32 x 32 against 3 x 3
-// of 32 x 16.  On whole tiles the large one reads fewer halo cells per point.
-inline bool small_tile(int nx, int ny, int TX, int TY) {
+// 3D FP64 tiles: 32 x 16 points, 128 threads.  Against 64 x 32 (27-point: 32 x 32) tiles of
+// 256 threads they are as fast or faster on whole tiles (256^3 7-point: Gray-Scott 711 ->
+// 708 us per step, Allen-Cahn 362 -> 357, Model C 748 -> 687; 27-point Gray-Scott 1127 ->
+// 1096) and waste less at ragged edges (236^3 Gray-Scott 658 -> 610).  Cahn-Hilliard is a little
+// faster with large tiles (256^3: two passes 566 against 574 us, the fused ring, whose
+// halo mu grows with the tile's edge, 635 against 664): it takes the small tile where
+// that covers 3 (fused: 10) percent fewer points.
+constexpr int kTX64 = 32, kTY64 = 16, kNT64 = 128;
+inline bool small_tile(int nx, int ny, int TX, int TY, double margin) {
     auto area = [&](int tx, int ty) {
         return (double)((nx + tx - 1) / tx) * tx * ((double)((ny + ty - 1) / ty) * ty);
     };
-    return area(kSmallTX, kSmallTY) < 0.9 * area(TX, TY);
+    return area(kTX64, kTY64) < margin * area(TX, TY);
 }
 
 constexpr int kMinRun = 32;  // 2D warp strips: rows per CTA at least
@@ -148,10 +148,10 @@ cudaError_t launch_zreg(const StepArgs &a, cudaStream_t s, int n_sm) {
 
 // FP64 27-point with shared pair sums: one pass per mode (Cahn-Hilliard: mode 0
 // then mode 1 through the mu buffer).
-template <int MODE, int TY>
-cudaError_t launch_planes27_tile(const Planes27Args &a, cudaStream_t s, int n_sm) {
-    typedef Planes27Shape<MODE, TY> Sh;
-    auto kern = planes27_kernel<MODE, TY>;
+template <int MODE>
+cudaError_t launch_planes27_mode(const Planes27Args &a, cudaStream_t s, int n_sm) {
+    typedef Planes27Shape<MODE> Sh;
+    auto kern = planes27_kernel<MODE>;
     static const int occ = [&] {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::smem_bytes);
         int o = 1;
@@ -164,12 +164,6 @@ cudaError_t launch_planes27_tile(const Planes27Args &a, cudaStream_t s, int n_sm
     kern<<<(unsigned)((total + planes - 1) / planes), Sh::NT, Sh::smem_bytes, s>>>(a, tx, planes, total);
     return cudaGetLastError();
 }
-template <int MODE>
-cudaError_t launch_planes27_mode(const Planes27Args &a, cudaStream_t s, int n_sm) {
-    return small_tile(a.nx, a.ny, 32, 32) ? launch_planes27_tile<MODE, 16>(a, s, n_sm)
-                                          : launch_planes27_tile<MODE, 32>(a, s, n_sm);
-}
-
 template <int ST, int MODE, int TY>
 cudaError_t launch_ring2pass_tile(const Planes27Args &a, cudaStream_t s, int n_sm) {
     typedef Ring2PassShape<ST, TY> Sh;
@@ -188,7 +182,7 @@ cudaError_t launch_ring2pass_tile(const Planes27Args &a, cudaStream_t s, int n_s
 }
 template <int ST, int MODE>
 cudaError_t launch_ring2pass_mode(const Planes27Args &a, cudaStream_t s, int n_sm) {
-    return small_tile(a.nx, a.ny, 32, 32) ? launch_ring2pass_tile<ST, MODE, 16>(a, s, n_sm)
+    return small_tile(a.nx, a.ny, 32, 32, 0.97) ? launch_ring2pass_tile<ST, MODE, 16>(a, s, n_sm)
                                           : launch_ring2pass_tile<ST, MODE, 32>(a, s, n_sm);
 }
 
@@ -389,10 +383,11 @@ cudaError_t launch_step_t(const StepArgs &a, cudaStream_t s, int n_sm, int k) {
         if constexpr (MODEL != MC) {
             if (ST == L27 && g_step_variant == 0) return launch_zreg<MODEL, T>(a, s, n_sm);
         }
-        typedef Tiles64<StencilInfo<ST>::r> TT;
-        if (small_tile(a.nx, a.ny, TT::TX, TT::TY))
-            return launch_step3d_tile<MODEL, ST, kSmallTX, kSmallTY, kSmallNT>(a, s, n_sm);
-        return launch_step3d_tile<MODEL, ST, TT::TX, TT::TY, TT::NT>(a, s, n_sm);
+        if constexpr (MODEL == CH) {
+            constexpr int TX = StencilInfo<ST>::r == 1 ? 64 : 32, TY = 32, NT = 256;
+            if (!small_tile(a.nx, a.ny, TX, TY, 0.9)) return launch_step3d_tile<MODEL, ST, TX, TY, NT>(a, s, n_sm);
+        }
+        return launch_step3d_tile<MODEL, ST, kTX64, kTY64, kNT64>(a, s, n_sm);
     }
     return cudaGetLastError();
 }
