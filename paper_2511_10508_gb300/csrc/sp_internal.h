@@ -140,9 +140,8 @@ cudaError_t launch_unfused_ch(int dtype, int stencil, const StepArgs &a, void *m
 // buffer.  Functions return SP_* status codes.  spectral_step with `more` set
 // also transforms the cubic term of the new field for the step that follows.
 struct SpectralPlan;
-int spectral_create(int dtype, int dims, int nx, int ny, int nz, double h, SpectralPlan **out);
+int spectral_create(int dtype, int dims, int nx, int ny, int nz, double h, double growth, SpectralPlan **out);
 void spectral_destroy(SpectralPlan *P);
-size_t spectral_bytes(const SpectralPlan *P);
 int spectral_load(SpectralPlan *P, const void *phi, cudaStream_t s);
 int spectral_step(SpectralPlan *P, int model, void *phi, double dt, double c1, double c2, double kappa, cudaStream_t s,
                   bool more);

@@ -385,7 +385,8 @@ extern "C" int sp_create(int model, int dims, const int64_t shape[3], double h, 
         return fail(SP_ECUDA, "initial condition: %s", cudaGetErrorString(e));
     }
     if (prm.scheme == SP_SCHEME_SPECTRAL) {
-        int rc = spectral_create(s->dtype, dims, s->nx, s->ny, s->nz, h, &s->spec);
+        // factor = dt max L(k) < 1: the fastest linear growth is 1 / (1 - factor) per step
+        int rc = spectral_create(s->dtype, dims, s->nx, s->ny, s->nz, h, 1.0 / (1.0 - factor), &s->spec);
         if (rc == SP_OK) rc = spectral_load(s->spec, s->f[0][0], s->stream);
         if (rc == SP_OK && cudaStreamSynchronize(s->stream) != cudaSuccess) rc = SP_ECUDA;
         if (rc != SP_OK) {

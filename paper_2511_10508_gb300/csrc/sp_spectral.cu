@@ -72,7 +72,7 @@ static bool factor_len(int n, FftLen *L) {
     return m == 1;
 }
 
-int spectral_create(int dtype, int dims, int nx, int ny, int nz, double h, SpectralPlan **out) {
+int spectral_create(int dtype, int dims, int nx, int ny, int nz, double h, double growth, SpectralPlan **out) {
     *out = nullptr;
     SpectralPlan *P = new (std::nothrow) SpectralPlan();
     if (!P) return SP_ENOMEM;
@@ -96,6 +96,18 @@ int spectral_create(int dtype, int dims, int nx, int ny, int nz, double h, Spect
             delete P;
             return SP_EINVAL;
         }
+    P->h = h;
+    // FP32 with G = 1 / (1 - dt max L(k)) > 4/3: the staged implementation (see its file)
+    if (!f64 && growth > 4.0 / 3.0) {
+        const int rc = staged::create(dims, nx, ny, nz, &P->stg);
+        if (rc != SP_OK) {
+            g_fft_err = "device allocation for the spectral plan failed";
+            delete P;
+            return rc;
+        }
+        *out = P;
+        return SP_OK;
+    }
     // twiddles of each distinct side (see FftStages, FftLen), in long double on the host,
     // rounded once to the working precision; squared wavenumbers of each axis in FP64,
     // rounded once
@@ -164,15 +176,12 @@ int spectral_create(int dtype, int dims, int nx, int ny, int nz, double h, Spect
 
 void spectral_destroy(SpectralPlan *P) {
     if (!P) return;
+    staged::destroy(P->stg);
     if (P->uh) cudaFree(P->uh);
     if (P->z) cudaFree(P->z);
     if (P->tw) cudaFree(P->tw);
     if (P->k2) cudaFree(P->k2);
     delete P;
-}
-
-size_t spectral_bytes(const SpectralPlan *P) {
-    return 2 * P->Nc * (P->dtype == SP_F64 ? sizeof(double2) : sizeof(float2));
 }
 
 // phi^ / N = forward transform of phi / N (after the initial condition or a write)
@@ -192,6 +201,12 @@ template <typename R> static int spectral_load_t(SpectralPlan *P, const R *phi, 
 }
 
 int spectral_load(SpectralPlan *P, const void *phi, cudaStream_t s) {
+    if (P->stg) {
+        const cudaError_t e = staged::load(P->stg, static_cast<const float *>(phi), s);
+        if (e == cudaSuccess) return SP_OK;
+        g_fft_err = std::string("forward transform: ") + cudaGetErrorString(e);
+        return SP_ECUDA;
+    }
     if (P->dtype == SP_F64) return spectral_load_t<double>(P, static_cast<const double *>(phi), s);
     return spectral_load_t<float>(P, static_cast<const float *>(phi), s);
 }
@@ -219,7 +234,8 @@ static cudaError_t spectral_step_t(SpectralPlan *P, int model, R *phi, double dt
 
 int spectral_step(SpectralPlan *P, int model, void *phi, double dt, double c1, double c2, double kappa, cudaStream_t s,
                   bool more) {
-    const cudaError_t e = P->dtype == SP_F64
+    const cudaError_t e = P->stg ? staged::step(P->stg, model, (float *)phi, P->h, dt, c1, c2, kappa, s, more)
+                          : P->dtype == SP_F64
                               ? spectral_step_t<double>(P, model, (double *)phi, dt, c1, c2, kappa, more, s)
                               : spectral_step_t<float>(P, model, (float *)phi, dt, c1, c2, kappa, more, s);
     if (e != cudaSuccess) {

@@ -33,7 +33,19 @@ template <typename R> struct Cplx;
 template <> struct Cplx<double> { typedef double2 type; };
 template <> struct Cplx<float> { typedef float2 type; };
 
+// The staged single-precision implementation (sp_spectral_staged.cu).
+namespace staged {
+struct Plan;
+int create(int dims, int nx, int ny, int nz, Plan **out);
+void destroy(Plan *P);
+cudaError_t load(Plan *P, const float *phi, cudaStream_t s);
+cudaError_t step(Plan *P, int model, float *phi, double h, double dt, double c1, double c2, double kappa, cudaStream_t s,
+                 bool more);
+}  // namespace staged
+
 struct SpectralPlan {
+    staged::Plan *stg;            // FP32 with strong linear growth: everything below but h is unused
+    double h;
     int dtype, dims, nx, ny, nz, nxh, n_sm;
     size_t N, Nc;                 // real points, half-spectrum modes
     FftLen lx, ly, lz;
