@@ -111,6 +111,19 @@ __device__ __forceinline__ void cp_async8(void *smem, const void *gmem) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem) : "memory");
 }
 
+// One element of a row whose start is not 16-byte aligned (rows of odd grids): 4 or 8
+// bytes asynchronously; 2-byte elements have no such copy and are moved at once.
+template <typename T> __device__ __forceinline__ void cp_async_elem(T *smem, const T *gmem) {
+    if constexpr (sizeof(T) == 4) {
+        const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem) : "memory");
+    } else if constexpr (sizeof(T) == 8) {
+        cp_async8(smem, gmem);
+    } else {
+        *smem = *gmem;
+    }
+}
+
 template <int N> __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }

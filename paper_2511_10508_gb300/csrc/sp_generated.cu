@@ -161,6 +161,7 @@ __device__ __forceinline__ void gen_seg(long long u, int segs, const StepArgs &a
 // Cahn-Hilliard pass 1: mu of every point
 template <int R, int DIMS, typename T>
 __global__ void __launch_bounds__(256) gen_mu_kernel(GenArgs g, int segs) {
+    pdl_enter();
     typedef typename Cmp<T>::type C;
     const StepArgs &a = g.a;
     const ConstsC<C> k(a.k, a.kf);
@@ -181,6 +182,7 @@ __global__ void __launch_bounds__(256) gen_mu_kernel(GenArgs g, int segs) {
 // one step of the model (Cahn-Hilliard: pass 2, from mu)
 template <int MODEL, int R, int DIMS, typename T>
 __global__ void __launch_bounds__(256) gen_step_kernel(GenArgs g, int segs) {
+    pdl_enter();
     typedef typename Cmp<T>::type C;
     const StepArgs &a = g.a;
     const ConstsC<C> k(a.k, a.kf);
@@ -296,6 +298,7 @@ struct GenTile2dShape {
 // three CTAs per SM where the registers allow it without spills (one-field models)
 template <int MODEL, int R, typename T, int BX, int BY, int NT>
 __global__ void __launch_bounds__(NT, (MODEL == GS || MODEL == MC) ? 2 : 3) gen_tile2d_kernel(GenArgs g) {
+    pdl_enter();
     typedef GenTile2dShape<MODEL, R, T, BX, BY> Sh;
     typedef typename Sh::C C;
     constexpr int RIN = Sh::RIN, CK = Sh::CK, NCK = Sh::NCK, SW = Sh::SW, X0 = Sh::X0, HIN = Sh::HIN;
@@ -320,11 +323,11 @@ __global__ void __launch_bounds__(NT, (MODEL == GS || MODEL == MC) ? 2 : 3) gen_
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
             T *dst = s_in + ((size_t)f * HIN + i) * SW + c * CK;
-            if (vec_ok && x >= 0 && x + CK <= nx) {
-                cp_async16(dst, in[f] + row + x);
+            if (vec_ok) {  // a chunk wraps as a whole
+                cp_async16(dst, in[f] + row + wrap_idx(x, nx));
             } else {
 #pragma unroll
-                for (int j = 0; j < CK; ++j) dst[j] = in[f][row + wrap_idx(x + j, nx)];
+                for (int j = 0; j < CK; ++j) cp_async_elem(dst + j, in[f] + row + wrap_idx(x + j, nx));
             }
         }
     }
@@ -455,16 +458,17 @@ static cudaError_t launch_gen_t(const GenArgs &g, cudaStream_t s, int n_sm) {
                 return true;
             }();
             (void)attr;
-            kern<<<dim3((g.a.nx + BX - 1) / BX, (g.a.ny + BY - 1) / BY), NT, Sh::smem_bytes, s>>>(g);
-            return cudaGetLastError();
+            return launch_pdl(kern, dim3((g.a.nx + BX - 1) / BX, (g.a.ny + BY - 1) / BY), dim3(NT), Sh::smem_bytes, s, g);
         }
     }
     const int segs = (g.a.nx + 255) / 256;
     const long long units = (long long)g.a.ny * g.a.nz * segs;
     const unsigned blocks = (unsigned)std::min<long long>(units, (long long)n_sm * 8);
-    if constexpr (MODEL == CH) gen_mu_kernel<R, DIMS, T><<<blocks, 256, 0, s>>>(g, segs);
-    gen_step_kernel<MODEL, R, DIMS, T><<<blocks, 256, 0, s>>>(g, segs);
-    return cudaGetLastError();
+    if constexpr (MODEL == CH) {
+        const cudaError_t e = launch_pdl(gen_mu_kernel<R, DIMS, T>, dim3(blocks), dim3(256), 0, s, g, segs);
+        if (e != cudaSuccess) return e;
+    }
+    return launch_pdl(gen_step_kernel<MODEL, R, DIMS, T>, dim3(blocks), dim3(256), 0, s, g, segs);
 }
 
 template <int MODEL, typename T>

@@ -79,9 +79,26 @@ inline int steps_per_launch_3d(int dtype, int model, int nx, int requested) {
     return (ok && requested >= 2) ? 2 : 1;
 }
 
-inline int steps_per_launch(int dims, int dtype, int model, int requested) {
+// 2D FP32 Allen-Cahn, Gray-Scott and Model C fuse steps by default: four up to 2^24 points
+// (radius-2 stencils, whose halo is twice as wide, 2^21), where the launch and the reuse in
+// L2 count (us per step with 2 and 4: Gray-Scott 2048^2 11.4 / 10.0, 4096^2 35.7 / 34.4, 8192^2
+// 128 / 130; Allen-Cahn 300 x 301 2.4 / 1.8; 4th order Allen-Cahn 3420 x 560 5.7 / 5.3, Model C
+// 4096^2 58 / 65), else two.  2D FP64 grids with a radius-1 stencil fuse two steps while the
+// 32 x 14 tiles of that kernel do not cost an SM one more tile than the 32 x 16 tiles of one step:
+// up to one tile per SM, and from two per SM up to 2^18 points (us per step with 1 and 2:
+// Allen-Cahn 256^2 3.5 / 2.7, 512^2 6.9 / 6.0, Gray-Scott 256^2 5.5 / 4.4; 257^2, where it does cost
+// one, 5.7 / 6.5).
+inline int steps_per_launch(int dims, int dtype, int model, int radius, int64_t nx, int64_t ny, int n_sm, int requested) {
     if (dims != 2 || model == SP_MODEL_H) return 1;
-    if (requested == 0) return (dtype == SP_F32 && model != CH) ? 2 : 1;
+    const int64_t npts = nx * ny;
+    if (requested == 0) {
+        if (dtype == SP_F64 && radius == 1 && npts <= (int64_t)1 << 18) {
+            const int64_t tx = (nx + 31) / 32, one = tx * ((ny + 15) / 16), two = tx * ((ny + 13) / 14);
+            return two <= n_sm || one >= 2 * n_sm ? 2 : 1;
+        }
+        if (dtype != SP_F32 || model == CH) return 1;
+        return npts <= (int64_t)1 << (radius == 1 ? 24 : 21) ? 4 : 2;
+    }
     if (requested >= 4) return 4;
     if (requested >= 2) return 2;
     return 1;
@@ -159,9 +176,11 @@ cudaError_t launch_reduce(int dtype, int what, const void *f, const ReduceGeom &
 cudaError_t launch_convert_from_f64(int dtype, const double *src, void *dst, uint64_t n, cudaStream_t s);
 cudaError_t launch_convert_to_f64(int dtype, const void *src, double *dst, uint64_t n, cudaStream_t s);
 
-// Launch with programmatic stream serialisation (the kernel calls pdl_enter()
-// before touching global memory): used where a launch is a few microseconds
-// long, so that the next step's CTAs are resident when this one completes.
+// Launch with programmatic stream serialisation (the kernel calls pdl_enter() before
+// touching global memory): the next step's CTAs are resident when this one completes,
+// about 0.5 us per launch (444 x 568 Cahn-Hilliard 2.96 -> 2.59 us per step).  Grids of many waves of
+// CTAs gain nothing and lose a little (16384^2 Gray-Scott, 131072 tiles: 4.84 -> 4.90 ms),
+// so they are launched plainly.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                        Args... args) {
@@ -174,7 +193,7 @@ cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t sme
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = (unsigned long long)grid.x * grid.y * grid.z <= 8192 ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 

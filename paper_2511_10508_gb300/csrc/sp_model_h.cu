@@ -73,6 +73,7 @@ __device__ __forceinline__ auto central(const Fn &f) -> decltype(f(0, 0, 0)) {
 
 template <int ST, typename T>
 __global__ void __launch_bounds__(256) mh_mu_kernel(MhArgs a, int segs) {
+    pdl_enter();
     typedef typename Cmp<T>::type C;
     constexpr int R = StencilInfo<ST>::r;
     const ConstsC<C> k(a.k, a.kf);
@@ -92,6 +93,7 @@ __global__ void __launch_bounds__(256) mh_mu_kernel(MhArgs a, int segs) {
 
 template <int ST, typename T, int DIMS>
 __global__ void __launch_bounds__(256) mh_update_kernel(MhArgs a, int segs, typename Cmp<T>::type c3g) {
+    pdl_enter();
     typedef typename Cmp<T>::type C;
     constexpr int R = StencilInfo<ST>::r;
     const ConstsC<C> k(a.k, a.kf);
@@ -155,6 +157,7 @@ struct MhTile2dShape {
 
 template <int ST, typename T, int BX, int BY, int NT>
 __global__ void __launch_bounds__(NT) mh_tile2d_kernel(MhArgs a, typename Cmp<T>::type c3g) {
+    pdl_enter();
     typedef MhTile2dShape<ST, T, BX, BY> Sh;
     typedef typename Sh::C C;
     constexpr int R = Sh::R, RIN = Sh::RIN, CK = Sh::CK, NCK = Sh::NCK, SW = Sh::SW, X0 = Sh::X0;
@@ -178,11 +181,11 @@ __global__ void __launch_bounds__(NT) mh_tile2d_kernel(MhArgs a, typename Cmp<T>
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
             T *dst = s_in + ((size_t)f * HIN + i) * SW + c * CK;
-            if (vec_ok && x >= 0 && x + CK <= nx) {
-                cp_async16(dst, in[f] + row + x);
+            if (vec_ok) {  // a chunk wraps as a whole
+                cp_async16(dst, in[f] + row + wrap_idx(x, nx));
             } else {
 #pragma unroll
-                for (int jj = 0; jj < CK; ++jj) dst[jj] = in[f][row + wrap_idx(x + jj, nx)];
+                for (int jj = 0; jj < CK; ++jj) cp_async_elem(dst + jj, in[f] + row + wrap_idx(x + jj, nx));
             }
         }
     }
@@ -242,6 +245,7 @@ struct MhRing3dShape {
 
 template <int ST, typename T, int TX, int TY, int NT>
 __global__ void __launch_bounds__(NT) mh_ring3d_kernel(MhArgs a, float c3g, int tiles_x, int tiles_y, int segs) {
+    pdl_enter();
     typedef float C;
     typedef MhRing3dShape<ST, T, TX, TY> Sh;
     constexpr int R = Sh::R, RIN = Sh::RIN, WIN = Sh::WIN, AIN = Sh::AIN, D = Sh::D, NF = Sh::NF;
@@ -358,8 +362,7 @@ static cudaError_t launch_mh_t(const MhArgs &a, double c3g, cudaStream_t s, int 
                 return true;
             }();
             (void)attr;
-            kern<<<dim3((a.nx + BX - 1) / BX, (a.ny + BY - 1) / BY), NT, Sh::smem_bytes, s>>>(a, (C)c3g);
-            return cudaGetLastError();
+            return launch_pdl(kern, dim3((a.nx + BX - 1) / BX, (a.ny + BY - 1) / BY), dim3(NT), Sh::smem_bytes, s, a, (C)c3g);
         }
     }
     if constexpr (StencilInfo<ST>::dims == 3 && !std::is_same<T, double>::value) {
@@ -378,19 +381,18 @@ static cudaError_t launch_mh_t(const MhArgs &a, double c3g, cudaStream_t s, int 
             const long long wave = (long long)n_sm * std::max(occ, 1);
             const int segs = lockstep_segments((long long)tx * ty, a.nz, 2 * Sh::RIN, wave);
             const long long items = (long long)tx * ty * segs;
-            kern<<<(unsigned)std::min(items, wave), NT, Sh::smem_bytes, s>>>(a, (C)c3g, tx, ty, segs);
-            return cudaGetLastError();
+            return launch_pdl(kern, dim3((unsigned)std::min(items, wave)), dim3(NT), Sh::smem_bytes, s, a, (C)c3g, tx, ty, segs);
         }
     }
     const int segs = (a.nx + 255) / 256;
     const long long units = (long long)a.ny * a.nz * segs;
     const unsigned blocks = (unsigned)std::min<long long>(units, (long long)n_sm * 8);
-    mh_mu_kernel<ST, T><<<blocks, 256, 0, s>>>(a, segs);
+    cudaError_t e = launch_pdl(mh_mu_kernel<ST, T>, dim3(blocks), dim3(256), 0, s, a, segs);
+    if (e != cudaSuccess) return e;
     if constexpr (StencilInfo<ST>::dims == 2)
-        mh_update_kernel<ST, T, 2><<<blocks, 256, 0, s>>>(a, segs, (C)c3g);
+        return launch_pdl(mh_update_kernel<ST, T, 2>, dim3(blocks), dim3(256), 0, s, a, segs, (C)c3g);
     else
-        mh_update_kernel<ST, T, 3><<<blocks, 256, 0, s>>>(a, segs, (C)c3g);
-    return cudaGetLastError();
+        return launch_pdl(mh_update_kernel<ST, T, 3>, dim3(blocks), dim3(256), 0, s, a, segs, (C)c3g);
 }
 
 template <typename T>

@@ -324,10 +324,6 @@ extern "C" int sp_create(int model, int dims, const int64_t shape[3], double h, 
     s->p.stencil = st;
     s->esize = dtype_size(prm.dtype);
     s->k = make_consts(*s);
-    s->spl = st == SP_LAP_GENERATED ? 1
-             : dims == 3 && prm.scheme == SP_SCHEME_FD
-                 ? steps_per_launch_3d(prm.dtype, model, (int)nx, prm.steps_per_launch)
-                 : steps_per_launch(dims, prm.dtype, model, prm.steps_per_launch);
     if (st == SP_LAP_GENERATED) generated_weights(prm.stencil_order, dims, s->genw, nullptr);
     s->variant = 0;
     s->tune_pending = (prm.flags & SP_FLAG_AUTOTUNE) != 0 && prm.steps_per_launch == 0;
@@ -339,6 +335,9 @@ extern "C" int sp_create(int model, int dims, const int64_t shape[3], double h, 
         release(s);
         return fail(SP_ECUDA, "device setup: %s", cudaGetErrorString(e));
     }
+    s->spl = st == SP_LAP_GENERATED || prm.scheme != SP_SCHEME_FD ? 1
+             : dims == 3 ? steps_per_launch_3d(prm.dtype, model, (int)nx, prm.steps_per_launch)
+                         : steps_per_launch(2, prm.dtype, model, stencil_radius(st), nx, ny, s->n_sm, prm.steps_per_launch);
     const size_t bytes = s->N * s->esize;
     for (int l = 0; l < 2; ++l)
         for (int f = 0; f < s->nf; ++f) {

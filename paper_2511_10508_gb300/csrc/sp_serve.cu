@@ -77,6 +77,7 @@ template <typename T> size_t largest_smem(int dims) {
 template <typename T>
 __global__ void __launch_bounds__(kBatchNT) batch2d_kernel(const GridDesc *__restrict__ grids,
                                                            const TileDesc *__restrict__ tiles, int j) {
+    pdl_enter();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const TileDesc td = tiles[blockIdx.x];
     const GridDesc &g = grids[td.grid];
@@ -99,6 +100,7 @@ __global__ void __launch_bounds__(kBatchNT) batch2d_kernel(const GridDesc *__res
 template <typename T>
 __global__ void __launch_bounds__(kBatchNT) batch3d_kernel(const GridDesc *__restrict__ grids,
                                                            const TileDesc *__restrict__ tiles, int j) {
+    pdl_enter();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const TileDesc td = tiles[blockIdx.x];
     const GridDesc &g = grids[td.grid];
@@ -140,12 +142,11 @@ static cudaError_t set_batch_attributes() {
 static cudaError_t launch_batch(int kind, const GridDesc *grids, const TileDesc *tiles, int ntiles, size_t smem, int j,
                                 cudaStream_t s) {
     switch (kind) {
-    case 0: batch2d_kernel<double><<<ntiles, kBatchNT, smem, s>>>(grids, tiles, j); break;
-    case 1: batch2d_kernel<float><<<ntiles, kBatchNT, smem, s>>>(grids, tiles, j); break;
-    case 2: batch3d_kernel<double><<<ntiles, kBatchNT, smem, s>>>(grids, tiles, j); break;
-    default: batch3d_kernel<float><<<ntiles, kBatchNT, smem, s>>>(grids, tiles, j); break;
+    case 0: return launch_pdl(batch2d_kernel<double>, dim3(ntiles), dim3(kBatchNT), smem, s, grids, tiles, j);
+    case 1: return launch_pdl(batch2d_kernel<float>, dim3(ntiles), dim3(kBatchNT), smem, s, grids, tiles, j);
+    case 2: return launch_pdl(batch3d_kernel<double>, dim3(ntiles), dim3(kBatchNT), smem, s, grids, tiles, j);
+    default: return launch_pdl(batch3d_kernel<float>, dim3(ntiles), dim3(kBatchNT), smem, s, grids, tiles, j);
     }
-    return cudaGetLastError();
 }
 
 // A grid of a million points and more fills the GPU by itself: it is stepped by the
@@ -354,7 +355,7 @@ static cudaError_t capture_quantum(sp_server *S, int Q) {
 // `steps` steps of one large grid from the level `parity` on; on return `parity` is the
 // current level.  One launch takes the library's default number of steps.
 static cudaError_t own_steps(const sp_server *S, const Req *q, int &parity, int steps, cudaStream_t s) {
-    const int spl = q->r.dims == 2 ? steps_per_launch(2, q->r.params.dtype, q->r.model, 0) : 1;
+    const int spl = q->r.dims == 3 ? 1 : steps_per_launch(2, q->r.params.dtype, q->r.model, q->stencil == SP_LAP_9CROSS4 ? 2 : 1, q->nx, q->ny, S->n_sm, 0);
     StepArgs a;
     a.nx = q->nx;
     a.ny = q->ny;

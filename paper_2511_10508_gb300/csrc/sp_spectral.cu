@@ -42,23 +42,23 @@ const char *spectral_last_error() { return g_fft_err.c_str(); }
 
 static bool is_pow2(int n) { return (n & (n - 1)) == 0; }
 
-// the stages of an n-point transform; false if n has another prime factor than 2, 3, 5, 7
-static bool factor_len(int n, FftLen *L) {
+// The stages of an n-point transform, `lines` of which make a pass; false if n has another
+// prime factor than 2, 3, 5, 7.  4 points per thread where 16 would leave an SM fewer than
+// four warps (256^2 FP64 75 -> 22 us per step, FP32 20 -> 8).
+static bool factor_len(int n, long long lines, int n_sm, FftLen *L) {
     L->n = n;
-    L->pow2 = is_pow2(n) && n >= 32;
     L->lgn = 0;
     while ((1 << L->lgn) < n) ++L->lgn;
-    L->nst = 0;
-    if (L->pow2) {
-        for (int v = 0; v < 2; ++v) {  // radix V, then as few stages as possible, of even radices
-            FftStages &S = L->reg[v];
-            const int lgv = v == 0 ? 4 : 2;
-            S.nst = 0;
-            S.lgr[S.nst++] = lgv;
-            for (int rest = L->lgn - lgv; rest > 0 && S.nst < 8; rest -= S.lgr[S.nst - 1]) {
-                const int left = (rest + lgv - 1) / lgv;
-                S.lgr[S.nst++] = (rest + left - 1) / left;
-            }
+    L->nst = L->V = 0;
+    if (is_pow2(n) && n >= 32) {
+        L->V = n <= 1024 && lines * (n / 16) < 4LL * 32 * n_sm ? 4 : 16;
+        FftStages &S = L->reg;  // radix V, then as few stages as possible, of even radices
+        const int lgv = L->V == 16 ? 4 : 2;
+        S.nst = 0;
+        S.lgr[S.nst++] = lgv;
+        for (int rest = L->lgn - lgv; rest > 0; rest -= S.lgr[S.nst - 1]) {
+            const int left = (rest + lgv - 1) / lgv;
+            S.lgr[S.nst++] = (rest + left - 1) / left;
         }
         return true;
     }
@@ -88,8 +88,16 @@ int spectral_create(int dtype, int dims, int nx, int ny, int nz, double h, doubl
     FftLen *ls[3] = {&P->lx, &P->ly, &P->lz};
     const bool f64 = dtype == SP_F64, pow2 = is_pow2(nx) && is_pow2(ny) && is_pow2(nz);
     const int longest = (f64 ? 4096 : 8192) / (pow2 ? 1 : 2);
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&P->n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        g_fft_err = "device look-up failed";
+        delete P;
+        return SP_ECUDA;
+    }
+    const long long lines[3] = {((long long)ny * nz + 1) / 2, (long long)P->nxh * nz, (long long)P->nxh * ny};
     for (int a = 0; a < 3; ++a)
-        if (sides[a] > longest || !factor_len(sides[a], ls[a])) {
+        if (sides[a] > longest || !factor_len(sides[a], lines[a], P->n_sm, ls[a])) {
             g_fft_err = std::string("the spectral scheme needs sides with prime factors 2, 3, 5, 7 of at most ") +
                         (f64 ? "4096 (FP64, powers of two; 2048 otherwise)" : "8192 (FP32, powers of two; 4096 otherwise)") +
                         " points (got " + std::to_string(sides[a]) + ")";
@@ -128,25 +136,23 @@ int spectral_create(int dtype, int dims, int nx, int ny, int nz, double h, doubl
         }
         int same = -1;
         for (int b = 0; b < a; ++b)
-            if (sides[b] == sides[a]) same = b;
+            if (sides[b] == sides[a] && ls[b]->V == L.V) same = b;
         if (same >= 0) {
             L.tw_off = ls[same]->tw_off;
-            for (int v = 0; v < 2; ++v) L.reg[v].tw_off = ls[same]->reg[v].tw_off;
+            L.reg.tw_off = ls[same]->reg.tw_off;
             continue;
         }
-        L.tw_off = (int)re.size();
-        if (!L.pow2)
+        L.tw_off = L.reg.tw_off = (int)re.size();
+        if (!L.V)
             for (int t = 0; t < L.n; ++t) root(t, L.n);
-        for (int v = 0; v < (L.pow2 ? 2 : 0); ++v) {
-            FftStages &S = L.reg[v];
-            S.tw_off = (int)re.size();
-            if (v == 1 && L.n > 1024) continue;  // never transformed with 4 points per thread
-            for (int i = 1, lgp = S.lgr[0]; i < S.nst; lgp += S.lgr[i++])
-                for (int l = 1; l <= S.lgr[i]; ++l)  // w^(R >> l) exp(-2 pi i m / 2^l)
+        else
+            for (int i = 1, lgp = L.reg.lgr[0]; i < L.reg.nst; lgp += L.reg.lgr[i++]) {
+                const int lgr = L.reg.lgr[i];
+                for (int l = 1; l <= lgr; ++l)  // w^(R >> l) exp(-2 pi i m / 2^l)
                     for (int m = 0; m < std::max(1, 1 << l >> 2); ++m)
                         for (int k = 0; k < (1 << lgp); ++k)
-                            root(((long long)k << (S.lgr[i] - l)) + ((long long)m << (lgp + S.lgr[i] - l)), 1 << (lgp + S.lgr[i]));
-        }
+                            root(((long long)k << (lgr - l)) + ((long long)m << (lgp + lgr - l)), 1 << (lgp + lgr));
+            }
     }
     const size_t rb = f64 ? sizeof(double) : sizeof(float), cb = 2 * rb;
     std::vector<unsigned char> host(re.size() * cb), host2(k2.size() * rb);
@@ -158,10 +164,7 @@ int spectral_create(int dtype, int dims, int nx, int ny, int nz, double h, doubl
         if (f64) reinterpret_cast<double *>(host2.data())[i] = k2[i];
         else reinterpret_cast<float *>(host2.data())[i] = (float)k2[i];
     }
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&P->n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaMalloc(&P->uh, P->Nc * cb) != cudaSuccess || cudaMalloc(&P->z, P->Nc * cb) != cudaSuccess ||
+    if (cudaMalloc(&P->uh, P->Nc * cb) != cudaSuccess || cudaMalloc(&P->z, P->Nc * cb) != cudaSuccess ||
         cudaMalloc(&P->tw, host.size()) != cudaSuccess || cudaMalloc(&P->k2, host2.size()) != cudaSuccess ||
         cudaMemcpy(P->tw, host.data(), host.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(P->k2, host2.data(), host2.size(), cudaMemcpyHostToDevice) != cudaSuccess) {

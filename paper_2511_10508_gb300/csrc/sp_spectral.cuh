@@ -22,8 +22,9 @@ struct FftStages {
 // One transform length.  A power of two from 32 on is transformed in registers
 // (fft_regs), other lengths by mixed-radix stages in shared memory (fft_lines).
 struct FftLen {
-    int n, pow2, lgn;      // pow2: the register transform
-    FftStages reg[2];      // 16 and 4 points per thread
+    int n, lgn;
+    int V;                 // points per thread of the register transform, 16 or 4; 0: mixed radices
+    FftStages reg;
     int nst, rad[kFftMaxStages];
     int tw_off;            // mixed: complex offset of exp(-2 pi i t / n), t < n, in the plan's table
     int k2_off;            // real offset of (2 pi freq(m) / (n h))^2, m < n, in the plan's wavenumber table
@@ -221,7 +222,7 @@ template <int LGR, int V, typename C> __device__ __forceinline__ void unscramble
 template <int V, typename C>
 __device__ __forceinline__ void fft_regs(C (&u)[V], C *buf, const FftLen &L, const C *tw_all, const LineThread &lt) {
     constexpr int LGV = V == 16 ? 4 : 2;
-    const FftStages &S = L.reg[V == 16 ? 0 : 1];
+    const FftStages &S = L.reg;
     const int t = lt.t, lgT = lt.lgT, sh = pad_shift<V>(L.n);
     const int rd = slot_of(t, sh), rinc = slot_of(1 << lgT, sh);
     const C *tw = tw_all + S.tw_off;
@@ -739,30 +740,27 @@ inline int lines_per_cta(int most, int least, long long lines, int n_sm) {
     return std::max(G, least);
 }
 
-// geometry, threads, points per thread (V; 0: mixed radices) and shared memory of a
-// pass; a CTA interleaves up to 2^lgI_max lines
+// geometry, threads and shared memory of a pass; a CTA interleaves up to 2^lgI_max lines
 template <typename R>
-void pass_shape(const SpectralPlan *P, const FftLen &L, long long lines, int lgI_max, PassGeom &g, int &threads, int &V,
+void pass_shape(const SpectralPlan *P, const FftLen &L, long long lines, int lgI_max, PassGeom &g, int &threads,
                 size_t &smem) {
     constexpr size_t cb = 2 * sizeof(R);
     g.ny = P->ny;
     g.nz = P->nz;
     g.nxh = P->nxh;
     g.nrows = P->ny * P->nz;
-    if (L.pow2) {
-        V = L.n <= 1024 && lines * (L.n / 16) < 4LL * 32 * P->n_sm ? 4 : 16;
-        const int T = L.n / V, most = std::max(1, (L.n >= 4096 ? FftBounds<R>::NT : 256) / T);
+    if (L.V) {
+        const int T = L.n / L.V, most = std::max(1, (L.n >= 4096 ? FftBounds<R>::NT : 256) / T);
         g.G = lines_per_cta(most, std::max(1, 32 / T), lines, P->n_sm);
         g.lgI = 0;
         while (g.lgI < lgI_max && (2 << g.lgI) <= g.G) ++g.lgI;
         // lines of adjacent threads start in different banks
         const int phase = sizeof(R) == 8 ? 8 : 16, want = g.lgI ? std::max(1, phase >> g.lgI) : 0;
-        g.LS = L.n + (L.n >> (V == 16 ? pad_shift<16>(L.n) : pad_shift<4>(L.n)));
+        g.LS = L.n + (L.n >> (L.V == 16 ? pad_shift<16>(L.n) : pad_shift<4>(L.n)));
         while (g.lgI && g.LS % phase != want % phase) ++g.LS;
         threads = g.G * T;
         smem = cb * (size_t)g.G * g.LS;
     } else {
-        V = 0;
         const int T = (L.n + kMixV - 1) / kMixV;
         int most = std::max(1, 256 / T);
         while (most > 1 && 2 * cb * most * L.n > 48 * 1024) --most;
@@ -786,14 +784,15 @@ static cudaError_t rows_mode(const SpectralPlan *P, R *f, typename Cplx<R>::type
     typedef typename Cplx<R>::type C;
     PassGeom g{};
     int threads;
-    int V;
     size_t smem;
     g.nlines = (P->ny * P->nz + 1) / 2;
     // FP32: adjacent threads take up to four row pairs, 64 bytes of every mode (one pair
     // is half a sector: 128^3 47.1 us per step with one, 40.2 with two, 37.3 with four)
-    pass_shape<R>(P, P->lx, g.nlines, sizeof(R) == 4 ? 2 : 0, g, threads, V, smem);
+    pass_shape<R>(P, P->lx, g.nlines, sizeof(R) == 4 ? 2 : 0, g, threads, smem);
     const unsigned blocks = (unsigned)((g.nlines + g.G - 1) / g.G);
-    auto kern = V == 16 ? rows_regs_kernel<R, MODE, 16> : V == 4 ? rows_regs_kernel<R, MODE, 4> : rows_mixed_kernel<R, MODE>;
+    auto kern = P->lx.V == 16  ? rows_regs_kernel<R, MODE, 16>
+                : P->lx.V == 4 ? rows_regs_kernel<R, MODE, 4>
+                               : rows_mixed_kernel<R, MODE>;
     const cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     return launch_pdl(kern, dim3(blocks), dim3(threads), smem, s, f, Z, g, coef, P->lx, static_cast<const C *>(P->tw));
@@ -816,20 +815,19 @@ static cudaError_t lines_mode(const SpectralPlan *P, int axis, const SpecCoef<R>
     const FftLen &L = axis == 1 ? P->ly : P->lz;
     PassGeom g{};
     int threads;
-    int V;
     size_t smem;
     const long long lines = (long long)P->nxh * (axis == 1 ? P->nz : P->ny);
     g.nlines = (int)lines;
-    pass_shape<R>(P, L, lines, axis == 1 ? 0 : 4, g, threads, V, smem);
+    pass_shape<R>(P, L, lines, axis == 1 ? 0 : 4, g, threads, smem);
     unsigned blocks = (unsigned)((lines + g.G - 1) / g.G);
     if (axis == 2) {
         g.per_kx = (P->ny + g.G - 1) / g.G;
         blocks = (unsigned)(P->nxh * g.per_kx);
     }
     g.ahead = axis == 1 && lines * L.n * 2 * sizeof(R) > (32u << 20) ? 2 * P->n_sm : 0;
-    auto kern = V == 16 ? lines_regs_kernel<R, MODE, MODEL, 16>
-                : V == 4 ? lines_regs_kernel<R, MODE, MODEL, 4>
-                         : lines_mixed_kernel<R, MODE, MODEL>;
+    auto kern = L.V == 16  ? lines_regs_kernel<R, MODE, MODEL, 16>
+                : L.V == 4 ? lines_regs_kernel<R, MODE, MODEL, 4>
+                           : lines_mixed_kernel<R, MODE, MODEL>;
     const cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     const R *k2 = static_cast<const R *>(P->k2);

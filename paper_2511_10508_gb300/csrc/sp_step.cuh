@@ -22,6 +22,8 @@
 //   step3d_box_kernel    3D, FP32/BF16 Model C: one CTA per box
 #pragma once
 
+#include <type_traits>
+
 #include "sp_common.cuh"
 
 namespace sp {
@@ -63,6 +65,7 @@ struct Step2dBatchShape {
 
 template <int MODEL, int ST, typename T, int NT, int RB>
 __global__ void __launch_bounds__(NT) step2d_batch_kernel(StepArgs a, int strips, long long rows_per_cta) {
+    pdl_enter();
     typedef Step2dBatchShape<MODEL, ST, T, NT, RB> Sh;
     typedef typename Sh::C C;
     constexpr int r = Sh::r, RIN = Sh::RIN, TW = Sh::TW, WIN = Sh::WIN, DIN = Sh::DIN, NF = Sh::NF;
@@ -277,11 +280,11 @@ __device__ __forceinline__ void tile2d(const T *in0, const T *in1, T *out0, T *o
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
             T *dst = s_in + ((size_t)f * HIN + i) * SW + c * CK;
-            if (vec_ok && x >= 0 && x + CK <= nx) {
-                cp_async16(dst, in[f] + row + x);
+            if (vec_ok) {  // a chunk wraps as a whole
+                cp_async16(dst, in[f] + row + wrap_idx(x, nx));
             } else {
 #pragma unroll
-                for (int j = 0; j < CK; ++j) dst[j] = in[f][row + wrap_idx(x + j, nx)];
+                for (int j = 0; j < CK; ++j) cp_async_elem(dst + j, in[f] + row + wrap_idx(x + j, nx));
             }
         }
     }
@@ -396,11 +399,11 @@ __global__ void __launch_bounds__(NT) step2d_tb_kernel(StepArgs a) {
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
             T *dst = buf + ((size_t)f * HIN + i) * SW + c * CK;
-            if (vec_ok && x >= 0 && x + CK <= nx) {
-                cp_async16(dst, in[f] + row + x);
+            if (vec_ok) {  // a chunk wraps as a whole
+                cp_async16(dst, in[f] + row + wrap_idx(x, nx));
             } else {
 #pragma unroll
-                for (int j = 0; j < CK; ++j) dst[j] = in[f][row + wrap_idx(x + j, nx)];
+                for (int j = 0; j < CK; ++j) cp_async_elem(dst + j, in[f] + row + wrap_idx(x + j, nx));
             }
         }
     }
@@ -507,8 +510,8 @@ __device__ __forceinline__ void box3d(const T *in0, const T *in1, T *out0, T *ou
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
             T *dst = s_in + (((size_t)f * DIN + zi) * HIN + i) * SW + c * CK;
-            if (vec_ok && x >= 0 && x + CK <= nx) {
-                cp_async16(dst, in[f] + row + x);
+            if (vec_ok) {  // a chunk wraps as a whole
+                cp_async16(dst, in[f] + row + wrap_idx(x, nx));
             } else {
 #pragma unroll
                 for (int j = 0; j < CK; ++j) dst[j] = in[f][row + wrap_idx(x + j, nx)];
@@ -565,6 +568,7 @@ __device__ __forceinline__ void box3d(const T *in0, const T *in1, T *out0, T *ou
 // One CTA per BX x BY x BZ box of a single grid (Model C, FP32 / BF16 3D).
 template <int MODEL, int ST, typename T, int BX, int BY, int BZ, int NT>
 __global__ void __launch_bounds__(NT) step3d_box_kernel(StepArgs a) {
+    pdl_enter();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const ConstsC<typename Cmp<T>::type> k(a.k, a.kf);
     box3d<MODEL, ST, T, BX, BY, BZ, NT>(static_cast<const T *>(a.in0), static_cast<const T *>(a.in1),
@@ -587,8 +591,12 @@ __global__ void __launch_bounds__(NT) step3d_box_kernel(StepArgs a) {
 // flight per warp.  Same expressions in the same order as the other FP32
 // kernels, so results are identical to them bit for bit.
 //
-// Requirements (checked by the launcher): nx a multiple of V and 16-byte
-// aligned field pointers, so that every vector, wrapped or not, is aligned.
+// AL: nx is a multiple of V and the field pointers are 16-byte aligned, so that every
+// vector, wrapped or not, is aligned.  Otherwise (FP32) a warp copies its row of 32 V
+// cells element by element, consecutive lanes consecutive cells, and its outputs reach
+// global memory the same way through 512 bytes of shared memory: 1503 x 1001
+// Cahn-Hilliard 4th order 10.6 us per step in tiles, 6.8 now; 4097 x 4095 5-point 53.7 ->
+// 30.2 (aligned 4096^2: 23.2).
 template <int MODEL, int ST, typename T>
 struct Step2dWarpShape {
     typedef typename Cmp<T>::type C;
@@ -600,19 +608,22 @@ struct Step2dWarpShape {
     static constexpr int XW = V + 2 * r;       // a row of the window: own vector plus r halo each side
     static constexpr int OUT_COLS = 30 * V;    // output columns per strip
     static constexpr int D = (NF == 1 && sizeof(T) == 2) ? 12 : 8;  // rows in the per-warp load ring
-    static constexpr size_t warp_smem = (size_t)D * NF * 32 * 16;
+    __host__ __device__ static constexpr size_t warp_smem(bool al) { return (size_t)(D * NF + (al ? 0 : NF)) * 32 * 16; }
     static_assert(V >= 2 * r, "the halo lanes must cover the mu halo");
 };
 
-template <int MODEL, int ST, typename T, int NT>
+template <int MODEL, int ST, typename T, int NT, bool AL>
 __global__ void __launch_bounds__(NT) step2d_warp_kernel(StepArgs a, int strips, int groups, long long rows_per_cta) {
+    pdl_enter();
     typedef Step2dWarpShape<MODEL, ST, T> Sh;
     typedef typename Sh::C C;
     typedef uint4 W;
     constexpr int r = Sh::r, V = Sh::V, RIN = Sh::RIN, NF = Sh::NF, U = Sh::U, XW = Sh::XW, D = Sh::D;
     constexpr unsigned FULL = 0xffffffffu;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    W *ring = reinterpret_cast<W *>(smem_raw) + (size_t)(threadIdx.x >> 5) * D * NF * 32;  // [D][NF][32]
+    W *ring = reinterpret_cast<W *>(smem_raw) + (threadIdx.x >> 5) * (Sh::warp_smem(AL) / 16);  // [D][NF][32]
+    T *stage = reinterpret_cast<T *>(ring + (size_t)D * NF * 32);                              // [NF][32 V] (not AL)
+    (void)stage;
 
     const ConstsC<C> k(a.k, a.kf);
     const ConstsF2 k2(k);
@@ -638,15 +649,48 @@ __global__ void __launch_bounds__(NT) step2d_warp_kernel(StepArgs a, int strips,
         const int col = strip * Sh::OUT_COLS + (lane - 1) * V;  // first column of this lane
         const int colw = wrap_idx(col, nx);
         const bool store = lane >= 1 && lane <= 30 && col < nx;
+        // not AL: cells lane + 32 q of the warp's row, which starts at the strip's left halo
+        const int left = strip * Sh::OUT_COLS - V;
+        int cw[AL ? 1 : V];
+        if constexpr (!AL) {
+#pragma unroll
+            for (int q = 0; q < V; ++q) cw[q] = wrap_idx(left + lane + 32 * q, nx);
+        }
+        (void)cw;
+        // output row: V cells of every lane of field f
+        auto put = [&](int f, size_t row, const C (&o)[V]) {
+            if constexpr (AL) {
+                if (store) store_vec<T, V>(out[f] + row + col, o);
+            } else {
+                T *st = stage + f * 32 * V;
+                __syncwarp();  // the previous row has left the buffer
+                store_vec<T, V>(st + lane * V, o);
+                __syncwarp();
+#pragma unroll
+                for (int q = 0; q < V; ++q) {
+                    const int e = lane + 32 * q;
+                    if (e >= V && e < 31 * V && left + e < nx) out[f][row + left + e] = st[e];
+                }
+            }
+        };
         const int jbeg = y0 - RIN;
         const int n = (y1 - y0) + 2 * RIN;
 
         // row i of the segment goes to ring slot i % D; one cp.async group per row
         auto issue = [&](int i) {
             if (i < n) {
-                const size_t off = (size_t)wrap_idx(jbeg + i, ny) * nx + colw;
+                const size_t row = (size_t)wrap_idx(jbeg + i, ny) * nx;
 #pragma unroll
-                for (int f = 0; f < NF; ++f) cp_async16(&ring[((i % D) * NF + f) * 32 + lane], in[f] + off);
+                for (int f = 0; f < NF; ++f) {
+                    W *dst = &ring[((i % D) * NF + f) * 32];
+                    if constexpr (AL) {
+                        cp_async16(dst + lane, in[f] + row + colw);
+                    } else {
+#pragma unroll
+                        for (int q = 0; q < V; ++q)
+                            cp_async_elem(reinterpret_cast<T *>(dst) + lane + 32 * q, in[f] + row + cw[q]);
+                    }
+                }
             }
             cp_async_commit();  // empty groups keep the count uniform
         };
@@ -663,8 +707,10 @@ __global__ void __launch_bounds__(NT) step2d_warp_kernel(StepArgs a, int strips,
                 if (i < n) {
                     const int j = jbeg + i;
                     // the slot read in the previous iteration is refilled; row i has landed
+                    if constexpr (!AL) __syncwarp();  // every lane has read it
                     issue(i + D - 1);
                     cp_async_wait<D - 1>();
+                    if constexpr (!AL) __syncwarp();  // every lane's cells have landed
                     // unpack row j and extend it with the neighbouring lanes' edge values
 #pragma unroll
                     for (int f = 0; f < NF; ++f) {
@@ -711,7 +757,7 @@ __global__ void __launch_bounds__(NT) step2d_warp_kernel(StepArgs a, int strips,
                                     o[c] = o2.x;
                                     o[c + 1] = o2.y;
                                 }
-                                if (store) store_vec<T, V>(out[0] + (size_t)(j - 2 * r) * nx + col, o);
+                                put(0, (size_t)(j - 2 * r) * nx, o);
                             }
                         }
                     } else {
@@ -734,11 +780,8 @@ __global__ void __launch_bounds__(NT) step2d_warp_kernel(StepArgs a, int strips,
                                                                second_sum<MODEL, ST, C>(P0, P1, k), k, o0[c], o1[c]);
                                 }
                             }
-                            if (store) {
-                                const size_t o = (size_t)(j - r) * nx + col;
-                                store_vec<T, V>(out[0] + o, o0);
-                                if constexpr (num_fields<MODEL>() == 2) store_vec<T, V>(out[NF - 1] + o, o1);
-                            }
+                            put(0, (size_t)(j - r) * nx, o0);
+                            if constexpr (num_fields<MODEL>() == 2) put(NF - 1, (size_t)(j - r) * nx, o1);
                         }
                     }
 #undef SLOT
@@ -773,6 +816,7 @@ struct Step3dShape {
 
 template <int MODEL, int ST, typename T, int TX, int TY, int NT>
 __global__ void __launch_bounds__(NT) step3d_kernel(StepArgs a, int tiles_x, int tiles_y, long long planes_per_cta) {
+    pdl_enter();
     typedef Step3dShape<MODEL, ST, T, TX, TY, NT> Sh;
     typedef typename Sh::C C;
     constexpr int r = Sh::r, RIN = Sh::RIN, WIN = Sh::WIN, AIN = Sh::AIN, DIN = Sh::DIN, NF = Sh::NF;
@@ -964,6 +1008,7 @@ __device__ __forceinline__ double combine27(double fm, double f0, double fp, dou
 template <int MODEL, int TX, int TY, int NT>
 __global__ void __launch_bounds__(NT) step3d_zreg_kernel(StepArgs a, int tiles_x, int tiles_y,
                                                          long long planes_per_cta) {
+    pdl_enter();
     static_assert(MODEL != MC, "Model C runs on the accessor-based kernels");
     typedef Step3dZregShape<MODEL, TX, TY, NT> Sh;
     typedef double C;
@@ -1164,6 +1209,7 @@ struct Planes27Shape {
 template <int MODE>
 __global__ void __launch_bounds__(128, MODE >= 3 ? 2 : 4)
     planes27_kernel(Planes27Args a, int tiles_x, long long planes_per_cta, long long total) {
+    pdl_enter();
     typedef Planes27Shape<MODE> Sh;
     constexpr int NF = Sh::NF, TX = Sh::TX, TY = Sh::TY, NT = Sh::NT, WIN = Sh::WIN, AIN = Sh::AIN, AP = Sh::AP;
     constexpr int EPT = Sh::EPT, EOUT = Sh::EOUT, OSTEP = Sh::OSTEP;
@@ -1297,6 +1343,7 @@ struct Ring2PassShape {
 template <int ST, int MODE, int TY_>
 __global__ void __launch_bounds__(8 * TY_, 64 / TY_)
     ring2pass_kernel(Planes27Args a, int tiles_x, long long planes_per_cta, long long total) {
+    pdl_enter();
     typedef Ring2PassShape<ST, TY_> Sh;
     constexpr int R = Sh::R, TX = Sh::TX, NT = Sh::NT, WIN = Sh::WIN, AIN = Sh::AIN, D = Sh::D;
     constexpr int EPT = Sh::EPT, EOUT = Sh::EOUT, OSTEP = Sh::OSTEP;
@@ -1371,6 +1418,37 @@ __global__ void __launch_bounds__(8 * TY_, 64 / TY_)
     }
 }
 
+struct NoRow {  // stands for RaggedRow where rows are aligned
+    __device__ __forceinline__ NoRow(int, int, int) {}
+};
+
+// A warp's row of 128 cells (lane l holds cells 4 l .. 4 l + 3) of a grid whose rows are not
+// 16-byte aligned: copied in and written out element by element, consecutive lanes
+// consecutive cells.  left: column of cell 0; cells 4 .. 123 are outputs.
+struct RaggedRow {
+    int left, lane, cw[4];
+    __device__ __forceinline__ RaggedRow(int left_, int lane_, int nx) : left(left_), lane(lane_) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) cw[q] = wrap_idx(left + lane + 32 * q, nx);
+    }
+    // row: the grid row's first element; dst: the 128 cells in shared memory
+    template <typename T> __device__ __forceinline__ void fetch(T *dst, const T *row) const {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) cp_async_elem(dst + lane + 32 * q, row + cw[q]);
+    }
+    // this lane's 4 outputs, through 512 bytes of shared memory of the warp
+    __device__ __forceinline__ void put(float *row, float *stage, const float (&o)[4], int nx) const {
+        __syncwarp();  // the previous row has left the buffer
+        store_vec<float, 4>(stage + 4 * lane, o);
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int e = lane + 32 * q;
+            if (e >= 4 && e < 124 && left + e < nx) row[left + e] = stage[e];
+        }
+    }
+};
+
 // ===================================================== 3D, warp rows ==
 //
 // FP32 / BF16-storage 3D kernel built like the 2D warp-strip kernel.  Warp w
@@ -1392,8 +1470,9 @@ __global__ void __launch_bounds__(8 * TY_, 64 / TY_)
 // Same expressions in the same order as the other FP32 kernels: identical
 // results bit for bit.
 //
-// Requirements (checked by the launcher): nx a multiple of 4 and 16-byte
-// aligned field pointers.
+// AL: nx is a multiple of 4 and the field pointers are 16-byte aligned.  Otherwise (FP32)
+// rows go through RaggedRow: 301 x 299 x 303 Cahn-Hilliard 7-point 162 us per step with the
+// register-staged kernel that took such grids before, @@ now (aligned 300^3 @@).
 
 // Number of in-plane partial sums per plane.
 template <int ST> struct Planar { static constexpr int NP = (ST == L7) ? 1 : 2; };
@@ -1462,15 +1541,17 @@ struct Step3dWrShape {
     static constexpr size_t mu_plane = (size_t)HIN * 32 * V;
     static constexpr size_t mu_bytes = (MODEL == CH) ? 2 * mu_plane * sizeof(float) : 0;
     static constexpr size_t smem_bytes = in_bytes + mu_bytes;
+    static constexpr size_t stage_bytes = (size_t)HIN * NF * 512;  // not AL: output rows
     // resident CTAs per SM asked of the register allocator (measured on GB300:
     // Allen-Cahn with radius-1 stencils gains from a third CTA; Cahn-Hilliard
     // 7-point needs two; elsewhere a bound would make the queues spill)
     static constexpr int MINB = (MODEL == AC && r == 1) ? 3 : ((MODEL == CH && ST == L7) ? 2 : 1);
 };
 
-template <int MODEL, int ST, typename T, int TY>
+template <int MODEL, int ST, typename T, int TY, bool AL>
 __global__ void __launch_bounds__(Step3dWrShape<MODEL, ST, T, TY>::NT, Step3dWrShape<MODEL, ST, T, TY>::MINB)
     step3d_wr_kernel(StepArgs a, int tiles_x, int tiles_y, int segs) {
+    pdl_enter();
     static_assert(MODEL != MC, "Model C runs on the accessor-based kernels");
     typedef Step3dWrShape<MODEL, ST, T, TY> Sh;
     typedef float C;
@@ -1498,6 +1579,8 @@ __global__ void __launch_bounds__(Step3dWrShape<MODEL, ST, T, TY>::NT, Step3dWrS
     constexpr size_t SLOT = (size_t)NF * HIN * 32, FLD = (size_t)HIN * 32;
     W *const s_own = s_in + (size_t)w * 32 + lane;
     float *const mu_own = s_mu + ((size_t)w * 32 + lane) * V;
+    float *const stage = reinterpret_cast<float *>(smem_raw + Sh::smem_bytes) + (size_t)w * NF * 128;  // not AL
+    (void)stage;
     // chunk at row offset dy of field f in the slot starting at `base`, widened
     auto ring_chunk = [&](const W *base, int f, int dy, float *dst) {
         union { W q; T t[V]; } u;
@@ -1522,20 +1605,30 @@ __global__ void __launch_bounds__(Step3dWrShape<MODEL, ST, T, TY>::NT, Step3dWrS
         const int n = (z1 - z0) + 2 * R;                           // planes fetched
         const int niter = n + (MODEL == CH ? 1 : 0);              // CH: the output stage lags one plane
         const int col = x0 + (lane - 1) * V;                       // first cell of this lane's chunk
-        const size_t goff = (size_t)wrap_idx(y0 - R + w, ny) * nx + wrap_idx(col, nx);
+        const size_t goff = (size_t)wrap_idx(y0 - R + w, ny) * nx + (AL ? wrap_idx(col, nx) : 0);
         const int yo = y0 - R + w;                                 // output row (if out_row)
         const bool store = out_row && lane >= 1 && lane <= 30 && col < nx && yo < ny;
+        const typename std::conditional<AL, NoRow, RaggedRow>::type rag(x0 - V, lane, nx);
+        // V outputs of every lane to row yo of field f, plane at dst_off
+        size_t dst_off = (size_t)z0 * plane + (size_t)yo * nx + (AL ? col : 0);
+        auto put = [&](int f, const float (&o)[V]) {
+            if constexpr (AL) {
+                if (store) store_vec<T, V>(out[f] + dst_off, o);
+            } else {
+                if (yo < ny) rag.put(out[f] + dst_off, stage + f * 128, o, nx);
+            }
+        };
         // element offsets: next plane to fetch (plane jn, wrapped z zn) and next output
         int jn = 0, zn = wrap_idx(z0 - R, nz);
         size_t src = (size_t)zn * plane + goff;
-        size_t dst_off = (size_t)z0 * plane + (size_t)yo * nx + col;
 
         auto issue = [&]() {
             if (jn < n) {
                 W *dst = s_own + (size_t)(jn & (D - 1)) * SLOT;
 #pragma unroll
                 for (int f = 0; f < NF; ++f) {
-                    if constexpr (CB == 16) cp_async16(dst + f * FLD, in[f] + src);
+                    if constexpr (!AL) rag.fetch(reinterpret_cast<T *>(dst + f * FLD - lane), in[f] + src);
+                    else if constexpr (CB == 16) cp_async16(dst + f * FLD, in[f] + src);
                     else cp_async8(dst + f * FLD, in[f] + src);
                 }
                 src += plane;
@@ -1623,7 +1716,7 @@ __global__ void __launch_bounds__(Step3dWrShape<MODEL, ST, T, TY>::NT, Step3dWrS
                                     o[2 * q] = o2.x;
                                     o[2 * q + 1] = o2.y;
                                 }
-                                if (store) store_vec<T, V>(out[0] + dst_off, o);
+                                put(0, o);
                                 dst_off += plane;
                             }
                         }
@@ -1687,10 +1780,8 @@ __global__ void __launch_bounds__(Step3dWrShape<MODEL, ST, T, TY>::NT, Step3dWrS
                                 o1[2 * q] = a1.x;
                                 o1[2 * q + 1] = a1.y;
                             }
-                            if (store) {
-                                store_vec<T, V>(out[0] + dst_off, o0);
-                                if constexpr (num_fields<MODEL>() == 2) store_vec<T, V>(out[NF - 1] + dst_off, o1);
-                            }
+                            put(0, o0);
+                            if constexpr (num_fields<MODEL>() == 2) put(NF - 1, o1);
                             dst_off += plane;
                         }
                     }
@@ -1801,8 +1892,8 @@ __device__ __forceinline__ void ring_stencil(const RowFn &row, const ExtFn &exte
 // round them, and every level evaluates the single-step expressions in the same
 // order, so K blocked steps equal K single steps bit for bit.
 //
-// Requirements (checked by the launcher): nx a multiple of 4 and 16-byte
-// aligned field pointers.
+// AL: nx is a multiple of 4 and the field pointers are 16-byte aligned; otherwise (FP32, one
+// step) rows go through RaggedRow.
 template <int MODEL, int ST, typename T, int TY, int K>
 struct Step3dTbsShape {
     static constexpr int V = 4;
@@ -1821,11 +1912,13 @@ struct Step3dTbsShape {
     static constexpr size_t lv_plane = (size_t)HIN * 32 * V * sizeof(float);
     static constexpr size_t in_bytes = (size_t)D0 * NF * in_plane;
     static constexpr size_t smem_bytes = in_bytes + (size_t)(K - 1) * DL * NF * lv_plane;
+    static constexpr size_t stage_bytes = (size_t)HIN * NF * 512;  // not AL: output rows
 };
 
-template <int MODEL, int ST, typename T, int TY, int K>
+template <int MODEL, int ST, typename T, int TY, int K, bool AL>
 __global__ void __launch_bounds__(Step3dTbsShape<MODEL, ST, T, TY, K>::NT)
     step3d_tbs_kernel(StepArgs a, int tiles_x, int tiles_y, int segs) {
+    pdl_enter();
     static_assert(MODEL == AC || MODEL == GS || MODEL == MC, "Allen-Cahn, Gray-Scott and Model C");
     typedef Step3dTbsShape<MODEL, ST, T, TY, K> Sh;
     constexpr int V = Sh::V, r = Sh::r, HIN = Sh::HIN, NF = Sh::NF, CB = Sh::CB, V2 = V / 2;
@@ -1845,6 +1938,8 @@ __global__ void __launch_bounds__(Step3dTbsShape<MODEL, ST, T, TY, K>::NT)
     // level rings [K-1][DL][NF][HIN][32][V] floats
     W *const in_own = reinterpret_cast<W *>(smem_raw) + (size_t)w * 32 + lane;
     float *const lv_own = reinterpret_cast<float *>(smem_raw + Sh::in_bytes) + ((size_t)w * 32 + lane) * V;
+    float *const stage = reinterpret_cast<float *>(smem_raw + Sh::smem_bytes) + (size_t)w * NF * 128;  // not AL
+    (void)stage;
     constexpr size_t IN_FLD = (size_t)HIN * 32, IN_SLOT = NF * IN_FLD;   // chunks
     constexpr size_t LV_FLD = (size_t)HIN * 32 * V, LV_SLOT = NF * LV_FLD, LV_LEVEL = DL * LV_SLOT;  // floats
     auto extend = [&](float *ext) {
@@ -1879,18 +1974,27 @@ __global__ void __launch_bounds__(Step3dTbsShape<MODEL, ST, T, TY, K>::NT)
         const int n = (z1 - z0) + 2 * K * r;
         const int niter = n + K - 1;
         const int col = x0 + (lane - 1) * V;
-        const size_t goff = (size_t)wrap_idx(y0 - K * r + w, ny) * nx + wrap_idx(col, nx);
+        const size_t goff = (size_t)wrap_idx(y0 - K * r + w, ny) * nx + (AL ? wrap_idx(col, nx) : 0);
         const int yo = y0 - K * r + w;
         const bool store = w >= K * r && w < HIN - K * r && lane >= 1 && lane <= 30 && col < nx && yo < ny;
+        const typename std::conditional<AL, NoRow, RaggedRow>::type rag(x0 - V, lane, nx);
         int jn = 0, zn = wrap_idx(z0 - K * r, nz);
         size_t src = (size_t)zn * plane + goff;
-        size_t dst_off = (size_t)z0 * plane + (size_t)yo * nx + col;
+        size_t dst_off = (size_t)z0 * plane + (size_t)yo * nx + (AL ? col : 0);
+        auto put = [&](int f, const float (&o)[V]) {
+            if constexpr (AL) {
+                if (store) store_vec<T, V>(out[f] + dst_off, o);
+            } else {
+                if (yo < ny) rag.put(out[f] + dst_off, stage + f * 128, o, nx);
+            }
+        };
         auto issue = [&]() {
             if (jn < n) {
                 W *dst = in_own + (size_t)(jn % D0) * IN_SLOT;
 #pragma unroll
                 for (int f = 0; f < NF; ++f) {
-                    if constexpr (CB == 16) cp_async16(dst + f * IN_FLD, in[f] + src);
+                    if constexpr (!AL) rag.fetch(reinterpret_cast<T *>(dst + f * IN_FLD - lane), in[f] + src);
+                    else if constexpr (CB == 16) cp_async16(dst + f * IN_FLD, in[f] + src);
                     else cp_async8(dst + f * IN_FLD, in[f] + src);
                 }
                 src += plane;
@@ -1961,10 +2065,8 @@ __global__ void __launch_bounds__(Step3dTbsShape<MODEL, ST, T, TY, K>::NT)
                                 make_float4(to_c(from_c<T>(res[f][0])), to_c(from_c<T>(res[f][1])),
                                             to_c(from_c<T>(res[f][2])), to_c(from_c<T>(res[f][3])));
                     } else {
-                        if (store) {
-                            store_vec<T, V>(out[0] + dst_off, res[0]);
-                            if constexpr (NF == 2) store_vec<T, V>(out[NF - 1] + dst_off, res[NF - 1]);
-                        }
+                        put(0, res[0]);
+                        if constexpr (NF == 2) put(NF - 1, res[NF - 1]);
                         dst_off += plane;
                     }
                 }
@@ -2081,6 +2183,7 @@ __device__ __forceinline__ void async_chunk_sums(const T *const (&pl)[2 * Stenci
 template <int MODEL, int ST, typename T, int TXT, int TY, bool TMA>
 __global__ void __launch_bounds__(TXT * TY) step3d_async_kernel(StepArgs a, int tiles_x, int tiles_y, int segs,
                                                                 const __grid_constant__ TmaMaps maps) {
+    pdl_enter();
     static_assert(MODEL != MC, "Model C runs on the accessor-based kernels");
     typedef Step3dAsyncShape<MODEL, ST, T, TXT, TY> Sh;
     typedef typename Sh::C C;
@@ -2354,6 +2457,7 @@ __device__ __forceinline__ void chunk_sums(const float *const (&pl)[2 * StencilI
 template <int MODEL, int ST, typename T, int TXT, int TYT>
 __global__ void __launch_bounds__(TXT * TYT) step3d_vec_kernel(StepArgs a, int tiles_x, int tiles_y,
                                                                long long planes_per_cta) {
+    pdl_enter();
     static_assert(MODEL != MC, "Model C runs on the accessor-based kernels");
     typedef Step3dVecShape<MODEL, ST, T, TXT, TYT> Sh;
     typedef typename Sh::C C;

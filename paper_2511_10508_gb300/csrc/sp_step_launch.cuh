@@ -30,8 +30,28 @@ inline bool small_tile(int nx, int ny, int TX, int TY, double margin) {
     return area(kTX64, kTY64) < margin * area(TX, TY);
 }
 
-constexpr int kMinRun = 32;  // 2D warp strips: rows per CTA at least
 constexpr size_t kMaxSmemPerCta = 227 * 1024;  // opt-in maximum of dynamic shared memory per CTA
+
+// Rows per CTA of the 2D warp-strip kernel, whose CTAs own equal runs of the flattened
+// (strip group, row) space: p rows cost p + halo, q CTAs of `load` (their share of 8
+// warps) on the fullest SM take about q load + latency of them (see planes_per_cta).
+// Runs of at least 32 rows left most SMs idle on small grids: 444 x 568 Cahn-Hilliard 9.2
+// us per step, 3.0 now; 1504 x 1000 4th order 13.2 -> 6.2 (runs of 8 rows; of 4: 7.5).
+inline long long rows_per_cta(long long total, int halo, double load, double latency, int occ, int n_sm) {
+    const long long wave = (long long)n_sm * std::max(occ, 1), p0 = (total + wave - 1) / wave;
+    long long best = p0;
+    double best_cost = 0;
+    for (long long p = p0; p <= std::min(total, 8 * p0 + 32); ++p) {
+        const long long ctas = (total + p - 1) / p, q = (ctas + n_sm - 1) / n_sm;
+        const double cost = (q * load + latency) * (p + halo);
+        if (p == p0 || cost < best_cost * 0.999) {
+            best = p;
+            best_cost = cost;
+        }
+        if (q == 1) break;
+    }
+    return best;
+}
 
 // Planes per CTA of a persistent 3D kernel whose CTAs own equal contiguous runs of
 // the flattened (tile, z) space; at most one resident wave (n_sm x occ CTAs).  A run
@@ -82,8 +102,7 @@ cudaError_t launch_strips(const StepArgs &a, cudaStream_t s, int n_sm) {
     ctas = std::max(1LL, std::min(ctas, total / (4 * RB)));
     const long long rows = (total + ctas - 1) / ctas;
     ctas = (total + rows - 1) / rows;
-    kern<<<(unsigned)ctas, NT, Sh::smem_bytes, s>>>(a, strips, rows);
-    return cudaGetLastError();
+    return launch_pdl(kern, dim3((unsigned)ctas), dim3(NT), Sh::smem_bytes, s, a, strips, rows);
 }
 
 // Temporally blocked 2D tile kernel: K steps per launch.  FP32 / BF16 tiles of
@@ -101,31 +120,48 @@ cudaError_t launch_tb(const StepArgs &a, cudaStream_t s) {
     }();
     (void)attr;
     dim3 grid((a.nx + BX - 1) / BX, (a.ny + BY - 1) / BY);
-    if constexpr (f64) return launch_pdl(kern, grid, dim3(NT), Sh::smem_bytes, s, a);  // small grids
-    kern<<<grid, NT, Sh::smem_bytes, s>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(kern, grid, dim3(NT), Sh::smem_bytes, s, a);
 }
 
 // 3D FP32 / BF16 Allen-Cahn and Gray-Scott with a plane ring per time level: K
 // steps per pass (temporal blocking for K = 2) on warp-row tiles of 120 x TY
 // outputs; lockstep z segments.  Needs nx a multiple of 4 and 16-byte aligned
 // fields (the runtime offers these families only then).
-template <int MODEL, int ST, typename T, int TY, int K>
+template <int MODEL, int ST, typename T, int TY, int K, bool AL>
 cudaError_t launch_tbs(const StepArgs &a, cudaStream_t s, int n_sm) {
     typedef Step3dTbsShape<MODEL, ST, T, TY, K> Sh;
-    auto kern = step3d_tbs_kernel<MODEL, ST, T, TY, K>;
+    constexpr size_t smem = Sh::smem_bytes + (AL ? 0 : Sh::stage_bytes);
+    auto kern = step3d_tbs_kernel<MODEL, ST, T, TY, K, AL>;
     static const int occ = [&] {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::smem_bytes);
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         int o = 1;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, Sh::NT, Sh::smem_bytes);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, Sh::NT, smem);
         return o;
     }();
     const int tx = (a.nx + Sh::TX - 1) / Sh::TX, ty = (a.ny + TY - 1) / TY;
     const long long wave = (long long)n_sm * std::max(occ, 1);
     const int segs = lockstep_segments((long long)tx * ty, a.nz, 2 * K * Sh::r, wave);
     const long long items = (long long)tx * ty * segs;
-    kern<<<(unsigned)std::min(items, wave), Sh::NT, Sh::smem_bytes, s>>>(a, tx, ty, segs);
-    return cudaGetLastError();
+    return launch_pdl(kern, dim3((unsigned)std::min(items, wave)), dim3(Sh::NT), smem, s, a, tx, ty, segs);
+}
+
+// 3D FP32 / BF16, warp per tile row with z neighbours in registers.
+template <int MODEL, int ST, typename T, int TY, bool AL>
+cudaError_t launch_wr(const StepArgs &a, cudaStream_t s, int n_sm) {
+    typedef Step3dWrShape<MODEL, ST, T, TY> Sh;
+    constexpr size_t smem = Sh::smem_bytes + (AL ? 0 : Sh::stage_bytes);
+    auto kern = step3d_wr_kernel<MODEL, ST, T, TY, AL>;
+    static const int occ = [&] {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        int o = 1;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, Sh::NT, smem);
+        return o;
+    }();
+    const int tx = (a.nx + Sh::TX - 1) / Sh::TX, ty = (a.ny + TY - 1) / TY;
+    const long long wave = (long long)n_sm * std::max(occ, 1);
+    const int segs = lockstep_segments((long long)tx * ty, a.nz, 2 * Sh::R, wave);
+    const long long items = (long long)tx * ty * segs;
+    return launch_pdl(kern, dim3((unsigned)std::min(items, wave)), dim3(Sh::NT), smem, s, a, tx, ty, segs);
 }
 
 // FP64 27-point: z-streaming kernel with per-plane partial sums in registers.
@@ -142,8 +178,7 @@ cudaError_t launch_zreg(const StepArgs &a, cudaStream_t s, int n_sm) {
     }();
     const int tx = (a.nx + TX - 1) / TX, ty = (a.ny + TY - 1) / TY;
     const long long planes = planes_per_cta((long long)tx * ty, a.nz, 1.0, occ, n_sm);
-    kern<<<(unsigned)(((long long)tx * ty * a.nz + planes - 1) / planes), NT, Sh::smem_bytes, s>>>(a, tx, ty, planes);
-    return cudaGetLastError();
+    return launch_pdl(kern, dim3((unsigned)(((long long)tx * ty * a.nz + planes - 1) / planes)), dim3(NT), Sh::smem_bytes, s, a, tx, ty, planes);
 }
 
 // FP64 27-point with shared pair sums: one pass per mode (Cahn-Hilliard: mode 0
@@ -161,8 +196,7 @@ cudaError_t launch_planes27_mode(const Planes27Args &a, cudaStream_t s, int n_sm
     const int tx = (a.nx + Sh::TX - 1) / Sh::TX, ty = (a.ny + Sh::TY - 1) / Sh::TY;
     const long long total = (long long)tx * ty * a.nz;
     const long long planes = planes_per_cta((long long)tx * ty, a.nz, 1.0, occ, n_sm);
-    kern<<<(unsigned)((total + planes - 1) / planes), Sh::NT, Sh::smem_bytes, s>>>(a, tx, planes, total);
-    return cudaGetLastError();
+    return launch_pdl(kern, dim3((unsigned)((total + planes - 1) / planes)), dim3(Sh::NT), Sh::smem_bytes, s, a, tx, planes, total);
 }
 template <int ST, int MODE, int TY>
 cudaError_t launch_ring2pass_tile(const Planes27Args &a, cudaStream_t s, int n_sm) {
@@ -177,8 +211,7 @@ cudaError_t launch_ring2pass_tile(const Planes27Args &a, cudaStream_t s, int n_s
     const int tx = (a.nx + Sh::TX - 1) / Sh::TX, ty = (a.ny + Sh::TY - 1) / Sh::TY;
     const long long total = (long long)tx * ty * a.nz;
     const long long planes = planes_per_cta((long long)tx * ty, a.nz, 0.7 * Sh::R, occ, n_sm);
-    kern<<<(unsigned)((total + planes - 1) / planes), Sh::NT, Sh::smem_bytes, s>>>(a, tx, planes, total);
-    return cudaGetLastError();
+    return launch_pdl(kern, dim3((unsigned)((total + planes - 1) / planes)), dim3(Sh::NT), Sh::smem_bytes, s, a, tx, planes, total);
 }
 template <int ST, int MODE>
 cudaError_t launch_ring2pass_mode(const Planes27Args &a, cudaStream_t s, int n_sm) {
@@ -199,8 +232,31 @@ cudaError_t launch_step3d_tile(const StepArgs &a, cudaStream_t s, int n_sm) {
     }();
     const int tx = (a.nx + TX - 1) / TX, ty = (a.ny + TY - 1) / TY;
     const long long planes = planes_per_cta((long long)tx * ty, a.nz, 0.7 * Sh::RIN, occ, n_sm);
-    kern<<<(unsigned)(((long long)tx * ty * a.nz + planes - 1) / planes), NT, Sh::smem_bytes, s>>>(a, tx, ty, planes);
-    return cudaGetLastError();
+    return launch_pdl(kern, dim3((unsigned)(((long long)tx * ty * a.nz + planes - 1) / planes)), dim3(NT), Sh::smem_bytes, s, a, tx, ty, planes);
+}
+
+// FP32 / BF16 2D: one warp per column strip, up to 8 adjacent strips per CTA,
+// persistent equal shares of (strip group, row).
+template <int MODEL, int ST, typename T, bool AL>
+cudaError_t launch_warp2d(const StepArgs &a, cudaStream_t s, int n_sm) {
+    typedef Step2dWarpShape<MODEL, ST, T> WS;
+    constexpr int NT = 256;
+    auto kern = step2d_warp_kernel<MODEL, ST, T, NT, AL>;
+    static const bool attr = [&] {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(WS::warp_smem(AL) * (NT / 32)));
+        return true;
+    }();
+    (void)attr;
+    const int strips = (a.nx + WS::OUT_COLS - 1) / WS::OUT_COLS;
+    const int wpc = std::min(NT / 32, strips);
+    const size_t smem = WS::warp_smem(AL) * wpc;
+    int occ = 1;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 32 * wpc, smem);
+    const int groups = (strips + wpc - 1) / wpc;
+    const long long total = (long long)groups * a.ny;
+    const long long rows = rows_per_cta(total, 2 * WS::RIN, wpc / 8.0, AL ? 1.0 : 4.0, occ, n_sm);
+    const long long ctas = (total + rows - 1) / rows;
+    return launch_pdl(kern, dim3((unsigned)ctas), dim3(32 * wpc), smem, s, a, strips, groups, rows);
 }
 
 template <int MODEL, int ST, typename T>
@@ -234,30 +290,11 @@ cudaError_t launch_step_t(const StepArgs &a, cudaStream_t s, int n_sm, int k) {
     } else if constexpr (StencilInfo<ST>::dims == 2) {
         typedef Step2dWarpShape<MODEL, ST, T> WS;
         const bool aligned = ((uintptr_t)a.in0 | (uintptr_t)a.in1 | (uintptr_t)a.out0 | (uintptr_t)a.out1) % 16 == 0;
-        if (g_step_variant == 0 && a.nx % WS::V == 0 && aligned) {
-            // FP32 / BF16: one warp per column strip, up to 8 adjacent strips per
-            // CTA, persistent equal shares of (strip group, row)
-            constexpr int NT = 256;
-            auto kern = step2d_warp_kernel<MODEL, ST, T, NT>;
-            static const bool attr = [&] {
-                cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(WS::warp_smem * (NT / 32)));
-                return true;
-            }();
-            (void)attr;
-            const int strips = (a.nx + WS::OUT_COLS - 1) / WS::OUT_COLS;
-            const int wpc = std::min(NT / 32, strips);
-            const size_t smem = WS::warp_smem * wpc;
-            int occ = 1;
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 32 * wpc, smem);
-            const int groups = (strips + wpc - 1) / wpc;
-            const long long total = (long long)groups * a.ny;
-            long long ctas = (long long)n_sm * std::max(occ, 1);
-            ctas = std::max(1LL, std::min(ctas, total / kMinRun));
-            const long long rows = (total + ctas - 1) / ctas;
-            ctas = (total + rows - 1) / rows;
-            kern<<<(unsigned)ctas, 32 * wpc, smem, s>>>(a, strips, groups, rows);
-            return cudaGetLastError();
+        // (16-bit storage has no element-wise asynchronous copy)
+        const bool al = a.nx % WS::V == 0 && aligned;
+        if (g_step_variant == 0 && al) return launch_warp2d<MODEL, ST, T, true>(a, s, n_sm);
+        if constexpr (sizeof(T) == 4) {
+            if (g_step_variant == 0) return launch_warp2d<MODEL, ST, T, false>(a, s, n_sm);
         }
         // FP32 / BF16: one CTA per 128 x 32 tile
         constexpr int BX = 128, BY = 32, NT = 256;
@@ -269,18 +306,21 @@ cudaError_t launch_step_t(const StepArgs &a, cudaStream_t s, int n_sm, int k) {
         }();
         (void)attr;
         dim3 grid((a.nx + BX - 1) / BX, (a.ny + BY - 1) / BY);
-        kern<<<grid, NT, Sh::smem_bytes, s>>>(a);
+        return launch_pdl(kern, grid, dim3(NT), Sh::smem_bytes, s, a);
     } else if constexpr (!std::is_same<T, double>::value && MODEL == MC) {
         // Model C, FP32 / BF16 3D: plane rings (two steps per launch: families 0 and 1,
-        // tiles of 8 and 16 rows; one step: families 4 and 5) where nx and the
-        // alignment allow, else one CTA per box (the accessor-based box code)
-        const bool al = ((uintptr_t)a.in0 | (uintptr_t)a.in1 | (uintptr_t)a.out0 | (uintptr_t)a.out1) % 16 == 0;
-        if (a.nx % 4 == 0 && al) {
+        // tiles of 8 and 16 rows; one step: families 0 and 4, 5); one CTA per box
+        // (families 1 and 2, and 16-bit storage with unaligned rows)
+        const bool al = a.nx % 4 == 0 &&
+                        ((uintptr_t)a.in0 | (uintptr_t)a.in1 | (uintptr_t)a.out0 | (uintptr_t)a.out1) % 16 == 0;
+        if (al) {
             constexpr bool tall2 = Step3dTbsShape<MODEL, ST, T, 16, 2>::smem_bytes <= kMaxSmemPerCta;
-            if (k == 2 && g_step_variant == 1 && tall2) return launch_tbs<MODEL, ST, T, (tall2 ? 16 : 8), 2>(a, s, n_sm);
-            if (k == 2) return launch_tbs<MODEL, ST, T, 8, 2>(a, s, n_sm);
-            if (g_step_variant == 5) return launch_tbs<MODEL, ST, T, 16, 1>(a, s, n_sm);
-            if (g_step_variant == 4) return launch_tbs<MODEL, ST, T, 8, 1>(a, s, n_sm);
+            if (k == 2 && g_step_variant == 1 && tall2) return launch_tbs<MODEL, ST, T, (tall2 ? 16 : 8), 2, true>(a, s, n_sm);
+            if (k == 2) return launch_tbs<MODEL, ST, T, 8, 2, true>(a, s, n_sm);
+            if (g_step_variant == 5) return launch_tbs<MODEL, ST, T, 16, 1, true>(a, s, n_sm);
+            if (g_step_variant == 4 || g_step_variant == 0) return launch_tbs<MODEL, ST, T, 8, 1, true>(a, s, n_sm);
+        } else if constexpr (sizeof(T) == 4) {
+            if (g_step_variant == 0) return launch_tbs<MODEL, ST, T, 8, 1, false>(a, s, n_sm);
         }
         constexpr int BX = 32, BY = 8, BZ = 8, NT = 256;
         typedef Step3dBoxShape<MODEL, ST, T, BX, BY, BZ> Sh;
@@ -291,21 +331,21 @@ cudaError_t launch_step_t(const StepArgs &a, cudaStream_t s, int n_sm, int k) {
         }();
         (void)attr;
         const int bx = (a.nx + BX - 1) / BX, by = (a.ny + BY - 1) / BY, bz = (a.nz + BZ - 1) / BZ;
-        kern<<<dim3((unsigned)bx, (unsigned)by, (unsigned)bz), NT, Sh::smem_bytes, s>>>(a);
+        return launch_pdl(kern, dim3((unsigned)bx, (unsigned)by, (unsigned)bz), dim3(NT), Sh::smem_bytes, s, a);
     } else if constexpr (!std::is_same<T, double>::value) {
         if constexpr (MODEL == AC || MODEL == GS) {
             // two steps per launch with a plane ring per time level (families 0 and 1:
             // tiles of 8 and 16 rows; the taller ones only where their rings fit)
             constexpr bool tall2 = Step3dTbsShape<MODEL, ST, T, 16, 2>::smem_bytes <= kMaxSmemPerCta;
-            if (k == 2 && g_step_variant == 1 && tall2) return launch_tbs<MODEL, ST, T, (tall2 ? 16 : 8), 2>(a, s, n_sm);
-            if (k == 2) return launch_tbs<MODEL, ST, T, 8, 2>(a, s, n_sm);
+            if (k == 2 && g_step_variant == 1 && tall2) return launch_tbs<MODEL, ST, T, (tall2 ? 16 : 8), 2, true>(a, s, n_sm);
+            if (k == 2) return launch_tbs<MODEL, ST, T, 8, 2, true>(a, s, n_sm);
         }
         constexpr int ATX = 16, ATY = 16;
         typedef Step3dAsyncShape<MODEL, ST, T, ATX, ATY> AS;
         const bool aligned = ((uintptr_t)a.in0 | (uintptr_t)a.in1 | (uintptr_t)a.out0 | (uintptr_t)a.out1) % 16 == 0;
         constexpr int WTY = 8;
         typedef Step3dWrShape<MODEL, ST, T, WTY> WS;
-        auto wkern = step3d_wr_kernel<MODEL, ST, T, WTY>;
+        auto wkern = step3d_wr_kernel<MODEL, ST, T, WTY, true>;
         // the warp-row kernel is the default unless its register queues spill
         // (a spill of a few words outside the queues costs nothing measurable)
         static const bool wr_spills = [&] {
@@ -313,21 +353,14 @@ cudaError_t launch_step_t(const StepArgs &a, cudaStream_t s, int n_sm, int k) {
             return cudaFuncGetAttributes(&fa, wkern) != cudaSuccess || fa.localSizeBytes > 16;
         }();
         const int fam = (g_step_variant == 0 && wr_spills) ? 1 : g_step_variant;
-        if (fam == 0 && a.nx % WS::V == 0 && aligned) {
-            // FP32 / BF16 3D: warp per tile row, z neighbours in registers
-            auto kern = wkern;
-            static const int occ = [&] {
-                cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WS::smem_bytes);
-                int o = 1;
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, WS::NT, WS::smem_bytes);
-                return o;
-            }();
-            const int tx = (a.nx + WS::TX - 1) / WS::TX, ty = (a.ny + WTY - 1) / WTY;
-            const long long wave = (long long)n_sm * std::max(occ, 1);
-            const int segs = lockstep_segments((long long)tx * ty, a.nz, 2 * WS::R, wave);
-            const long long items = (long long)tx * ty * segs;
-            kern<<<(unsigned)std::min(items, wave), WS::NT, WS::smem_bytes, s>>>(a, tx, ty, segs);
-            return cudaGetLastError();
+        if (fam == 0 && a.nx % WS::V == 0 && aligned) return launch_wr<MODEL, ST, T, WTY, true>(a, s, n_sm);
+        if constexpr (sizeof(T) == 4) {
+            // unaligned rows: the same kernel, or the plane ring for Gray-Scott, whose two
+            // fields' queues spill
+            if (g_step_variant == 0 && !(a.nx % WS::V == 0 && aligned)) {
+                if constexpr (MODEL == GS) return launch_tbs<MODEL, ST, T, 8, 1, false>(a, s, n_sm);
+                else return launch_wr<MODEL, ST, T, WTY, false>(a, s, n_sm);
+            }
         }
         if (fam == kTmaFamily && a.nx % AS::V == 0 && aligned) {
             // FP32 / BF16 3D: the plane ring with tensor-map plane loads
@@ -346,8 +379,7 @@ cudaError_t launch_step_t(const StepArgs &a, cudaStream_t s, int n_sm, int k) {
             const long long wave = (long long)n_sm * std::max(occ, 1);
             const int segs = lockstep_segments((long long)tx * ty, a.nz, 2 * AS::R, wave);
             const long long items = (long long)tx * ty * segs;
-            kern<<<(unsigned)std::min(items, wave), AS::NT, AS::smem_bytes, s>>>(a, tx, ty, segs, maps);
-            return cudaGetLastError();
+            return launch_pdl(kern, dim3((unsigned)std::min(items, wave)), dim3(AS::NT), AS::smem_bytes, s, a, tx, ty, segs, maps);
         }
         if (fam != 2 && a.nx % AS::V == 0 && aligned) {
             // FP32 / BF16 3D: cp.async plane ring with planes in flight
@@ -362,8 +394,7 @@ cudaError_t launch_step_t(const StepArgs &a, cudaStream_t s, int n_sm, int k) {
             const long long wave = (long long)n_sm * std::max(occ, 1);
             const int segs = lockstep_segments((long long)tx * ty, a.nz, 2 * AS::R, wave);
             const long long items = (long long)tx * ty * segs;
-            kern<<<(unsigned)std::min(items, wave), AS::NT, AS::smem_bytes, s>>>(a, tx, ty, segs, TmaMaps{});
-            return cudaGetLastError();
+            return launch_pdl(kern, dim3((unsigned)std::min(items, wave)), dim3(AS::NT), AS::smem_bytes, s, a, tx, ty, segs, TmaMaps{});
         }
         // FP32 / BF16 3D, any nx: vectorised plane kernel, 64 x 32 tiles
         constexpr int TXT = 16, TYT = 32;
@@ -377,8 +408,7 @@ cudaError_t launch_step_t(const StepArgs &a, cudaStream_t s, int n_sm, int k) {
         }();
         const int tx = (a.nx + Sh::TX - 1) / Sh::TX, ty = (a.ny + Sh::TY - 1) / Sh::TY;
         const long long planes = planes_per_cta((long long)tx * ty, a.nz, Sh::R, occ, n_sm);
-        kern<<<(unsigned)(((long long)tx * ty * a.nz + planes - 1) / planes), Sh::NT, Sh::smem_bytes, s>>>(
-            a, tx, ty, planes);
+        return launch_pdl(kern, dim3((unsigned)(((long long)tx * ty * a.nz + planes - 1) / planes)), dim3(Sh::NT), Sh::smem_bytes, s, a, tx, ty, planes);
     } else {
         if constexpr (MODEL != MC) {
             if (ST == L27 && g_step_variant == 0) return launch_zreg<MODEL, T>(a, s, n_sm);

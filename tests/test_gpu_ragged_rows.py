@@ -1,0 +1,56 @@
+"""FP32 kernels on grids whose rows are not 16-byte aligned (nx odd, or 2 mod 4), and the row
+and plane splits of small grids: rows shorter than a warp's 120 outputs, just above them,
+and several strips; every model and stencil.  Families evaluate the same expressions in
+the same order, so the default must equal the tile / staged family bit for bit, and fused
+steps single ones."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sp():
+    import __graft_entry__
+
+    __graft_entry__._load_builder().build()
+    import paper_2511_10508_gb300 as sp
+
+    return sp
+
+
+def run(sp, model, shape, st, dtype, cfg, steps=7):
+    kw = dict(seed=9, ic_amp=0.3)
+    if model == 2:
+        kw = dict(seed=9, ic_amp=0.01, gs_patches=3, gs_patch=min(3, *shape))
+    with sp.Simulation(model, shape, dt=0.001, stencil=st, dtype=dtype, **kw) as s:
+        if cfg:
+            s.launch_config = cfg
+        s.step(steps)
+        return [s.read(f) for f in range(s.nfields)]
+
+
+@pytest.mark.parametrize("st", [0, 1, 2])
+@pytest.mark.parametrize("model", [0, 1, 2, 3])
+@pytest.mark.parametrize("shape", [(1, 1), (3, 5), (40, 7), (9, 121), (70, 123), (33, 250), (5, 963), (64, 120), (300, 4)])
+def test_2d_rows(sp, model, st, shape):
+    a = run(sp, model, shape, st, 1, (1, 0))
+    for cfg in ((1, 1), (2, 0), None):
+        for x, y in zip(a, run(sp, model, shape, st, 1, cfg)):
+            assert np.array_equal(x, y), cfg
+
+
+@pytest.mark.parametrize("st", [3, 4, 5])
+@pytest.mark.parametrize("model", [0, 1, 2, 3])
+@pytest.mark.parametrize("shape", [(1, 1, 1), (2, 3, 5), (9, 10, 121), (5, 17, 130), (40, 9, 7), (6, 33, 245), (7, 8, 120)])
+def test_3d_rows(sp, model, st, shape):
+    a = run(sp, model, shape, st, 1, None)
+    for x, y in zip(a, run(sp, model, shape, st, 1, (1, 2))):  # staged planes (Model C: boxes)
+        assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("model", [0, 1, 2, 3])
+@pytest.mark.parametrize("shape", [(64, 64), (257, 257), (256, 256), (80, 856), (411, 411), (31, 33)])
+def test_2d_fp64_default_equals_single_steps(sp, model, shape):
+    for x, y in zip(run(sp, model, shape, 0, 0, None), run(sp, model, shape, 0, 0, (1, 0))):
+        assert np.array_equal(x, y)
