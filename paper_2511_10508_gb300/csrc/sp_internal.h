@@ -51,6 +51,16 @@ cudaError_t launch_step_bf16(int model, int stencil, const StepArgs &a, cudaStre
 // the runtime.
 extern thread_local int g_step_variant;
 
+// 3D FP32 warp-row kernel, any alignment (sp_wr.cuh, one translation unit per model);
+// cudaErrorNotSupported where the plane ring is the cheaper one.
+cudaError_t launch_wr_ac(int stencil, const StepArgs &a, cudaStream_t s, int n_sm);
+cudaError_t launch_wr_ch(int stencil, const StepArgs &a, cudaStream_t s, int n_sm);
+cudaError_t launch_wr_gs(int stencil, const StepArgs &a, cudaStream_t s, int n_sm);
+inline cudaError_t launch_wr_f32(int model, int stencil, const StepArgs &a, cudaStream_t s, int n_sm) {
+    return model == AC ? launch_wr_ac(stencil, a, s, n_sm)
+           : model == CH ? launch_wr_ch(stencil, a, s, n_sm) : launch_wr_gs(stencil, a, s, n_sm);
+}
+
 // Number of equal z segments for a lockstep schedule of `tiles` x segments work
 // items over `wave` resident CTAs: minimises rounds x (planes per segment +
 // halo planes), the time of the slowest CTA.

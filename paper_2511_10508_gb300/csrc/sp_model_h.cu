@@ -21,6 +21,7 @@
 #include <type_traits>
 
 #include "sp_internal.h"
+#include "sp_step.cuh"
 
 namespace sp {
 
@@ -348,6 +349,200 @@ __global__ void __launch_bounds__(NT) mh_ring3d_kernel(MhArgs a, float c3g, int 
     }
 }
 
+// 3D FP32 / BF16, radius-1 stencils: rows of LN = 32 lanes or, two per warp, 16.  A row of a
+// tile of 4 (LN - 2) x TY outputs (TY + 4 rows with the 2-cell halo) has the cells 4 l .. 4 l + 3 in
+// lane l (the first and the last lane are halo), so every
+// shared-memory access is a 16-byte chunk and the x neighbours come from the adjacent
+// lanes (ring_stencil).  Planes stream along z through cp.async rings: m needs 3R + 2
+// planes, the components of j, whose loads trail by R + 1 planes, 2R + 1, each plus P in
+// flight; mu of plane j - R goes to a ring of 2R + 2 planes, the update runs one plane
+// behind it, so one barrier per plane suffices.  The same expressions as the per-point
+// kernels, so the results are identical.  (z segment, tile) items segment-major, as in
+// mh_ring3d_kernel, which reads ~50 scalar shared-memory values per point and was bound by
+// them: 256^3 7-point 195 us per step, 166 now; 27-point 413 -> 271.  One CTA of 448 threads fits
+// an SM beside the rings, so latency between barriers bounds it now.  The radius-2 rings
+// would not fit beside a useful tile; those stencils keep it.
+// AL: nx a multiple of 4 and 16-byte aligned fields; otherwise (FP32) RaggedRow.
+template <int ST, typename T, int TY, int LN_>
+struct MhRows3dShape {
+    static constexpr int R = StencilInfo<ST>::r, V = 4, CB = V * (int)sizeof(T), LN = LN_;
+    static_assert(R == 1, "radius-2 rings do not fit");
+    static constexpr int TX = (LN - 2) * V, HIN = TY + 4 * R, NT = LN * HIN;
+    static_assert(NT % 32 == 0 && R % 2 == 1, "whole warps; the output rows of a warp are both or none");
+    static constexpr int P = 2, DM = 3 * R + 2 + P, DJ = 2 * R + 1 + P, DMU = 2 * R + 2;
+    static constexpr size_t plane_bytes = (size_t)HIN * LN * CB, mu_plane = (size_t)HIN * LN * V;
+    static constexpr size_t in_bytes = (DM + 3 * DJ) * plane_bytes;
+    static constexpr size_t smem_bytes = in_bytes + DMU * mu_plane * sizeof(float);
+    static constexpr size_t stage_bytes = (size_t)HIN * LN * 16;  // not AL: an output row per row
+};
+
+template <int ST, typename T, int TY, int LN, bool AL>
+__global__ void __launch_bounds__(MhRows3dShape<ST, T, TY, LN>::NT)
+    mh_rows3d_kernel(MhArgs a, float c3g, int tiles_x, int tiles_y, int segs) {
+    pdl_enter();
+    typedef MhRows3dShape<ST, T, TY, LN> Sh;
+    constexpr int R = Sh::R, V = Sh::V, CB = Sh::CB, HIN = Sh::HIN, P = Sh::P;
+    constexpr unsigned FULL = 0xffffffffu;
+    typedef typename VecT<CB>::type W;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const ConstsC<float> k(a.k, a.kf);
+    const int nx = a.nx, ny = a.ny, nz = a.nz;
+    const int lane = threadIdx.x & (LN - 1), w = threadIdx.x / LN;
+    const size_t plane = (size_t)nx * (size_t)ny;
+    constexpr size_t PL = (size_t)HIN * LN;  // chunks of a plane
+    W *const m_own = reinterpret_cast<W *>(smem_raw) + (size_t)w * LN + lane;
+    W *const j_own = m_own + Sh::DM * PL;    // [3][DJ] planes
+    float *const mu_own = reinterpret_cast<float *>(smem_raw + Sh::in_bytes) + ((size_t)w * LN + lane) * V;
+    float *const stage = reinterpret_cast<float *>(smem_raw + Sh::smem_bytes) + w * LN * V;  // not AL
+    (void)stage;
+    const T *in[4] = {static_cast<const T *>(a.m), static_cast<const T *>(a.j[0]), static_cast<const T *>(a.j[1]),
+                      static_cast<const T *>(a.j[2])};
+    T *out[4] = {static_cast<T *>(a.mo), static_cast<T *>(a.jo[0]), static_cast<T *>(a.jo[1]), static_cast<T *>(a.jo[2])};
+    auto extend = [&](float *e) {
+        e[0] = __shfl_up_sync(FULL, e[V], 1, LN);
+        e[V + 1] = __shfl_down_sync(FULL, e[1], 1, LN);
+    };
+    auto widen = [&](const W *p, float *dst) {
+        union { W c; T t[V]; } u;
+        u.c = *p;
+#pragma unroll
+        for (int i = 0; i < V; ++i) dst[i] = to_c(u.t[i]);
+    };
+    // chunks of m, component f of j and mu: plane q, row offset dy
+    auto m_at = [&](int q, int dy, float *dst) { widen(m_own + (q % Sh::DM) * PL + dy * LN, dst); };
+    auto j_at = [&](int f, int q, int dy, float *dst) { widen(j_own + (f * Sh::DJ + q % Sh::DJ) * PL + dy * LN, dst); };
+    auto mu_at = [&](int q, int dy, float *dst) {
+        const float4 v = *reinterpret_cast<const float4 *>(mu_own + (q % Sh::DMU) * Sh::mu_plane + dy * LN * V);
+        dst[0] = v.x, dst[1] = v.y, dst[2] = v.z, dst[3] = v.w;
+    };
+    const bool out_row = w >= 2 * R && w < HIN - 2 * R;  // the same for both rows of a warp
+    // mu is formed by whole warps: the outermost rows, which need none, repeat their neighbour's
+    const int mu_dy = w < R ? R - w : w >= HIN - R ? HIN - 1 - R - w : 0;
+
+    const int tiles = tiles_x * tiles_y;
+    for (long long it = blockIdx.x; it < (long long)tiles * segs; it += gridDim.x) {
+        const int seg = (int)(it / tiles), tile = (int)(it - (long long)seg * tiles);
+        const int z0 = (int)((long long)seg * nz / segs), z1 = (int)((long long)(seg + 1) * nz / segs);
+        const int x0 = (tile % tiles_x) * Sh::TX, y0 = (tile / tiles_x) * TY;
+        const int n = (z1 - z0) + 4 * R;  // loaded plane i is z = z0 - 2R + i
+        const int col = x0 + (lane - 1) * V, yo = y0 - 2 * R + w;
+        const size_t roff = (size_t)wrap_idx(yo, ny) * nx + (AL ? wrap_idx(col, nx) : 0);
+        const bool store = out_row && lane >= 1 && lane <= LN - 2 && col < nx && yo < ny;
+        const typename std::conditional<AL, NoRow, RaggedRow<LN>>::type rag(x0 - V, lane, nx);
+        size_t dst_off = (size_t)z0 * plane + (size_t)yo * nx + (AL ? col : 0);
+        auto put = [&](int f, const float (&o)[V]) {
+            if constexpr (AL) {
+                if (store) store_vec<T, V>(out[f] + dst_off, o);
+            } else {
+                rag.put(out[f] + dst_off, stage, o, nx, yo < ny);
+            }
+        };
+        auto fetch = [&](W *dst, const T *field, int i) {
+            const T *src = field + (size_t)wrap_idx(z0 - 2 * R + i, nz) * plane + roff;
+            if constexpr (!AL) rag.fetch(reinterpret_cast<T *>(dst - lane), src);
+            else if constexpr (CB == 16) cp_async16(dst, src);
+            else cp_async8(dst, src);
+        };
+        // group g: plane g of m, plane g - 1 - R of j (planes R .. n-1-R are read)
+        auto issue = [&](int g) {
+            if (g < n) fetch(m_own + (g % Sh::DM) * PL, in[0], g);
+            const int i = g - 1 - R;
+            if (i >= R && i < n - R)
+#pragma unroll
+                for (int f = 0; f < 3; ++f) fetch(j_own + (f * Sh::DJ + i % Sh::DJ) * PL, in[1 + f], i);
+            cp_async_commit();
+        };
+#pragma unroll
+        for (int g = 0; g < P; ++g) issue(g);
+        for (int j = 0; j <= n; ++j) {
+            cp_async_wait<P - 1>();
+            __syncthreads();  // group j and mu of plane j-1-R published; slots written below are no longer read
+            issue(j + P);
+            const int t = j - 1 - 2 * R;  // output plane
+            if (out_row && t >= 2 * R) {
+                float S[V], cen[V], mu_e[V + 2], up[V], dn[V];
+                float mc[V], o[V], div[V];
+                m_at(t, 0, mc);
+                {   // D_x(m j_x) + D_y(m j_y) + D_z(m j_z), the product formed at every tap
+                    float e[V + 2], q[V];
+                    j_at(0, t, 0, q);
+#pragma unroll
+                    for (int c = 0; c < V; ++c) e[1 + c] = mc[c] * q[c];
+                    extend(e);
+#pragma unroll
+                    for (int c = 0; c < V; ++c) div[c] = e[c + 2] - e[c];
+                    float ma[V], mb[V];
+                    m_at(t, 1, ma), j_at(1, t, 1, up), m_at(t, -1, mb), j_at(1, t, -1, dn);
+#pragma unroll
+                    for (int c = 0; c < V; ++c) div[c] = div[c] + (ma[c] * up[c] - mb[c] * dn[c]);
+                    m_at(t + 1, 0, ma), j_at(2, t + 1, 0, up), m_at(t - 1, 0, mb), j_at(2, t - 1, 0, dn);
+#pragma unroll
+                    for (int c = 0; c < V; ++c) div[c] = div[c] + (ma[c] * up[c] - mb[c] * dn[c]);
+                }
+                ring_stencil<ST>([&](int dz, int dy, float *d) { mu_at(t + dz, dy, d); }, extend, S, cen);
+#pragma unroll
+                for (int c = 0; c < V; ++c) o[c] = FMA(k.dt, FMA(k.sAC, S[c], -(c3g * div[c])), mc[c]);
+                put(0, o);
+#pragma unroll
+                for (int c = 0; c < V; ++c) mu_e[1 + c] = cen[c];
+                extend(mu_e);
+#pragma unroll
+                for (int f = 0; f < 3; ++f) {
+                    if (f == 1) mu_at(t, 1, up), mu_at(t, -1, dn);
+                    if (f == 2) mu_at(t + 1, 0, up), mu_at(t - 1, 0, dn);
+                    ring_stencil<ST>([&](int dz, int dy, float *d) { j_at(f, t + dz, dy, d); }, extend, S, cen);
+#pragma unroll
+                    for (int c = 0; c < V; ++c) {
+                        const float g = f == 0 ? mu_e[c + 2] - mu_e[c] : up[c] - dn[c];
+                        o[c] = FMA(k.dt, FMA(k.sAC, S[c], -(c3g * (mc[c] * g))), cen[c]);
+                    }
+                    put(1 + f, o);
+                }
+                dst_off += plane;
+            }
+            if (j >= 2 * R && j < n) {  // mu of plane j - R
+                float S[V], cen[V];
+                ring_stencil<ST>([&](int dz, int dy, float *d) { m_at(j - R + dz, mu_dy + dy, d); }, extend, S, cen);
+                *reinterpret_cast<float4 *>(mu_own + ((j - R) % Sh::DMU) * Sh::mu_plane) =
+                    make_float4(ch_mu<float>(cen[0], S[0], k), ch_mu<float>(cen[1], S[1], k),
+                                ch_mu<float>(cen[2], S[2], k), ch_mu<float>(cen[3], S[3], k));
+            }
+        }
+        cp_async_wait<0>();
+        __syncthreads();  // the rings are reused by the next item
+    }
+}
+
+template <int ST, typename T, int TY, int LN, bool AL>
+static cudaError_t launch_mh_rows_tile(const MhArgs &a, double c3g, cudaStream_t s, int n_sm) {
+    typedef MhRows3dShape<ST, T, TY, LN> Sh;
+    constexpr size_t smem = Sh::smem_bytes + (AL ? 0 : Sh::stage_bytes);
+    static_assert(smem <= 227 * 1024, "shared memory per CTA");
+    auto kern = mh_rows3d_kernel<ST, T, TY, LN, AL>;
+    static const int occ = [&] {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        int o = 1;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, Sh::NT, smem);
+        return o;
+    }();
+    const int tx = (a.nx + Sh::TX - 1) / Sh::TX, ty = (a.ny + TY - 1) / TY;
+    const long long wave = (long long)n_sm * std::max(occ, 1);
+    const int segs = lockstep_segments((long long)tx * ty, a.nz, 4 * Sh::R, wave);
+    return launch_pdl(kern, dim3((unsigned)std::min((long long)tx * ty * segs, wave)), dim3(Sh::NT), smem, s, a,
+                      (float)c3g, tx, ty, segs);
+}
+
+// 120 x 12 tiles (32-lane rows) or 56 x 28 (16-lane rows): the one whose tiles cover the grid
+// in less time, 1.2 to 1.33 (12 to 13.5 us per 1000 planes of a tile): 256^3 7-point 208 against
+// 166 us per step, 360 x 300 x 400 345 / 432, 320 x 161 x 112 63 / 58.
+template <int ST, typename T, bool AL>
+static cudaError_t launch_mh_rows(const MhArgs &a, double c3g, cudaStream_t s, int n_sm) {
+    const double wide = 1.2 * ((a.nx + 119) / 120) * ((a.ny + 11) / 12);
+    const double narrow = 1.33 * ((a.nx + 55) / 56) * ((a.ny + 27) / 28);
+    if (wide <= narrow) return launch_mh_rows_tile<ST, T, 12, 32, AL>(a, c3g, s, n_sm);
+    return launch_mh_rows_tile<ST, T, 28, 16, AL>(a, c3g, s, n_sm);
+}
+
 template <int ST, typename T>
 static cudaError_t launch_mh_t(const MhArgs &a, double c3g, cudaStream_t s, int n_sm) {
     typedef typename Cmp<T>::type C;
@@ -366,7 +561,18 @@ static cudaError_t launch_mh_t(const MhArgs &a, double c3g, cudaStream_t s, int 
         }
     }
     if constexpr (StencilInfo<ST>::dims == 3 && !std::is_same<T, double>::value) {
-        // family 0: z-streaming tiles; family 1: the two per-point passes
+        // family 0: warp rows (radius 1) or z-streaming tiles; family 1: the two per-point passes
+        if constexpr (StencilInfo<ST>::r == 1) {
+            bool al = a.nx % 4 == 0;
+            for (int f = 0; f < 3; ++f) al = al && ((uintptr_t)a.j[f] | (uintptr_t)a.jo[f]) % 16 == 0;
+            al = al && ((uintptr_t)a.m | (uintptr_t)a.mo) % 16 == 0;
+            if (g_step_variant != 1 && al) return launch_mh_rows<ST, T, true>(a, c3g, s, n_sm);
+            // unaligned rows cost the 7-point kernel more than the tile ring's scalar reads
+            // (255 x 253 x 257: 254 against 207 us; 27-point 364 against 464)
+            if constexpr (sizeof(T) == 4 && ST == L27) {
+                if (g_step_variant != 1) return launch_mh_rows<ST, T, false>(a, c3g, s, n_sm);
+            }
+        }
         if (g_step_variant != 1) {
             constexpr int TX = 32, TY = 16, NT = 256;
             typedef MhRing3dShape<ST, T, TX, TY> Sh;

@@ -1422,39 +1422,40 @@ struct NoRow {  // stands for RaggedRow where rows are aligned
     __device__ __forceinline__ NoRow(int, int, int) {}
 };
 
-// A warp's row of 128 cells (lane l holds cells 4 l .. 4 l + 3) of a grid whose rows are not
-// 16-byte aligned: copied in and written out element by element, consecutive lanes
-// consecutive cells.  left: column of cell 0; cells 4 .. 123 are outputs.
-struct RaggedRow {
+// A row of LN lanes (lane l holds cells 4 l .. 4 l + 3; the first and the last lane are halo)
+// of a grid whose rows are not 16-byte aligned: copied in and written out element by
+// element, consecutive lanes consecutive cells.  left: column of cell 0.
+template <int LN> struct RaggedRow {
     int left, lane, cw[4];
     __device__ __forceinline__ RaggedRow(int left_, int lane_, int nx) : left(left_), lane(lane_) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) cw[q] = wrap_idx(left + lane + 32 * q, nx);
+        for (int q = 0; q < 4; ++q) cw[q] = wrap_idx(left + lane + LN * q, nx);
     }
-    // row: the grid row's first element; dst: the 128 cells in shared memory
+    // row: the grid row's first element; dst: cell 0 in shared memory
     template <typename T> __device__ __forceinline__ void fetch(T *dst, const T *row) const {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) cp_async_elem(dst + lane + 32 * q, row + cw[q]);
+        for (int q = 0; q < 4; ++q) cp_async_elem(dst + lane + LN * q, row + cw[q]);
     }
-    // this lane's 4 outputs, through 512 bytes of shared memory of the warp
-    __device__ __forceinline__ void put(float *row, float *stage, const float (&o)[4], int nx) const {
+    // this lane's 4 outputs, through 16 LN bytes of shared memory (every lane of the warp
+    // calls; on: whether the row is written)
+    __device__ __forceinline__ void put(float *row, float *stage, const float (&o)[4], int nx, bool on) const {
         __syncwarp();  // the previous row has left the buffer
         store_vec<float, 4>(stage + 4 * lane, o);
         __syncwarp();
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const int e = lane + 32 * q;
-            if (e >= 4 && e < 124 && left + e < nx) row[left + e] = stage[e];
+            const int e = lane + LN * q;
+            if (on && e >= 4 && e < 4 * LN - 4 && left + e < nx) row[left + e] = stage[e];
         }
     }
 };
 
 // ===================================================== 3D, warp rows ==
 //
-// FP32 / BF16-storage 3D kernel built like the 2D warp-strip kernel.  Warp w
-// of a CTA owns input row w of a tile (TY output rows plus R halo rows on each
-// side) and lane l the chunk l of 4 cells of that row (16 bytes FP32, 8 bytes
-// BF16): lanes 1..30 are the tile's 30 chunks, lanes 0 and 31 halo chunks.
+// FP32 / BF16-storage 3D kernel built like the 2D warp-strip kernel.  LN = 32 lanes (a
+// warp) or 16 (half of one) own an input row of a tile (TY output rows plus R halo rows on
+// each side), lane l the chunk l of 4 cells of that row (16 bytes FP32, 8 bytes BF16): the
+// first and the last lane are halo chunks, the others the tile's.
 // Planes stream along z through a ring of P+1 planes in shared memory filled by
 // cp.async (each thread copies its own chunk; one base pointer per plane, the
 // global source and destination offsets advance by a plane each step).
@@ -1471,8 +1472,9 @@ struct RaggedRow {
 // results bit for bit.
 //
 // AL: nx is a multiple of 4 and the field pointers are 16-byte aligned.  Otherwise (FP32)
-// rows go through RaggedRow: 301 x 299 x 303 Cahn-Hilliard 7-point 162 us per step with the
-// register-staged kernel that took such grids before, @@ now (aligned 300^3 @@).
+// rows go through RaggedRow: 301 x 299 x 303 Cahn-Hilliard 7-point 165 us per step with the
+// register-staged kernel that took such grids before, 92 now (300^3 66); 27-point 381 -> 157,
+// Gray-Scott 7-point 280 -> 114.
 
 // Number of in-plane partial sums per plane.
 template <int ST> struct Planar { static constexpr int NP = (ST == L7) ? 1 : 2; };
@@ -1517,74 +1519,84 @@ __device__ __forceinline__ float2 planar_combine2(const FA &f, const PA &p, int 
     }
 }
 
-template <int MODEL, int ST, typename T, int TY>
+template <int MODEL, int ST, typename T, int TY, int LN_ = 32>
 struct Step3dWrShape {
+    static constexpr int LN = LN_;                    // lanes of a row
     typedef typename Cmp<T>::type C;
     static constexpr int V = 4;                       // cells per lane (16 bytes FP32, 8 bytes BF16)
     static constexpr int CB = V * (int)sizeof(T);     // chunk bytes
     static constexpr int r = StencilInfo<ST>::r;
     static constexpr int R = (MODEL == CH) ? 2 * r : r;
     static_assert(V >= 2 * r, "a lane's chunk must cover the halo");
-    static constexpr int TXC = 30;                    // output chunks per tile row
+    static constexpr int TXC = LN - 2;                // output chunks per tile row
     static constexpr int TX = TXC * V;
-    static constexpr int HIN = TY + 2 * R;            // warps = input rows
-    static constexpr int NT = 32 * HIN;
+    static constexpr int HIN = TY + 2 * R;            // input rows
+    static constexpr int NT = LN * HIN;
+    static_assert(NT % 32 == 0, "whole warps");
     static constexpr int XW = V + 2 * r;
     static constexpr int NP = Planar<ST>::NP;
     static constexpr int Q = 2 * r + 1;               // planes in a queue (incl. the newest)
     static constexpr int P = 3;                       // planes in flight
     static constexpr int NF = num_fields<MODEL>();
-    static constexpr size_t plane_bytes = (size_t)HIN * 32 * CB;
+    static constexpr size_t plane_bytes = (size_t)HIN * LN * CB;
     static constexpr size_t in_bytes = (size_t)(P + 1) * NF * plane_bytes;
     // Cahn-Hilliard: two mu planes (plane j - r is written while the output stage
     // reads plane j - 1 - r), so one barrier per plane suffices
-    static constexpr size_t mu_plane = (size_t)HIN * 32 * V;
+    static constexpr size_t mu_plane = (size_t)HIN * LN * V;
     static constexpr size_t mu_bytes = (MODEL == CH) ? 2 * mu_plane * sizeof(float) : 0;
     static constexpr size_t smem_bytes = in_bytes + mu_bytes;
-    static constexpr size_t stage_bytes = (size_t)HIN * NF * 512;  // not AL: output rows
+    static constexpr size_t stage_bytes = (size_t)HIN * NF * LN * 16;  // not AL: output rows
     // resident CTAs per SM asked of the register allocator (measured on GB300:
     // Allen-Cahn with radius-1 stencils gains from a third CTA; Cahn-Hilliard
     // 7-point needs two; elsewhere a bound would make the queues spill)
     static constexpr int MINB = (MODEL == AC && r == 1) ? 3 : ((MODEL == CH && ST == L7) ? 2 : 1);
 };
 
-template <int MODEL, int ST, typename T, int TY, bool AL>
-__global__ void __launch_bounds__(Step3dWrShape<MODEL, ST, T, TY>::NT, Step3dWrShape<MODEL, ST, T, TY>::MINB)
+template <int MODEL, int ST, typename T, int TY, int LN, bool AL>
+__global__ void __launch_bounds__(Step3dWrShape<MODEL, ST, T, TY, LN>::NT, Step3dWrShape<MODEL, ST, T, TY, LN>::MINB)
     step3d_wr_kernel(StepArgs a, int tiles_x, int tiles_y, int segs) {
     pdl_enter();
     static_assert(MODEL != MC, "Model C runs on the accessor-based kernels");
-    typedef Step3dWrShape<MODEL, ST, T, TY> Sh;
+    typedef Step3dWrShape<MODEL, ST, T, TY, LN> Sh;
     typedef float C;
     constexpr int V = Sh::V, r = Sh::r, R = Sh::R, HIN = Sh::HIN, XW = Sh::XW, NP = Sh::NP, Q = Sh::Q;
     constexpr int P = Sh::P, NF = Sh::NF, CB = Sh::CB;
     constexpr unsigned FULL = 0xffffffffu;
     typedef typename VecT<CB>::type W;                                      // one chunk
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    W *s_in = reinterpret_cast<W *>(smem_raw);                              // [P+1][NF][HIN][32]
-    float *s_mu = reinterpret_cast<float *>(smem_raw + Sh::in_bytes);      // [2][HIN][32][V]
+    W *s_in = reinterpret_cast<W *>(smem_raw);                              // [P+1][NF][HIN][LN]
+    float *s_mu = reinterpret_cast<float *>(smem_raw + Sh::in_bytes);      // [2][HIN][LN][V]
 
     const ConstsF2 k2(ConstsC<C>(a.k, a.kf));
     const int nx = a.nx, ny = a.ny, nz = a.nz;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int lane = threadIdx.x & (LN - 1), w = threadIdx.x / LN;
     const size_t plane = (size_t)nx * (size_t)ny;
     const T *in[2] = {static_cast<const T *>(a.in0), static_cast<const T *>(a.in1)};
     T *out[2] = {static_cast<T *>(a.out0), static_cast<T *>(a.out1)};
-    const bool mu_row = (MODEL == CH) && w >= r && w < HIN - r;
     const bool out_row = w >= R && w < HIN - R;
+    // Rows whose stencil sums are formed (Cahn-Hilliard: of mu, and of phi for mu), the whole
+    // warp where one of its rows is (LN = 16: two rows per warp): a row that is not reads in
+    // place of its own the nearest one that is, so that every access stays in the plane.
+    constexpr int RPW = 32 / LN;
+    auto any_row = [&](int lo) { return (w | (RPW - 1)) >= lo && (w & ~(RPW - 1)) < HIN - lo; };
+    const bool mu_rows = (MODEL == CH) && any_row(r), out_rows = any_row(R);
+    const int wy = LN == 32 ? w : min(max(w, r), HIN - 1 - r), wo = LN == 32 ? w : min(max(w, R), HIN - 1 - R);
 
     // this lane's chunk of its own row in ring slot 0 (field 0); other slots,
     // fields and rows lie at fixed offsets, so each plane needs one base pointer
     constexpr int D = P + 1;  // ring slots
     static_assert((D & (D - 1)) == 0, "ring slots must be a power of two");
-    constexpr size_t SLOT = (size_t)NF * HIN * 32, FLD = (size_t)HIN * 32;
-    W *const s_own = s_in + (size_t)w * 32 + lane;
-    float *const mu_own = s_mu + ((size_t)w * 32 + lane) * V;
-    float *const stage = reinterpret_cast<float *>(smem_raw + Sh::smem_bytes) + (size_t)w * NF * 128;  // not AL
+    constexpr size_t SLOT = (size_t)NF * HIN * LN, FLD = (size_t)HIN * LN;
+    W *const s_own = s_in + (size_t)w * LN + lane;
+    const W *const s_read = LN == 32 ? s_own : s_in + (size_t)wy * LN + lane;
+    float *const mu_own = s_mu + ((size_t)w * LN + lane) * V;
+    const float *const mu_read = LN == 32 ? mu_own : s_mu + ((size_t)wo * LN + lane) * V;
+    float *const stage = reinterpret_cast<float *>(smem_raw + Sh::smem_bytes) + (size_t)w * NF * 4 * LN;  // not AL
     (void)stage;
     // chunk at row offset dy of field f in the slot starting at `base`, widened
     auto ring_chunk = [&](const W *base, int f, int dy, float *dst) {
         union { W q; T t[V]; } u;
-        u.q = base[f * FLD + dy * 32];
+        u.q = base[f * FLD + dy * LN];
 #pragma unroll
         for (int i = 0; i < V; ++i) dst[i] = to_c(u.t[i]);
     };
@@ -1592,8 +1604,8 @@ __global__ void __launch_bounds__(Step3dWrShape<MODEL, ST, T, TY>::NT, Step3dWrS
     auto extend = [&](float *ext) {
 #pragma unroll
         for (int h = 0; h < r; ++h) {
-            ext[h] = __shfl_up_sync(FULL, ext[V + h], 1);
-            ext[r + V + h] = __shfl_down_sync(FULL, ext[r + h], 1);
+            ext[h] = __shfl_up_sync(FULL, ext[V + h], 1, LN);
+            ext[r + V + h] = __shfl_down_sync(FULL, ext[r + h], 1, LN);
         }
     };
 
@@ -1607,15 +1619,15 @@ __global__ void __launch_bounds__(Step3dWrShape<MODEL, ST, T, TY>::NT, Step3dWrS
         const int col = x0 + (lane - 1) * V;                       // first cell of this lane's chunk
         const size_t goff = (size_t)wrap_idx(y0 - R + w, ny) * nx + (AL ? wrap_idx(col, nx) : 0);
         const int yo = y0 - R + w;                                 // output row (if out_row)
-        const bool store = out_row && lane >= 1 && lane <= 30 && col < nx && yo < ny;
-        const typename std::conditional<AL, NoRow, RaggedRow>::type rag(x0 - V, lane, nx);
+        const bool store = out_row && lane >= 1 && lane <= LN - 2 && col < nx && yo < ny;
+        const typename std::conditional<AL, NoRow, RaggedRow<LN>>::type rag(x0 - V, lane, nx);
         // V outputs of every lane to row yo of field f, plane at dst_off
         size_t dst_off = (size_t)z0 * plane + (size_t)yo * nx + (AL ? col : 0);
         auto put = [&](int f, const float (&o)[V]) {
             if constexpr (AL) {
                 if (store) store_vec<T, V>(out[f] + dst_off, o);
             } else {
-                if (yo < ny) rag.put(out[f] + dst_off, stage + f * 128, o, nx);
+                rag.put(out[f] + dst_off, stage + f * 4 * LN, o, nx, out_row && yo < ny);
             }
         };
         // element offsets: next plane to fetch (plane jn, wrapped z zn) and next output
@@ -1669,7 +1681,7 @@ __global__ void __launch_bounds__(Step3dWrShape<MODEL, ST, T, TY>::NT, Step3dWrS
                     // published and the mu buffer of plane j-2-r free
                     __syncthreads();
                     issue();          // plane j + P into plane j-1's slot
-                    const W *cur = s_own + (size_t)(j & (D - 1)) * SLOT;
+                    const W *cur = s_read + (size_t)(j & (D - 1)) * SLOT;
 #define QS(m) ((u - (m) + 4 * Q) % Q)   /* queue slot of plane j - m */
                     if constexpr (MODEL == CH) {
                         // output stage on mu plane j - 1 - r (written in the previous
@@ -1677,9 +1689,9 @@ __global__ void __launch_bounds__(Step3dWrShape<MODEL, ST, T, TY>::NT, Step3dWrS
                         // first because phi of its output plane j - 1 - 2r and the mu
                         // of plane j - 1 - 3r sit in the queue slots that plane j and
                         // mu plane j - r take below
-                        if (out_row && j >= 2 * r + 1) {
+                        if (out_rows && j >= 2 * r + 1) {
                             const float2 *mu = qm[QS(1)];
-                            const float *mu_prev = mu_own + (size_t)((j - 1) & 1) * Sh::mu_plane;
+                            const float *mu_prev = mu_read + (size_t)((j - 1) & 1) * Sh::mu_plane;
                             float ext[2 * r + 1][XW];
 #pragma unroll
                             for (int q = 0; q < V2; ++q) {
@@ -1690,7 +1702,7 @@ __global__ void __launch_bounds__(Step3dWrShape<MODEL, ST, T, TY>::NT, Step3dWrS
 #pragma unroll
                             for (int dy = -r; dy <= r; ++dy) {
                                 if (dy == 0) continue;
-                                const float *src_mu = mu_prev + dy * 32 * V;
+                                const float *src_mu = mu_prev + dy * LN * V;
 #pragma unroll
                                 for (int i = 0; i < V; i += 4) {
                                     const float4 v4 = *reinterpret_cast<const float4 *>(src_mu + i);
@@ -1721,7 +1733,7 @@ __global__ void __launch_bounds__(Step3dWrShape<MODEL, ST, T, TY>::NT, Step3dWrS
                             }
                         }
                     }
-                    if (j < n && ((MODEL == CH && mu_row) || (MODEL != CH && out_row))) {
+                    if (j < n && ((MODEL == CH && mu_rows) || (MODEL != CH && out_rows))) {
 #pragma unroll
                         for (int f = 0; f < NF; ++f) {
                             float ext[2 * r + 1][XW];
@@ -1750,7 +1762,7 @@ __global__ void __launch_bounds__(Step3dWrShape<MODEL, ST, T, TY>::NT, Step3dWrS
                     (void)f1q; (void)p1q;
                     if constexpr (MODEL == CH) {
                         // mu of plane j - r into the queue and the mu buffer of this iteration
-                        if (mu_row && j >= 2 * r && j < n) {
+                        if (mu_rows && j >= 2 * r && j < n) {
                             float2 *mu = qm[QS(0)];
 #pragma unroll
                             for (int q = 0; q < V2; ++q)
@@ -1762,7 +1774,7 @@ __global__ void __launch_bounds__(Step3dWrShape<MODEL, ST, T, TY>::NT, Step3dWrS
                                     make_float4(mu[q].x, mu[q].y, mu[q + 1].x, mu[q + 1].y);
                         }
                     } else {
-                        if (out_row && j >= 2 * r) {
+                        if (out_rows && j >= 2 * r) {
                             float o0[V], o1[V];
 #pragma unroll
                             for (int q = 0; q < V2; ++q) {
@@ -1977,7 +1989,7 @@ __global__ void __launch_bounds__(Step3dTbsShape<MODEL, ST, T, TY, K>::NT)
         const size_t goff = (size_t)wrap_idx(y0 - K * r + w, ny) * nx + (AL ? wrap_idx(col, nx) : 0);
         const int yo = y0 - K * r + w;
         const bool store = w >= K * r && w < HIN - K * r && lane >= 1 && lane <= 30 && col < nx && yo < ny;
-        const typename std::conditional<AL, NoRow, RaggedRow>::type rag(x0 - V, lane, nx);
+        const typename std::conditional<AL, NoRow, RaggedRow<32>>::type rag(x0 - V, lane, nx);
         int jn = 0, zn = wrap_idx(z0 - K * r, nz);
         size_t src = (size_t)zn * plane + goff;
         size_t dst_off = (size_t)z0 * plane + (size_t)yo * nx + (AL ? col : 0);
@@ -1985,7 +1997,7 @@ __global__ void __launch_bounds__(Step3dTbsShape<MODEL, ST, T, TY, K>::NT)
             if constexpr (AL) {
                 if (store) store_vec<T, V>(out[f] + dst_off, o);
             } else {
-                if (yo < ny) rag.put(out[f] + dst_off, stage + f * 128, o, nx);
+                rag.put(out[f] + dst_off, stage + f * 128, o, nx, yo < ny);
             }
         };
         auto issue = [&]() {

@@ -12,6 +12,7 @@
 
 #include "sp_internal.h"
 #include "sp_step.cuh"
+#include "sp_wr.cuh"
 
 namespace sp {
 
@@ -141,25 +142,6 @@ cudaError_t launch_tbs(const StepArgs &a, cudaStream_t s, int n_sm) {
     const int tx = (a.nx + Sh::TX - 1) / Sh::TX, ty = (a.ny + TY - 1) / TY;
     const long long wave = (long long)n_sm * std::max(occ, 1);
     const int segs = lockstep_segments((long long)tx * ty, a.nz, 2 * K * Sh::r, wave);
-    const long long items = (long long)tx * ty * segs;
-    return launch_pdl(kern, dim3((unsigned)std::min(items, wave)), dim3(Sh::NT), smem, s, a, tx, ty, segs);
-}
-
-// 3D FP32 / BF16, warp per tile row with z neighbours in registers.
-template <int MODEL, int ST, typename T, int TY, bool AL>
-cudaError_t launch_wr(const StepArgs &a, cudaStream_t s, int n_sm) {
-    typedef Step3dWrShape<MODEL, ST, T, TY> Sh;
-    constexpr size_t smem = Sh::smem_bytes + (AL ? 0 : Sh::stage_bytes);
-    auto kern = step3d_wr_kernel<MODEL, ST, T, TY, AL>;
-    static const int occ = [&] {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        int o = 1;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, Sh::NT, smem);
-        return o;
-    }();
-    const int tx = (a.nx + Sh::TX - 1) / Sh::TX, ty = (a.ny + TY - 1) / TY;
-    const long long wave = (long long)n_sm * std::max(occ, 1);
-    const int segs = lockstep_segments((long long)tx * ty, a.nz, 2 * Sh::R, wave);
     const long long items = (long long)tx * ty * segs;
     return launch_pdl(kern, dim3((unsigned)std::min(items, wave)), dim3(Sh::NT), smem, s, a, tx, ty, segs);
 }
@@ -345,22 +327,28 @@ cudaError_t launch_step_t(const StepArgs &a, cudaStream_t s, int n_sm, int k) {
         const bool aligned = ((uintptr_t)a.in0 | (uintptr_t)a.in1 | (uintptr_t)a.out0 | (uintptr_t)a.out1) % 16 == 0;
         constexpr int WTY = 8;
         typedef Step3dWrShape<MODEL, ST, T, WTY> WS;
-        auto wkern = step3d_wr_kernel<MODEL, ST, T, WTY, true>;
-        // the warp-row kernel is the default unless its register queues spill
-        // (a spill of a few words outside the queues costs nothing measurable)
-        static const bool wr_spills = [&] {
-            cudaFuncAttributes fa{};
-            return cudaFuncGetAttributes(&fa, wkern) != cudaSuccess || fa.localSizeBytes > 16;
-        }();
-        const int fam = (g_step_variant == 0 && wr_spills) ? 1 : g_step_variant;
-        if (fam == 0 && a.nx % WS::V == 0 && aligned) return launch_wr<MODEL, ST, T, WTY, true>(a, s, n_sm);
+        // Family 0: the warp-row kernel.  FP32 chooses among its tiles, any alignment
+        // (sp_wr.cuh); 16-bit storage takes rows of 32 lanes unless its queues spill.
+        int fam = g_step_variant;
         if constexpr (sizeof(T) == 4) {
-            // unaligned rows: the same kernel, or the plane ring for Gray-Scott, whose two
-            // fields' queues spill
-            if (g_step_variant == 0 && !(a.nx % WS::V == 0 && aligned)) {
-                if constexpr (MODEL == GS) return launch_tbs<MODEL, ST, T, 8, 1, false>(a, s, n_sm);
-                else return launch_wr<MODEL, ST, T, WTY, false>(a, s, n_sm);
+            if (fam == 0) {
+                const cudaError_t e = launch_wr_f32(MODEL, ST, a, s, n_sm);
+                if (e != cudaErrorNotSupported) return e;
+                fam = 1;  // the plane ring is the cheaper one
             }
+        } else if (fam == 0) {
+            auto wkern = step3d_wr_kernel<MODEL, ST, T, WTY, 32, true>;
+            static const bool spills = [&] {
+                cudaFuncAttributes fa{};
+                return cudaFuncGetAttributes(&fa, wkern) != cudaSuccess || fa.localSizeBytes > 16;
+            }();
+            if (!spills && a.nx % 4 == 0 && aligned) {
+                const int tx = (a.nx + WS::TX - 1) / WS::TX, ty = (a.ny + WTY - 1) / WTY;
+                const long long wave = (long long)n_sm * std::max(wr_occupancy<MODEL, ST, T, WTY, 32, true>(), 1);
+                return launch_wr<MODEL, ST, T, WTY, 32, true>(
+                    a, s, n_sm, lockstep_segments((long long)tx * ty, a.nz, 2 * WS::R, wave));
+            }
+            fam = 1;
         }
         if (fam == kTmaFamily && a.nx % AS::V == 0 && aligned) {
             // FP32 / BF16 3D: the plane ring with tensor-map plane loads

@@ -54,3 +54,18 @@ def test_3d_rows(sp, model, st, shape):
 def test_2d_fp64_default_equals_single_steps(sp, model, shape):
     for x, y in zip(run(sp, model, shape, 0, 0, None), run(sp, model, shape, 0, 0, (1, 0))):
         assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("dtype", [1, 2])
+@pytest.mark.parametrize("st", [3, 4])
+@pytest.mark.parametrize("shape", [(1, 1, 1), (2, 3, 5), (9, 12, 120), (5, 13, 130), (40, 9, 7), (3, 25, 245), (7, 8, 124)])
+def test_model_h_rows(sp, st, shape, dtype):
+    """Warp rows against the two per-point passes (tiles of 12 rows x 120 cells)."""
+    def go(fam):
+        kw = dict(flags=sp.FLAG_BF16_NO_BOUND) if dtype == 2 else {}
+        with sp.Simulation(sp.MODEL_H, shape, dt=0.001, stencil=st, dtype=dtype, seed=4, ic_amp=0.5, **kw) as s:
+            s.launch_config = (1, fam)
+            s.step(5)
+            return [s.read(f) for f in range(4)]
+    for x, y in zip(go(0), go(1)):
+        assert np.array_equal(x, y)
