@@ -312,7 +312,8 @@ template <typename R> struct FftBounds {
 
 template <typename R, int MODE, int V>
 __global__ void __launch_bounds__(FftBounds<R>::NT, FftBounds<R>::MINB)
-    rows_regs_kernel(R *f, typename Cplx<R>::type *Z, PassGeom g, R coef, FftLen L, const typename Cplx<R>::type *tw) {
+    rows_regs_kernel(R *f, typename Cplx<R>::type *Z, const __grid_constant__ PassGeom g, R coef,
+                     const __grid_constant__ FftLen L, const typename Cplx<R>::type *tw) {
     typedef typename Cplx<R>::type C;
     constexpr int H = V / 2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -327,8 +328,7 @@ __global__ void __launch_bounds__(FftBounds<R>::NT, FftBounds<R>::MINB)
     const bool has_b = ra + 1 < g.nrows, vec = (g.nrows & 1) == 0;
     const size_t ro = (size_t)ra * n;
     C u[V];
-    auto read_pair = [&](int k, C &A, C &B) {  // modes k of the two rows
-        const C *p = Z + ((uint64_t)(uint32_t)k * (uint32_t)g.nrows + (uint32_t)ra);
+    auto read_pair = [&](const C *p, C &A, C &B) {  // a mode of the two rows
         if (sizeof(R) == 4 && vec) {
             const float4 q = *reinterpret_cast<const float4 *>(p);
             A = C{(R)q.x, (R)q.y};
@@ -344,16 +344,18 @@ __global__ void __launch_bounds__(FftBounds<R>::NT, FftBounds<R>::MINB)
         // bins are real.  Values are held with real and imaginary part exchanged.
         if (on) {
             C A, B;
+            const C *p = Z + ((uint64_t)(uint32_t)t * (uint32_t)g.nrows + (uint32_t)ra);
+            const size_t step = (size_t)T * g.nrows;
 #pragma unroll
-            for (int j = 0; j < H; ++j) {
+            for (int j = 0; j < H; ++j, p += step) {
                 const int i = t + j * T;
-                read_pair(i, A, B);
+                read_pair(p, A, B);
                 if (i == 0) A.y = B.y = R(0);
                 u[j] = C{A.y + B.x, A.x - B.y};
                 if (i > 0) buf[slot_of(n - i, sh)] = C{B.x - A.y, A.x + B.y};
             }
             if (t == 0) {
-                read_pair(n / 2, A, B);
+                read_pair(p, A, B);  // mode n/2
                 buf[slot_of(n / 2, sh)] = C{B.x, A.x};
             }
         }
@@ -395,9 +397,8 @@ __global__ void __launch_bounds__(FftBounds<R>::NT, FftBounds<R>::MINB)
         for (int j = H; j < V; ++j) buf[slot_of(t + j * T, sh)] = u[j];
         lt.sync();
         if (on) {
-            auto put = [&](int k, C zk, C zc) {
+            auto put = [&](C *p, C zk, C zc) {
                 const C A{zk.x + zc.x, zk.y - zc.y}, B{zk.y + zc.y, zc.x - zk.x};
-                C *p = Z + ((uint64_t)(uint32_t)k * (uint32_t)g.nrows + (uint32_t)ra);
                 if (sizeof(R) == 4 && vec) {
                     *reinterpret_cast<float4 *>(p) = make_float4((float)A.x, (float)A.y, (float)B.x, (float)B.y);
                 } else {
@@ -405,12 +406,16 @@ __global__ void __launch_bounds__(FftBounds<R>::NT, FftBounds<R>::MINB)
                     if (has_b) p[1] = B;
                 }
             };
+            // from the highest mode down (see lines_regs_kernel)
+            const size_t step = (size_t)T * g.nrows;
+            C *p = Z + ((uint64_t)(uint32_t)(t + H * T) * (uint32_t)g.nrows + (uint32_t)ra);
+            if (t == 0) put(p, u[H], u[H]);
 #pragma unroll
-            for (int j = 0; j < H; ++j) {
+            for (int j = H - 1; j >= 0; --j) {
                 const int k = t + j * T;
-                put(k, u[j], k == 0 ? u[j] : buf[slot_of(n - k, sh)]);
+                p -= step;
+                put(p, u[j], k == 0 ? u[j] : buf[slot_of(n - k, sh)]);
             }
-            if (t == 0) put(n / 2, u[H], u[H]);
         }
     }
 }
@@ -435,7 +440,7 @@ __device__ __forceinline__ void prefetch_lines(const C *Z, const C *uh, const Pa
 
 template <typename R, int MODE, int MODEL, int V>
 __global__ void __launch_bounds__(FftBounds<R>::NT, FftBounds<R>::MINB)
-    lines_regs_kernel(typename Cplx<R>::type *Z, typename Cplx<R>::type *uh, PassGeom g, FftLen L,
+    lines_regs_kernel(typename Cplx<R>::type *Z, typename Cplx<R>::type *uh, const __grid_constant__ PassGeom g, const __grid_constant__ FftLen L,
                       const typename Cplx<R>::type *tw, const R *kx2, const R *ky2, const R *kz2, SpecCoef<R> c) {
     typedef typename Cplx<R>::type C;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -465,28 +470,29 @@ __global__ void __launch_bounds__(FftBounds<R>::NT, FftBounds<R>::MINB)
         if (MODE == kLineUpdate && on) kb = kx2[kx] + ky2[y];
     }
     if (MODE == kLineUpdate || g.ahead) prefetch_lines(Z, uh, g, L.n, MODE == kLineUpdate, base, l, t, T);
+    // Addresses advance by `step`; the stores at the end run backwards, so that the compiler
+    // does not keep the loads' 16 addresses for them (it spilled 430 bytes per thread).
+    const size_t step = (size_t)T * es, own = base + (uint64_t)(uint32_t)t * es;
     C u[V];
     if (on) {
+        const C *p = Z + own;
 #pragma unroll
-        for (int j = 0; j < V; ++j) {
-            const C v = Z[base + (uint32_t)(t + j * T) * es];
-            u[j] = MODE == kLineInverse ? swapped(v) : v;
-        }
+        for (int j = 0; j < V; ++j, p += step) u[j] = MODE == kLineInverse ? swapped(*p) : *p;
     }
 #pragma unroll 1
     for (int pass = 0; pass < (MODE == kLineUpdate ? 2 : 1); ++pass) {
         fft_regs(u, buf, L, tw, lt);
         if (MODE == kLineUpdate && pass == 0 && on) {
+            C *p = uh + own;
+            const R *k = kl + t;
 #pragma unroll
-            for (int j = 0; j < V; ++j) {
-                const int i = t + j * T;
-                u[j] = swapped(update_mode<R, MODEL>(uh + base + (uint32_t)i * es, u[j], kb + kl[i], c));
-            }
+            for (int j = 0; j < V; ++j, p += step, k += T) u[j] = swapped(update_mode<R, MODEL>(p, u[j], kb + *k, c));
         }
     }
     if (on) {
+        C *p = Z + own + (V - 1) * step;
 #pragma unroll
-        for (int j = 0; j < V; ++j) Z[base + (uint32_t)(t + j * T) * es] = MODE == kLineForward ? u[j] : swapped(u[j]);
+        for (int j = V - 1; j >= 0; --j, p -= step) *p = MODE == kLineForward ? u[j] : swapped(u[j]);
     }
 }
 
@@ -626,8 +632,9 @@ __device__ __forceinline__ C *fft_lines(C *buf, C *alt, const FftLen &L, int G, 
 }
 
 template <typename R, int MODE>
-__global__ void __launch_bounds__(512) rows_mixed_kernel(R *f, typename Cplx<R>::type *Z, PassGeom g, R coef, FftLen L,
-                                                          const typename Cplx<R>::type *tw) {
+__global__ void __launch_bounds__(512)
+    rows_mixed_kernel(R *f, typename Cplx<R>::type *Z, const __grid_constant__ PassGeom g, R coef,
+                      const __grid_constant__ FftLen L, const typename Cplx<R>::type *tw) {
     typedef typename Cplx<R>::type C;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *buf = reinterpret_cast<C *>(smem_raw), *alt = buf + g.G * L.n;
@@ -676,7 +683,7 @@ __global__ void __launch_bounds__(512) rows_mixed_kernel(R *f, typename Cplx<R>:
 
 template <typename R, int MODE, int MODEL>
 __global__ void __launch_bounds__(512)
-    lines_mixed_kernel(typename Cplx<R>::type *Z, typename Cplx<R>::type *uh, PassGeom g, FftLen L,
+    lines_mixed_kernel(typename Cplx<R>::type *Z, typename Cplx<R>::type *uh, const __grid_constant__ PassGeom g, const __grid_constant__ FftLen L,
                        const typename Cplx<R>::type *tw, const R *kx2, const R *ky2, const R *kz2, SpecCoef<R> c) {
     typedef typename Cplx<R>::type C;
     extern __shared__ __align__(16) unsigned char smem_raw[];
