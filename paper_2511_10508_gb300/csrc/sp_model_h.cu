@@ -415,6 +415,7 @@ __global__ void __launch_bounds__(MhRows3dShape<ST, T, TY, LN>::NT)
         const float4 v = *reinterpret_cast<const float4 *>(mu_own + (q % Sh::DMU) * Sh::mu_plane + dy * LN * V);
         dst[0] = v.x, dst[1] = v.y, dst[2] = v.z, dst[3] = v.w;
     };
+    const bool pair = !AL && pair_rows(nx, a.m, a.j[0], a.mo, a.jo[0]) && pair_rows(nx, a.j[1], a.j[2], a.jo[1], a.jo[2]);
     const bool out_row = w >= 2 * R && w < HIN - 2 * R;  // the same for both rows of a warp
     // mu is formed by whole warps: the outermost rows, which need none, repeat their neighbour's
     const int mu_dy = w < R ? R - w : w >= HIN - R ? HIN - 1 - R - w : 0;
@@ -428,7 +429,7 @@ __global__ void __launch_bounds__(MhRows3dShape<ST, T, TY, LN>::NT)
         const int col = x0 + (lane - 1) * V, yo = y0 - 2 * R + w;
         const size_t roff = (size_t)wrap_idx(yo, ny) * nx + (AL ? wrap_idx(col, nx) : 0);
         const bool store = out_row && lane >= 1 && lane <= LN - 2 && col < nx && yo < ny;
-        const typename std::conditional<AL, NoRow, RaggedRow<LN>>::type rag(x0 - V, lane, nx);
+        const typename std::conditional<AL, NoRow, RaggedRow<LN>>::type rag(x0 - V, lane, nx, pair);
         size_t dst_off = (size_t)z0 * plane + (size_t)yo * nx + (AL ? col : 0);
         auto put = [&](int f, const float (&o)[V]) {
             if constexpr (AL) {

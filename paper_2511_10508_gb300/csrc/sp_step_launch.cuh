@@ -128,11 +128,11 @@ cudaError_t launch_tb(const StepArgs &a, cudaStream_t s) {
 // steps per pass (temporal blocking for K = 2) on warp-row tiles of 120 x TY
 // outputs; lockstep z segments.  Needs nx a multiple of 4 and 16-byte aligned
 // fields (the runtime offers these families only then).
-template <int MODEL, int ST, typename T, int TY, int K, bool AL>
+template <int MODEL, int ST, typename T, int TY, int K, bool AL, int LN = 32>
 cudaError_t launch_tbs(const StepArgs &a, cudaStream_t s, int n_sm) {
-    typedef Step3dTbsShape<MODEL, ST, T, TY, K> Sh;
+    typedef Step3dTbsShape<MODEL, ST, T, TY, K, LN> Sh;
     constexpr size_t smem = Sh::smem_bytes + (AL ? 0 : Sh::stage_bytes);
-    auto kern = step3d_tbs_kernel<MODEL, ST, T, TY, K, AL>;
+    auto kern = step3d_tbs_kernel<MODEL, ST, T, TY, K, LN, AL>;
     static const int occ = [&] {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         int o = 1;
@@ -144,6 +144,17 @@ cudaError_t launch_tbs(const StepArgs &a, cudaStream_t s, int n_sm) {
     const int segs = lockstep_segments((long long)tx * ty, a.nz, 2 * K * Sh::r, wave);
     const long long items = (long long)tx * ty * segs;
     return launch_pdl(kern, dim3((unsigned)std::min(items, wave)), dim3(Sh::NT), smem, s, a, tx, ty, segs);
+}
+
+// Model C, one step: tiles of 120 x 8 (32-lane rows) or 56 x 16 (16-lane rows), whichever covers
+// the grid in less time (us per 1000 planes of a tile, 384^3: 7-point 2.5 both, 27-point 4.4 / 4.9,
+// 13-point 5.0 / 3.4; 256^3 7-point 64.9 against 55.2 us per step, 360^3 128 / 146).
+template <int ST, typename T, bool AL>
+cudaError_t launch_mc_rows(const StepArgs &a, cudaStream_t s, int n_sm) {
+    constexpr double c32 = ST == L7 ? 0.955 : ST == L27 ? 1.675 : 1.918, c16 = ST == L7 ? 0.935 : ST == L27 ? 1.883 : 1.295;
+    const double t32 = c32 * ((a.nx + 119) / 120) * ((a.ny + 7) / 8), t16 = c16 * ((a.nx + 55) / 56) * ((a.ny + 15) / 16);
+    if (t16 < t32) return launch_tbs<MC, ST, T, 16, 1, AL, 16>(a, s, n_sm);
+    return launch_tbs<MC, ST, T, 8, 1, AL>(a, s, n_sm);
 }
 
 // FP64 27-point: z-streaming kernel with per-plane partial sums in registers.
@@ -300,9 +311,10 @@ cudaError_t launch_step_t(const StepArgs &a, cudaStream_t s, int n_sm, int k) {
             if (k == 2 && g_step_variant == 1 && tall2) return launch_tbs<MODEL, ST, T, (tall2 ? 16 : 8), 2, true>(a, s, n_sm);
             if (k == 2) return launch_tbs<MODEL, ST, T, 8, 2, true>(a, s, n_sm);
             if (g_step_variant == 5) return launch_tbs<MODEL, ST, T, 16, 1, true>(a, s, n_sm);
-            if (g_step_variant == 4 || g_step_variant == 0) return launch_tbs<MODEL, ST, T, 8, 1, true>(a, s, n_sm);
+            if (g_step_variant == 4) return launch_tbs<MODEL, ST, T, 8, 1, true>(a, s, n_sm);
+            if (g_step_variant == 0) return launch_mc_rows<ST, T, true>(a, s, n_sm);
         } else if constexpr (sizeof(T) == 4) {
-            if (g_step_variant == 0) return launch_tbs<MODEL, ST, T, 8, 1, false>(a, s, n_sm);
+            if (g_step_variant == 0) return launch_mc_rows<ST, T, false>(a, s, n_sm);
         }
         constexpr int BX = 32, BY = 8, BZ = 8, NT = 256;
         typedef Step3dBoxShape<MODEL, ST, T, BX, BY, BZ> Sh;
