@@ -20,6 +20,7 @@
 #include <type_traits>
 
 #include "sp_internal.h"
+#include "sp_step.cuh"
 
 namespace sp {
 
@@ -440,6 +441,207 @@ __global__ void __launch_bounds__(NT, (MODEL == GS || MODEL == MC) ? 2 : 3) gen_
     }
 }
 
+// 3D FP32 / BF16: rows of 16 lanes (two per warp), lane l the 4 cells 4 l .. 4 l + 3, the first
+// and the last lane halo: tiles of 56 x TY outputs streamed along z.  2R + 1 planes of each
+// field (and P in flight) lie in a cp.async ring; a lane reads its chunk, the two beside it
+// and 2R chunks above, below, before and behind, 4 R + 3 reads of 16 bytes for 4 cells, where
+// the per-point kernels gather 6 R + 1 scalars per cell from L1 through 64-bit addresses.
+// PASS 0: mu of Cahn-Hilliard; 1: its update from mu; 2: a step of the other models (Model C
+// forms the density's chemical potential at every tap).  gen_sum's expressions in its
+// order, so the results are the per-point kernels'.  us per step, per point before and now:
+// Model C 130 x 328 x 232 order 2 247 / 65, 175 x 259 x 232 order 4 385 / 93, Gray-Scott 204 x 32 x
+// 272 order 4 43 / 12, Cahn-Hilliard 256^3 order 6 566 / 131, order 8 692 / 146.
+// AL: nx a multiple of 4 and 16-byte aligned fields; otherwise (FP32) RaggedRow.
+template <int PASS, int MODEL, int R, typename T>
+struct GenRows3dShape {
+    typedef typename std::conditional<PASS == 1, float, T>::type TI;  // streamed type
+    static constexpr int V = 4, CB = V * (int)sizeof(TI), LN = 16, TY = 16, P = 2;
+    static constexpr int TX = (LN - 2) * V, HIN = TY + 2 * R, NT = LN * HIN;
+    static_assert(NT % 32 == 0 && R <= V, "whole warps; one halo chunk");
+    static constexpr int NF = num_fields<MODEL>(), D = 2 * R + 1 + P;
+    static constexpr size_t PL = (size_t)HIN * LN;  // chunks of a plane
+    // a chunk of guard on each side: halo lanes read beside the first and the last row
+    static constexpr size_t smem_bytes = (D * NF * PL + 2) * CB;
+    static constexpr size_t stage_off = (smem_bytes + 15) / 16 * 16, stage_bytes = (size_t)HIN * LN * 16;
+};
+
+// Stencil sums and centre values of a lane's 4 cells; chunk(dz, offset in chunks, dst) reads
+// 4 cells of the plane dz away (LN chunks make a row).
+template <int R, int LN, typename Chunk>
+__device__ __forceinline__ void gen_row_sums(const Chunk &chunk, const GenW &W, float (&S)[4], float (&cen)[4]) {
+    float row[12], acc[4];
+    chunk(0, -1, row);
+    chunk(0, 0, row + 4);
+    chunk(0, 1, row + 8);
+#pragma unroll
+    for (int j = R; j >= 1; --j) {
+        float ym[4], yp[4], zm[4], zp[4];
+        chunk(0, -j * LN, ym);
+        chunk(0, j * LN, yp);
+        chunk(-j, 0, zm);
+        chunk(j, 0, zp);
+        const float2 wj = splat2(W.wf[j]);
+#pragma unroll
+        for (int c = 0; c < 4; c += 2) {
+            const float2 xs = make_float2(row[4 + c + j] + row[4 + c - j], row[5 + c + j] + row[5 + c - j]);
+            const float2 ys = add2(make_float2(yp[c], yp[c + 1]), make_float2(ym[c], ym[c + 1]));
+            const float2 zs = add2(make_float2(zp[c], zp[c + 1]), make_float2(zm[c], zm[c + 1]));
+            const float2 pj = add2(add2(xs, ys), zs);
+            const float2 r2 = j == R ? mul2(wj, pj) : fma2(wj, pj, make_float2(acc[c], acc[c + 1]));
+            acc[c] = r2.x;
+            acc[c + 1] = r2.y;
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        cen[c] = row[4 + c];
+        S[c] = FMA(W.wf[0], cen[c], acc[c]);
+    }
+}
+
+template <int PASS, int MODEL, int R, typename T, bool AL>
+__global__ void __launch_bounds__(GenRows3dShape<PASS, MODEL, R, T>::NT)
+    gen_rows3d_kernel(const __grid_constant__ GenArgs g, int tiles_x, int tiles_y, int segs) {
+    pdl_enter();
+    typedef GenRows3dShape<PASS, MODEL, R, T> Sh;
+    typedef typename Sh::TI TI;
+    typedef typename std::conditional<PASS == 0, float, T>::type TO;
+    constexpr int V = Sh::V, CB = Sh::CB, LN = Sh::LN, TY = Sh::TY, HIN = Sh::HIN, NF = Sh::NF, D = Sh::D, P = Sh::P;
+    typedef typename VecT<CB>::type W;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const StepArgs &a = g.a;
+    const ConstsC<float> k(a.k, a.kf);
+    const int nx = a.nx, ny = a.ny, nz = a.nz;
+    const int lane = threadIdx.x & (LN - 1), w = threadIdx.x / LN;
+    const size_t plane = (size_t)nx * (size_t)ny;
+    const TI *in[2] = {static_cast<const TI *>(PASS == 1 ? g.mu : a.in0), static_cast<const TI *>(a.in1)};
+    TO *out[2] = {static_cast<TO *>(PASS == 0 ? g.mu : a.out0), static_cast<TO *>(a.out1)};
+    const bool pair = !AL && pair_rows(nx, in[0], in[NF - 1], out[0], out[NF - 1]);
+    const bool out_row = w >= R && w < HIN - R;
+    const int wo = min(max(w, R), HIN - 1 - R);  // a halo row's lanes follow their warp on the nearest output row
+    const bool busy = (w | 1) >= R && (w & ~1) < HIN - R;
+    W *const own = reinterpret_cast<W *>(smem_raw) + 1 + (size_t)w * LN + lane;
+    const W *const mid = reinterpret_cast<W *>(smem_raw) + 1 + (size_t)wo * LN + lane;
+    float *const stage = reinterpret_cast<float *>(smem_raw + Sh::stage_off) + w * LN * V;
+    (void)stage;
+    auto widen = [&](const W *p, float *dst) {
+        union { W c; TI t[V]; } u;
+        u.c = *p;
+#pragma unroll
+        for (int i = 0; i < V; ++i) dst[i] = to_c(u.t[i]);
+    };
+    const int tiles = tiles_x * tiles_y;
+    for (long long it = blockIdx.x; it < (long long)tiles * segs; it += gridDim.x) {
+        const int seg = (int)(it / tiles), tile = (int)(it - (long long)seg * tiles);
+        const int z0 = (int)((long long)seg * nz / segs), z1 = (int)((long long)(seg + 1) * nz / segs);
+        const int x0 = (tile % tiles_x) * Sh::TX, y0 = (tile / tiles_x) * TY;
+        const int n = (z1 - z0) + 2 * R;  // loaded plane i is z = z0 - R + i
+        const int col = x0 + (lane - 1) * V, yo = y0 - R + w;
+        const size_t roff = (size_t)wrap_idx(yo, ny) * nx + (AL ? wrap_idx(col, nx) : 0);
+        const bool store = out_row && lane >= 1 && lane <= LN - 2 && col < nx && yo < ny;
+        const typename std::conditional<AL, NoRow, RaggedRow<LN>>::type rag(x0 - V, lane, nx, pair);
+        size_t dst_off = (size_t)z0 * plane + (size_t)yo * nx + (AL ? col : 0);
+        auto put = [&](int f, const float (&o)[V]) {
+            if constexpr (AL) {
+                if (store) store_vec<TO, V>(out[f] + dst_off, o);
+            } else {
+                rag.put(out[f] + dst_off, stage, o, nx, out_row && yo < ny);
+            }
+        };
+        auto issue = [&](int i) {
+            if (i < n) {
+                const size_t src = (size_t)wrap_idx(z0 - R + i, nz) * plane + roff;
+#pragma unroll
+                for (int f = 0; f < NF; ++f) {
+                    W *dst = own + ((i % D) * NF + f) * Sh::PL;
+                    if constexpr (!AL) rag.fetch(reinterpret_cast<TI *>(dst - lane), in[f] + src);
+                    else if constexpr (CB == 16) cp_async16(dst, in[f] + src);
+                    else cp_async8(dst, in[f] + src);
+                }
+            }
+            cp_async_commit();
+        };
+#pragma unroll
+        for (int i = 0; i < P; ++i) issue(i);
+        for (int i = 0; i < n; ++i) {
+            cp_async_wait<P - 1>();
+            __syncthreads();  // plane i published; plane i - 2R - 1's slot is free
+            issue(i + P);
+            if (i < 2 * R || !busy) continue;
+            const int t = i - R;  // output plane
+            auto at = [&](int f, int dz, int off) { return mid + (((t + dz) % D) * NF + f) * Sh::PL + off; };
+            float S[V], cen[V], o[V];
+            gen_row_sums<R, LN>([&](int dz, int off, float *d) { widen(at(0, dz, off), d); }, g.W, S, cen);
+            if constexpr (PASS == 2 && NF == 2) {
+                float S1[V], c1[V], v1[V], o1[V];
+                if constexpr (MODEL == MC) {
+                    auto tap = [&](int dz, int off, float *d) {
+                        float p[V], q[V];
+                        widen(at(0, dz, off), p), widen(at(NF - 1, dz, off), q);
+#pragma unroll
+                        for (int c = 0; c < V; ++c) d[c] = mc_mu<float>(p[c], q[c], k);
+                    };
+                    gen_row_sums<R, LN>(tap, g.W, S1, c1);
+                    widen(at(NF - 1, 0, 0), v1);
+                } else {
+                    gen_row_sums<R, LN>([&](int dz, int off, float *d) { widen(at(NF - 1, dz, off), d); }, g.W, S1, v1);
+                }
+#pragma unroll
+                for (int c = 0; c < V; ++c) two_field_update<MODEL, float>(cen[c], v1[c], S[c], S1[c], k, o[c], o1[c]);
+                put(0, o);
+                put(1, o1);
+            } else {
+                if constexpr (PASS == 1) {  // phi at the output points
+                    const T *phi = static_cast<const T *>(a.in0) + dst_off + (AL ? 0 : col);
+                    if constexpr (AL) {
+                        if (store) load_vec<T, V>(phi, cen);
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < V; ++c) cen[c] = store && col + c < nx ? load_one(phi + c) : 0.f;
+                    }
+                }
+#pragma unroll
+                for (int c = 0; c < V; ++c)
+                    o[c] = PASS == 0   ? ch_mu<float>(cen[c], S[c], k)
+                           : PASS == 1 ? ch_update<float>(cen[c], S[c], k)
+                                       : ac_update<float>(cen[c], S[c], k);
+                put(0, o);
+            }
+            dst_off += plane;
+        }
+        cp_async_wait<0>();
+        __syncthreads();  // the ring is reused by the next item
+    }
+}
+
+template <int PASS, int MODEL, int R, typename T, bool AL>
+static cudaError_t launch_gen_rows(const GenArgs &g, cudaStream_t s, int n_sm) {
+    typedef GenRows3dShape<PASS, MODEL, R, T> Sh;
+    constexpr size_t smem = Sh::stage_off + (AL ? 0 : Sh::stage_bytes);
+    static_assert(smem <= 227 * 1024, "shared memory per CTA");
+    auto kern = gen_rows3d_kernel<PASS, MODEL, R, T, AL>;
+    static const int occ = [&] {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        int o = 1;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, Sh::NT, smem);
+        return o;
+    }();
+    const int tx = (g.a.nx + Sh::TX - 1) / Sh::TX, ty = (g.a.ny + Sh::TY - 1) / Sh::TY;
+    const long long wave = (long long)n_sm * std::max(occ, 1);
+    const int segs = lockstep_segments((long long)tx * ty, g.a.nz, 2 * R, wave);
+    return launch_pdl(kern, dim3((unsigned)std::min((long long)tx * ty * segs, wave)), dim3(Sh::NT), smem, s, g, tx, ty, segs);
+}
+
+template <int MODEL, int R, typename T, bool AL>
+static cudaError_t launch_gen_rows_model(const GenArgs &g, cudaStream_t s, int n_sm) {
+    if constexpr (MODEL == CH) {
+        const cudaError_t e = launch_gen_rows<0, CH, R, T, AL>(g, s, n_sm);
+        return e != cudaSuccess ? e : launch_gen_rows<1, CH, R, T, AL>(g, s, n_sm);
+    } else {
+        return launch_gen_rows<2, MODEL, R, T, AL>(g, s, n_sm);
+    }
+}
+
 template <int MODEL, int R, int DIMS, typename T>
 static cudaError_t launch_gen_t(const GenArgs &g, cudaStream_t s, int n_sm) {
     if constexpr (DIMS == 2 && !std::is_same<T, double>::value) {
@@ -460,6 +662,12 @@ static cudaError_t launch_gen_t(const GenArgs &g, cudaStream_t s, int n_sm) {
             (void)attr;
             return launch_pdl(kern, dim3((g.a.nx + BX - 1) / BX, (g.a.ny + BY - 1) / BY), dim3(NT), Sh::smem_bytes, s, g);
         }
+    }
+    if constexpr (DIMS == 3 && !std::is_same<T, double>::value) {
+        const bool al = g.a.nx % 4 == 0 &&
+                        ((uintptr_t)g.a.in0 | (uintptr_t)g.a.in1 | (uintptr_t)g.a.out0 | (uintptr_t)g.a.out1) % 16 == 0;
+        if (al) return launch_gen_rows_model<MODEL, R, T, true>(g, s, n_sm);
+        if constexpr (sizeof(T) == 4) return launch_gen_rows_model<MODEL, R, T, false>(g, s, n_sm);
     }
     const int segs = (g.a.nx + 255) / 256;
     const long long units = (long long)g.a.ny * g.a.nz * segs;
