@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <array>
 
 #include "sp.h"
 #include "sp_common.cuh"
@@ -61,6 +62,61 @@ inline cudaError_t launch_wr_f32(int model, int stencil, const StepArgs &a, cuda
            : model == CH ? launch_wr_ch(stencil, a, s, n_sm) : launch_wr_gs(stencil, a, s, n_sm);
 }
 
+// 2D FP32, k = 2 or 4 steps per launch on warp rows (sp_w2d.cuh, one translation unit per
+// model); cudaErrorNotSupported where the tiles are to be used.
+cudaError_t launch_w2d_ac(int stencil, const StepArgs &a, cudaStream_t s, int n_sm, int k);
+cudaError_t launch_w2d_ch(int stencil, const StepArgs &a, cudaStream_t s, int n_sm, int k);
+cudaError_t launch_w2d_gs(int stencil, const StepArgs &a, cudaStream_t s, int n_sm, int k);
+cudaError_t launch_w2d_mc(int stencil, const StepArgs &a, cudaStream_t s, int n_sm, int k);
+inline cudaError_t launch_w2d(int model, int stencil, const StepArgs &a, cudaStream_t s, int n_sm, int k) {
+    return model == AC   ? launch_w2d_ac(stencil, a, s, n_sm, k)
+           : model == CH ? launch_w2d_ch(stencil, a, s, n_sm, k)
+           : model == GS ? launch_w2d_gs(stencil, a, s, n_sm, k) : launch_w2d_mc(stencil, a, s, n_sm, k);
+}
+
+// Rows per CTA of the 2D warp-strip kernel, whose CTAs own equal runs of the flattened
+// (strip group, row) space: p rows cost p + halo, q CTAs of `load` (their share of 8
+// warps) on the fullest SM take about q load + latency of them (see planes_per_cta).
+// Runs of at least 32 rows left most SMs idle on small grids: 444 x 568 Cahn-Hilliard 9.2
+// us per step, 3.0 now; 1504 x 1000 4th order 13.2 -> 6.2 (runs of 8 rows; of 4: 7.5).
+inline long long rows_per_cta(long long total, int halo, double load, double latency, int occ, int n_sm) {
+    const long long wave = (long long)n_sm * std::max(occ, 1), p0 = (total + wave - 1) / wave;
+    long long best = p0;
+    double best_cost = 0;
+    for (long long p = p0; p <= std::min(total, 8 * p0 + 32); ++p) {
+        const long long ctas = (total + p - 1) / p, q = (ctas + n_sm - 1) / n_sm;
+        const double cost = (q * load + latency) * (p + halo);
+        if (p == p0 || cost < best_cost * 0.999) {
+            best = p;
+            best_cost = cost;
+        }
+        if (q == 1) break;
+    }
+    return best;
+}
+
+// Warps per CTA of the 2D warp-strip kernels, whose CTAs take that many adjacent strips: the
+// most of at least max / 2 that leave the fewest warps without a strip (13 strips: two CTAs of
+// 7 warps, not of 8).
+inline int warps_per_cta(int strips, int max) {
+    if (strips <= max) return strips;
+    int best = max;
+    for (int w = max - 1; 2 * w >= max; --w)
+        if ((strips + w - 1) / w * w < (strips + best - 1) / best * best) best = w;
+    return best;
+}
+
+// Resident CTAs per SM by warps per CTA (1 .. MAXW) of a kernel that takes `smem` bytes per warp.
+template <int MAXW, typename Kern> std::array<int, MAXW + 1> warp_occupancy(Kern kern, size_t smem) {
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem * MAXW));
+    std::array<int, MAXW + 1> o{};
+    for (int w = 1; w <= MAXW; ++w) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o[w], kern, 32 * w, smem * w);
+        o[w] = std::max(o[w], 1);
+    }
+    return o;
+}
+
 // Number of equal z segments for a lockstep schedule of `tiles` x segments work
 // items over `wave` resident CTAs: minimises rounds x (planes per segment +
 // halo planes), the time of the slowest CTA.
@@ -89,16 +145,21 @@ inline int steps_per_launch_3d(int dtype, int model, int nx, int requested) {
     return (ok && requested >= 2) ? 2 : 1;
 }
 
-// 2D FP32 Allen-Cahn, Gray-Scott and Model C fuse steps by default: four up to 2^24 points
-// (radius-2 stencils, whose halo is twice as wide, 2^21), where the launch and the reuse in
-// L2 count (us per step with 2 and 4: Gray-Scott 2048^2 11.4 / 10.0, 4096^2 35.7 / 34.4, 8192^2
-// 128 / 130; Allen-Cahn 300 x 301 2.4 / 1.8; 4th order Allen-Cahn 3420 x 560 5.7 / 5.3, Model C
-// 4096^2 58 / 65), else two.  2D FP64 grids with a radius-1 stencil fuse two steps while the
+// 2D FP32 grids fuse steps by default where warp rows do (sp_w2d.cuh; us per step with 1, 2 and 4):
+// Allen-Cahn, Gray-Scott and Model C four with a radius-1 stencil (Gray-Scott 300 x 301 2.2 / 2.2 /
+// 1.9, 2048^2 10.4 / 6.9 / 5.8, 16384^2 785 / 398 / 216).  A radius-2 stencil leaves room for two; four
+// on tiles are the better choice on small grids (Allen-Cahn 1024^2 4.8 / 4.0 / 3.3, 2048^2 7.8 /
+// 5.4 / 8.7; Gray-Scott 512^2 3.4 / 3.5 / 2.5, 1024^2 5.6 / 3.9 / 5.5).  Cahn-Hilliard
+// (a step takes two halos) two with a radius-1 stencil on large grids (5-point 1024^2 3.7 / 3.1,
+// 8192^2 98 / 57, odd rows 1503 x 1001 4.6 / 5.0, 4097 x 4095 27 / 18; 9-point box 2048^2 7.7 / 9.1, 3000^2
+// 12.8 / 11.5, 8192^2 104 / 66).
+// 2D FP64 grids with a radius-1 stencil fuse two steps while the
 // 32 x 14 tiles of that kernel do not cost an SM one more tile than the 32 x 16 tiles of one step:
 // up to one tile per SM, and from two per SM up to 2^18 points (us per step with 1 and 2:
 // Allen-Cahn 256^2 3.5 / 2.7, 512^2 6.9 / 6.0, Gray-Scott 256^2 5.5 / 4.4; 257^2, where it does cost
 // one, 5.7 / 6.5).
-inline int steps_per_launch(int dims, int dtype, int model, int radius, int64_t nx, int64_t ny, int n_sm, int requested) {
+inline int steps_per_launch(int dims, int dtype, int model, int stencil, int64_t nx, int64_t ny, int n_sm, int requested) {
+    const int radius = stencil == SP_LAP_9CROSS4 ? 2 : 1;
     if (dims != 2 || model == SP_MODEL_H) return 1;
     const int64_t npts = nx * ny;
     if (requested == 0) {
@@ -106,8 +167,10 @@ inline int steps_per_launch(int dims, int dtype, int model, int radius, int64_t 
             const int64_t tx = (nx + 31) / 32, one = tx * ((ny + 15) / 16), two = tx * ((ny + 13) / 14);
             return two <= n_sm || one >= 2 * n_sm ? 2 : 1;
         }
-        if (dtype != SP_F32 || model == CH) return 1;
-        return npts <= (int64_t)1 << (radius == 1 ? 24 : 21) ? 4 : 2;
+        if (dtype != SP_F32) return 1;
+        if (model == SP_CAHN_HILLIARD)
+            return radius == 1 && npts >= (int64_t)1 << (stencil != SP_LAP_5 ? 23 : nx % 4 == 0 ? 20 : 22) ? 2 : 1;
+        return radius == 1 || npts <= (int64_t)1 << (model == SP_ALLEN_CAHN ? 21 : 18) ? 4 : 2;
     }
     if (requested >= 4) return 4;
     if (requested >= 2) return 2;

@@ -337,7 +337,7 @@ extern "C" int sp_create(int model, int dims, const int64_t shape[3], double h, 
     }
     s->spl = st == SP_LAP_GENERATED || prm.scheme != SP_SCHEME_FD ? 1
              : dims == 3 ? steps_per_launch_3d(prm.dtype, model, (int)nx, prm.steps_per_launch)
-                         : steps_per_launch(2, prm.dtype, model, stencil_radius(st), nx, ny, s->n_sm, prm.steps_per_launch);
+                         : steps_per_launch(2, prm.dtype, model, st, nx, ny, s->n_sm, prm.steps_per_launch);
     const size_t bytes = s->N * s->esize;
     for (int l = 0; l < 2; ++l)
         for (int f = 0; f < s->nf; ++f) {
@@ -646,6 +646,11 @@ extern "C" int sp_step(sp_sim *s, int64_t nsteps, void *stream) {
             s->cur ^= 1;  // one launch swaps the levels, however many steps it fuses
             s->steps += s->spl;
             nsteps -= s->spl;
+        } else if (nsteps >= 2 && s->spl == 4 && s->steps > 0) {  // two of the rest in one launch
+            SP_CUDA(launch_one_step(s, st, 2));
+            s->cur ^= 1;
+            s->steps += 2;
+            nsteps -= 2;
         } else {
             SP_CUDA(launch_one_step(s, st));
             s->cur ^= 1;

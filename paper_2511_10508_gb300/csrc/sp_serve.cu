@@ -355,7 +355,7 @@ static cudaError_t capture_quantum(sp_server *S, int Q) {
 // `steps` steps of one large grid from the level `parity` on; on return `parity` is the
 // current level.  One launch takes the library's default number of steps.
 static cudaError_t own_steps(const sp_server *S, const Req *q, int &parity, int steps, cudaStream_t s) {
-    const int spl = q->r.dims == 3 ? 1 : steps_per_launch(2, q->r.params.dtype, q->r.model, q->stencil == SP_LAP_9CROSS4 ? 2 : 1, q->nx, q->ny, S->n_sm, 0);
+    const int spl = q->r.dims == 3 ? 1 : steps_per_launch(2, q->r.params.dtype, q->r.model, q->stencil, q->nx, q->ny, S->n_sm, 0);
     StepArgs a;
     a.nx = q->nx;
     a.ny = q->ny;
@@ -363,7 +363,7 @@ static cudaError_t own_steps(const sp_server *S, const Req *q, int &parity, int 
     a.k = q->k;
     a.kf = to_float(q->k);
     for (int j = 0; j < steps;) {
-        const int k = steps - j >= spl ? spl : 1, f1 = q->nf > 1 ? 1 : 0;
+        const int left = steps - j, k = left >= spl ? spl : left >= 2 && spl == 4 ? 2 : 1, f1 = q->nf > 1 ? 1 : 0;
         a.in0 = q->buf[parity][0];
         a.in1 = q->buf[parity][f1];
         a.out0 = q->buf[parity ^ 1][0];

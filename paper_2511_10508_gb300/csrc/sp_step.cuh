@@ -576,6 +576,60 @@ __global__ void __launch_bounds__(NT) step3d_box_kernel(StepArgs a) {
                                         blockIdx.x * BX, blockIdx.y * BY, blockIdx.z * BZ, smem_raw);
 }
 
+struct NoRow {  // stands for RaggedRow where rows are aligned
+    __device__ __forceinline__ NoRow(int, int, int, bool) {}
+};
+
+// whether rows of nx 4-byte cells and the given fields are 8-byte aligned
+__device__ __forceinline__ bool pair_rows(int nx, const void *a, const void *b, const void *c, const void *d) {
+    return nx % 2 == 0 && (((uintptr_t)a | (uintptr_t)b | (uintptr_t)c | (uintptr_t)d) & 7) == 0;
+}
+
+// A row of LN lanes (lane l holds cells 4 l .. 4 l + 3; the first and the last lane are halo)
+// of a grid whose rows are not 16-byte aligned: copied in and written out element by
+// element, or pair by pair where rows are 8-byte aligned (PAIR), consecutive lanes
+// consecutive cells.  left: column of cell 0, a multiple of 4.  Model C 250 x 198 x 301 74.0 us
+// per step by elements, 70.9 by pairs; Cahn-Hilliard 255 x 253 rows of 257 76.5, of 258 64.8.
+template <int LN> struct RaggedRow {
+    int left, lane, cw[4];
+    bool pair;
+    __device__ __forceinline__ RaggedRow(int left_, int lane_, int nx, bool pair_) : left(left_), lane(lane_), pair(pair_) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) cw[q] = wrap_idx(pair ? left + 2 * (lane + LN * (q & 1)) : left + lane + LN * q, nx);
+    }
+    // row: the grid row's first element; dst: cell 0 in shared memory
+    template <typename T> __device__ __forceinline__ void fetch(T *dst, const T *row) const {
+        if (pair) {
+#pragma unroll
+            for (int q = 0; q < 2; ++q) cp_async8(dst + 2 * (lane + LN * q), row + cw[q]);
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) cp_async_elem(dst + lane + LN * q, row + cw[q]);
+        }
+    }
+    // this lane's 4 outputs, through 16 LN bytes of shared memory (every lane of the warp
+    // calls; on: whether the row is written)
+    __device__ __forceinline__ void put(float *row, float *stage, const float (&o)[4], int nx, bool on) const {
+        __syncwarp();  // the previous row has left the buffer
+        store_vec<float, 4>(stage + 4 * lane, o);
+        __syncwarp();
+        if (pair) {
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int e = 2 * (lane + LN * q);
+                if (on && e >= 4 && e < 4 * LN - 4 && left + e < nx)
+                    *reinterpret_cast<float2 *>(row + left + e) = *reinterpret_cast<const float2 *>(stage + e);
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int e = lane + LN * q;
+                if (on && e >= 4 && e < 4 * LN - 4 && left + e < nx) row[left + e] = stage[e];
+            }
+        }
+    }
+};
+
 // ===================================================== 2D, warp rows ==
 //
 // FP32 / BF16-storage 2D kernel without shared memory or barriers.  A warp
@@ -595,8 +649,8 @@ __global__ void __launch_bounds__(NT) step3d_box_kernel(StepArgs a) {
 // vector, wrapped or not, is aligned.  Otherwise (FP32) a warp copies its row of 32 V
 // cells element by element, consecutive lanes consecutive cells, and its outputs reach
 // global memory the same way through 512 bytes of shared memory: 1503 x 1001
-// Cahn-Hilliard 4th order 10.6 us per step in tiles, 6.8 now; 4097 x 4095 5-point 53.7 ->
-// 30.2 (aligned 4096^2: 23.2).
+// Cahn-Hilliard 4th order 10.6 us per step in tiles, 6.2 now; 4097 x 4095 5-point 53.7 ->
+// 27.1 (aligned 4096^2: 20.4).
 template <int MODEL, int ST, typename T>
 struct Step2dWarpShape {
     typedef typename Cmp<T>::type C;
@@ -621,7 +675,10 @@ __global__ void __launch_bounds__(NT) step2d_warp_kernel(StepArgs a, int strips,
     constexpr int r = Sh::r, V = Sh::V, RIN = Sh::RIN, NF = Sh::NF, U = Sh::U, XW = Sh::XW, D = Sh::D;
     constexpr unsigned FULL = 0xffffffffu;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    W *ring = reinterpret_cast<W *>(smem_raw) + (threadIdx.x >> 5) * (Sh::warp_smem(AL) / 16);  // [D][NF][32]
+    // (broadcast, so that the strip is known to be the same for the whole warp: fewer registers,
+    // Cahn-Hilliard 4096^2 23.0 -> 20.4 us per step)
+    const int wpc = blockDim.x >> 5, warp = __shfl_sync(FULL, threadIdx.x >> 5, 0);
+    W *ring = reinterpret_cast<W *>(smem_raw) + warp * (Sh::warp_smem(AL) / 16);  // [D][NF][32]
     T *stage = reinterpret_cast<T *>(ring + (size_t)D * NF * 32);                              // [NF][32 V] (not AL)
     (void)stage;
 
@@ -633,7 +690,6 @@ __global__ void __launch_bounds__(NT) step2d_warp_kernel(StepArgs a, int strips,
     // CTA reads contiguous spans of each row and the strips' overlapping halo
     // columns are shared through the caches.  CTAs own equal shares of the
     // flattened (group, row) space.
-    const int wpc = blockDim.x >> 5, warp = threadIdx.x >> 5;
     const T *in[2] = {static_cast<const T *>(a.in0), static_cast<const T *>(a.in1)};
     T *out[2] = {static_cast<T *>(a.out0), static_cast<T *>(a.out1)};
 
@@ -789,6 +845,193 @@ __global__ void __launch_bounds__(NT) step2d_warp_kernel(StepArgs a, int strips,
             }
         }
         cp_async_wait<0>();  // the ring is reused by the next segment
+    }
+}
+
+// K steps per launch on warp rows: the register windows of step2d_warp_kernel once per
+// step.  A row enters the windows of step 0; the row that step s completes, r (2 r for
+// Cahn-Hilliard) rows behind, enters those of step s + 1, extended by the neighbouring
+// lanes' cells; only the last step's rows reach memory.  Every step spoils one more halo
+// width of a strip's halo lane, so K halos must fit one lane's vector.  Intermediate rows
+// are rounded as a store would round them: bit for bit K single steps.  What bounds it is
+// instruction issue (K steps of it) or one read and one write per K steps, not shared
+// memory as on tiles, which keep every step's taps there.
+// Per step, tiles and now: Gray-Scott 16384^2 491 us (two steps per launch, the better of the
+// tiles) -> 216 (four; 5.0 TB/s), 8192^2 126 -> 51, 2048^2 9.3 -> 5.8; Allen-Cahn 8192^2 71 -> 30;
+// Cahn-Hilliard 8192^2 101 (one step per launch) -> 57; Model C 4096^2 35 -> 17.
+template <int MODEL, int ST, typename T, int K>
+struct Step2dWarpTbShape {
+    typedef typename Cmp<T>::type C;
+    static constexpr int r = StencilInfo<ST>::r, V = 16 / (int)sizeof(T), RIN = (MODEL == CH) ? 2 * r : r;
+    static constexpr int NF = num_fields<MODEL>(), U = 2 * r + 1, XW = V + 2 * r, OUT_COLS = 30 * V, D = 8;
+    static constexpr int LAG = K * RIN;  // rows the last step trails the loads by
+    static constexpr bool fits = LAG <= V;
+    static constexpr int NT = 64;
+    __host__ __device__ static constexpr size_t warp_smem(bool al) { return (size_t)(D * NF + (al ? 0 : 1)) * 32 * 16; }
+};
+
+template <int MODEL, int ST, typename T, int K, bool AL>
+__global__ void __launch_bounds__(Step2dWarpTbShape<MODEL, ST, T, K>::NT)
+    step2d_warptb_kernel(StepArgs a, int strips, int groups, long long rows_per_cta) {
+    pdl_enter();
+    typedef Step2dWarpTbShape<MODEL, ST, T, K> Sh;
+    typedef typename Sh::C C;
+    typedef uint4 W;
+    constexpr int r = Sh::r, V = Sh::V, NF = Sh::NF, U = Sh::U, XW = Sh::XW, D = Sh::D, LAG = Sh::LAG;
+    constexpr unsigned FULL = 0xffffffffu;
+    static_assert(Sh::fits, "the halo lanes must cover K steps' halos");
+    const ConstsC<C> k(a.k, a.kf);
+    const ConstsF2 k2(k);
+    (void)k2;
+    const int nx = a.nx, ny = a.ny;
+    const int lane = threadIdx.x & 31;
+    // (broadcast, so that the strip is known to be the same for the whole warp: fewer registers)
+    const int wpc = blockDim.x >> 5, warp = __shfl_sync(FULL, threadIdx.x >> 5, 0);
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    W *ring = reinterpret_cast<W *>(smem_raw) + warp * (Sh::warp_smem(AL) / 16);  // [D][NF][32]
+    float *stage = reinterpret_cast<float *>(ring + (size_t)D * NF * 32);                      // [32 V] (not AL)
+    (void)stage;
+    const T *in[2] = {static_cast<const T *>(a.in0), static_cast<const T *>(a.in1)};
+    T *out[2] = {static_cast<T *>(a.out0), static_cast<T *>(a.out1)};
+    const bool pair = !AL && pair_rows(nx, in[0], in[NF - 1], out[0], out[NF - 1]);
+
+    // equal shares of the flattened (strip group, row) space, as in step2d_warp_kernel
+    long long g0 = (long long)blockIdx.x * rows_per_cta;
+    const long long gend = min(g0 + rows_per_cta, (long long)groups * ny);
+    while (g0 < gend) {
+        const int group = (int)(g0 / ny);
+        const int y0 = (int)(g0 - (long long)group * ny);
+        const int y1 = (int)min((long long)ny, (long long)y0 + (gend - g0));
+        g0 += y1 - y0;
+        const int strip = group * wpc + warp;
+        if (strip >= strips) continue;
+        const int col = strip * Sh::OUT_COLS + (lane - 1) * V;
+        const int colw = wrap_idx(col, nx);
+        const bool store = lane >= 1 && lane <= 30 && col < nx;
+        const typename std::conditional<AL, NoRow, RaggedRow<32>>::type rag(strip * Sh::OUT_COLS - V, lane, nx, pair);
+        const int jbeg = y0 - LAG;
+        const int n = (y1 - y0) + 2 * LAG;
+
+        auto issue = [&](int i) {
+            if (i < n) {
+                const size_t row = (size_t)wrap_idx(jbeg + i, ny) * nx;
+#pragma unroll
+                for (int f = 0; f < NF; ++f) {
+                    W *dst = &ring[((i % D) * NF + f) * 32];
+                    if constexpr (AL) {
+                        cp_async16(dst + lane, in[f] + row + colw);
+                    } else {
+                        rag.fetch(reinterpret_cast<T *>(dst), in[f] + row);
+                    }
+                }
+            }
+            cp_async_commit();  // empty groups keep the count uniform
+        };
+#pragma unroll
+        for (int s = 0; s < D - 1; ++s) issue(s);
+
+        C ph[K][NF][U][XW] = {};  // the last U rows step s reads, newest in slot u
+        C mu[MODEL == CH ? K : 1][U][XW] = {};
+        (void)mu;
+        auto extend = [&](C (&row)[XW]) {
+#pragma unroll
+            for (int h = 0; h < r; ++h) {
+                row[h] = __shfl_up_sync(FULL, row[V + h], 1);
+                row[r + V + h] = __shfl_down_sync(FULL, row[r + h], 1);
+            }
+        };
+        for (int i0 = 0; i0 < n; i0 += U) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int i = i0 + u;
+                if (i < n) {
+                    // row i of the segment; the slot read in the previous iteration is refilled
+                    if constexpr (!AL) __syncwarp();  // every lane has read it
+                    issue(i + D - 1);
+                    cp_async_wait<D - 1>();
+                    if constexpr (!AL) __syncwarp();  // every lane's cells have landed
+#pragma unroll
+                    for (int f = 0; f < NF; ++f) {
+                        union { W w; T t[V]; } raw;
+                        raw.w = ring[((i % D) * NF + f) * 32 + lane];
+#pragma unroll
+                        for (int c = 0; c < V; ++c) ph[0][f][u][r + c] = to_c(raw.t[c]);
+                        extend(ph[0][f][u]);
+                    }
+                    // window slot of the row `m` iterations back
+#define SLOT(m) ((u - (m) + 4 * U) % U)
+                    C o[2][V];
+#pragma unroll
+                    for (int s = 0; s < K; ++s) {
+                        auto P0 = [&](int dx, int dy, int c) -> C { return ph[s][0][SLOT(r - dy)][r + c + dx]; };
+                        auto P1 = [&](int dx, int dy, int c) -> C { return ph[s][NF - 1][SLOT(r - dy)][r + c + dx]; };
+                        (void)P1;
+                        if constexpr (MODEL == CH) {
+                            auto Pm = [&](int dx, int dy, int c) -> C { return mu[s][SLOT(r - dy)][r + c + dx]; };
+#pragma unroll
+                            for (int c = 0; c < V; c += 2) {
+                                const float2 m2 = ch_mu2(make_float2(P0(0, 0, c), P0(0, 0, c + 1)), stencil_sum2_2d<ST>(P0, c), k2);
+                                mu[s][u][r + c] = m2.x;
+                                mu[s][u][r + c + 1] = m2.y;
+                            }
+                            extend(mu[s][u]);
+#pragma unroll
+                            for (int c = 0; c < V; c += 2) {
+                                const C *p = &ph[s][0][SLOT(2 * r)][r + c];
+                                const float2 o2 = ch_update2(make_float2(p[0], p[1]), stencil_sum2_2d<ST>(Pm, c), k2);
+                                o[0][c] = o2.x;
+                                o[0][c + 1] = o2.y;
+                            }
+                        } else if constexpr (MODEL == AC || MODEL == GS) {
+                            // two cells per instruction
+#pragma unroll
+                            for (int c = 0; c < V; c += 2) {
+                                const float2 p0 = make_float2(P0(0, 0, c), P0(0, 0, c + 1));
+                                const float2 S0 = stencil_sum2_2d<ST>(P0, c);
+                                float2 a0, a1 = make_float2(0.0f, 0.0f);
+                                if constexpr (MODEL == AC) a0 = ac_update2(p0, S0, k2);
+                                else gs_update2(p0, make_float2(P1(0, 0, c), P1(0, 0, c + 1)), S0,
+                                                stencil_sum2_2d<ST>(P1, c), k2, a0, a1);
+                                o[0][c] = a0.x;
+                                o[0][c + 1] = a0.y;
+                                o[1][c] = a1.x;
+                                o[1][c + 1] = a1.y;
+                            }
+                        } else {
+#pragma unroll
+                            for (int c = 0; c < V; ++c) {
+                                auto Q0 = [&](int dx, int dy, int) -> C { return P0(dx, dy, c); };
+                                auto Q1 = [&](int dx, int dy, int) -> C { return P1(dx, dy, c); };
+                                two_field_update<MODEL, C>(P0(0, 0, c), P1(0, 0, c), stencil_sum<ST, C>(Q0),
+                                                           second_sum<MODEL, ST, C>(Q0, Q1, k), k, o[0][c], o[1][c]);
+                            }
+                        }
+                        if (s + 1 < K) {
+#pragma unroll
+                            for (int f = 0; f < NF; ++f) {
+#pragma unroll
+                                for (int c = 0; c < V; ++c) ph[s + 1][f][u][r + c] = to_c(from_c<T>(o[f][c]));
+                                extend(ph[s + 1][f][u]);
+                            }
+                        }
+                    }
+#undef SLOT
+                    if (i >= 2 * LAG) {
+                        const size_t row = (size_t)(jbeg + i - LAG) * nx;
+#pragma unroll
+                        for (int f = 0; f < NF; ++f) {
+                            if constexpr (AL) {
+                                if (store) store_vec<T, V>(out[f] + row + col, o[f]);
+                            } else {
+                                rag.put(out[f] + row, stage, o[f], nx, true);
+                            }
+                        }
+                    }
+                }
+            }
+        }
+        cp_async_wait<0>();  // the ring is reused by the next segment
+        if constexpr (!AL) __syncwarp();
     }
 }
 
@@ -1417,60 +1660,6 @@ __global__ void __launch_bounds__(8 * TY_, 64 / TY_)
         __syncthreads();  // the ring is reused by the next tile
     }
 }
-
-struct NoRow {  // stands for RaggedRow where rows are aligned
-    __device__ __forceinline__ NoRow(int, int, int, bool) {}
-};
-
-// whether rows of nx 4-byte cells and the given fields are 8-byte aligned
-__device__ __forceinline__ bool pair_rows(int nx, const void *a, const void *b, const void *c, const void *d) {
-    return nx % 2 == 0 && (((uintptr_t)a | (uintptr_t)b | (uintptr_t)c | (uintptr_t)d) & 7) == 0;
-}
-
-// A row of LN lanes (lane l holds cells 4 l .. 4 l + 3; the first and the last lane are halo)
-// of a grid whose rows are not 16-byte aligned: copied in and written out element by
-// element, or pair by pair where rows are 8-byte aligned (PAIR), consecutive lanes
-// consecutive cells.  left: column of cell 0, a multiple of 4.  Model C 250 x 198 x 301 74.0 us
-// per step by elements, 70.9 by pairs; Cahn-Hilliard 255 x 253 rows of 257 76.5, of 258 64.8.
-template <int LN> struct RaggedRow {
-    int left, lane, cw[4];
-    bool pair;
-    __device__ __forceinline__ RaggedRow(int left_, int lane_, int nx, bool pair_) : left(left_), lane(lane_), pair(pair_) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) cw[q] = wrap_idx(pair ? left + 2 * (lane + LN * (q & 1)) : left + lane + LN * q, nx);
-    }
-    // row: the grid row's first element; dst: cell 0 in shared memory
-    template <typename T> __device__ __forceinline__ void fetch(T *dst, const T *row) const {
-        if (pair) {
-#pragma unroll
-            for (int q = 0; q < 2; ++q) cp_async8(dst + 2 * (lane + LN * q), row + cw[q]);
-        } else {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) cp_async_elem(dst + lane + LN * q, row + cw[q]);
-        }
-    }
-    // this lane's 4 outputs, through 16 LN bytes of shared memory (every lane of the warp
-    // calls; on: whether the row is written)
-    __device__ __forceinline__ void put(float *row, float *stage, const float (&o)[4], int nx, bool on) const {
-        __syncwarp();  // the previous row has left the buffer
-        store_vec<float, 4>(stage + 4 * lane, o);
-        __syncwarp();
-        if (pair) {
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                const int e = 2 * (lane + LN * q);
-                if (on && e >= 4 && e < 4 * LN - 4 && left + e < nx)
-                    *reinterpret_cast<float2 *>(row + left + e) = *reinterpret_cast<const float2 *>(stage + e);
-            }
-        } else {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int e = lane + LN * q;
-                if (on && e >= 4 && e < 4 * LN - 4 && left + e < nx) row[left + e] = stage[e];
-            }
-        }
-    }
-};
 
 // ===================================================== 3D, warp rows ==
 //

@@ -33,27 +33,6 @@ inline bool small_tile(int nx, int ny, int TX, int TY, double margin) {
 
 constexpr size_t kMaxSmemPerCta = 227 * 1024;  // opt-in maximum of dynamic shared memory per CTA
 
-// Rows per CTA of the 2D warp-strip kernel, whose CTAs own equal runs of the flattened
-// (strip group, row) space: p rows cost p + halo, q CTAs of `load` (their share of 8
-// warps) on the fullest SM take about q load + latency of them (see planes_per_cta).
-// Runs of at least 32 rows left most SMs idle on small grids: 444 x 568 Cahn-Hilliard 9.2
-// us per step, 3.0 now; 1504 x 1000 4th order 13.2 -> 6.2 (runs of 8 rows; of 4: 7.5).
-inline long long rows_per_cta(long long total, int halo, double load, double latency, int occ, int n_sm) {
-    const long long wave = (long long)n_sm * std::max(occ, 1), p0 = (total + wave - 1) / wave;
-    long long best = p0;
-    double best_cost = 0;
-    for (long long p = p0; p <= std::min(total, 8 * p0 + 32); ++p) {
-        const long long ctas = (total + p - 1) / p, q = (ctas + n_sm - 1) / n_sm;
-        const double cost = (q * load + latency) * (p + halo);
-        if (p == p0 || cost < best_cost * 0.999) {
-            best = p;
-            best_cost = cost;
-        }
-        if (q == 1) break;
-    }
-    return best;
-}
-
 // Planes per CTA of a persistent 3D kernel whose CTAs own equal contiguous runs of
 // the flattened (tile, z) space; at most one resident wave (n_sm x occ CTAs).  A run
 // of p planes costs p + halo planes, halo standing for the planes it only warms its
@@ -235,19 +214,12 @@ cudaError_t launch_warp2d(const StepArgs &a, cudaStream_t s, int n_sm) {
     typedef Step2dWarpShape<MODEL, ST, T> WS;
     constexpr int NT = 256;
     auto kern = step2d_warp_kernel<MODEL, ST, T, NT, AL>;
-    static const bool attr = [&] {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(WS::warp_smem(AL) * (NT / 32)));
-        return true;
-    }();
-    (void)attr;
+    static const auto occ = warp_occupancy<NT / 32>(kern, WS::warp_smem(AL));
     const int strips = (a.nx + WS::OUT_COLS - 1) / WS::OUT_COLS;
-    const int wpc = std::min(NT / 32, strips);
+    const int wpc = warps_per_cta(strips, NT / 32), groups = (strips + wpc - 1) / wpc;
     const size_t smem = WS::warp_smem(AL) * wpc;
-    int occ = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 32 * wpc, smem);
-    const int groups = (strips + wpc - 1) / wpc;
     const long long total = (long long)groups * a.ny;
-    const long long rows = rows_per_cta(total, 2 * WS::RIN, wpc / 8.0, AL ? 1.0 : 4.0, occ, n_sm);
+    const long long rows = rows_per_cta(total, 2 * WS::RIN, wpc / 8.0, AL ? 1.0 : 4.0, occ[wpc], n_sm);
     const long long ctas = (total + rows - 1) / rows;
     return launch_pdl(kern, dim3((unsigned)ctas), dim3(32 * wpc), smem, s, a, strips, groups, rows);
 }
@@ -255,6 +227,12 @@ cudaError_t launch_warp2d(const StepArgs &a, cudaStream_t s, int n_sm) {
 template <int MODEL, int ST, typename T>
 cudaError_t launch_step_t(const StepArgs &a, cudaStream_t s, int n_sm, int k) {
     if constexpr (StencilInfo<ST>::dims == 2) {
+        if constexpr (sizeof(T) == 4) {
+            if (k > 1) {
+                const cudaError_t e = launch_w2d(MODEL, ST, a, s, n_sm, k);
+                if (e != cudaErrorNotSupported) return e;
+            }
+        }
         if (k == 4) return launch_tb<MODEL, ST, T, 4>(a, s);
         if (k == 2) return launch_tb<MODEL, ST, T, 2>(a, s);
     }
