@@ -11,14 +11,16 @@
 // P_j = ((f(+j e_x) + f(-j e_x)) + (f(+j e_y) + f(-j e_y))) [+ (z pair)], in the
 // fixed order  acc = w_r P_r; acc = fma(w_j, P_j, acc) for j = r-1..1;
 // S = fma(d w_0, f_0, acc).  2D FP32 / BF16 grids use shared-memory tiles (one
-// pass, mu in shared memory); FP64 (bound by the FP64 pipe, where the halo mu
-// of a tile would cost more than it saves) and 3D grids use per-point kernels
-// (a block per 256-point row segment, tap offsets computed once per segment;
-// Cahn-Hilliard takes two passes through a mu buffer).
+// pass, mu in shared memory) or, FP32, warp rows (sp_gen2d.cu); 3D FP32 / BF16
+// grids plane rings; FP64 (bound by the FP64 pipe, where the halo mu of a tile
+// would cost more than it saves) per-point kernels (a block per 256-point row
+// segment, tap offsets computed once per segment; Cahn-Hilliard takes two passes
+// through a mu buffer).
 #include <cstdint>
 #include <cstdlib>
 #include <type_traits>
 
+#include "sp_gen.cuh"
 #include "sp_internal.h"
 #include "sp_step.cuh"
 
@@ -107,11 +109,6 @@ int generated_weights(int order, int dims, double *wk, double *lambda_max) {
 
 // -------------------------------------------------------------- kernels --
 
-struct GenW {
-    double w[kMaxGenRadius + 1];  // d w_0, w_1, ..., w_r
-    float wf[kMaxGenRadius + 1];
-};
-
 template <int R>
 struct GenTaps {
     size_t zb[2 * R + 1], yb[2 * R + 1];
@@ -143,12 +140,6 @@ __device__ __forceinline__ C gen_sum(const Acc &P, const GenW &W) {
     }
     return FMA(gw<C>(W, 0), P(0, 0, 0), acc);
 }
-
-struct GenArgs {
-    StepArgs a;
-    GenW W;
-    void *mu;
-};
 
 __device__ __forceinline__ void gen_seg(long long u, int segs, const StepArgs &a, int &x, int &y, int &z,
                                         size_t &row) {
@@ -647,6 +638,10 @@ static cudaError_t launch_gen_t(const GenArgs &g, cudaStream_t s, int n_sm) {
     if constexpr (DIMS == 2 && !std::is_same<T, double>::value) {
         // family 0: shared-memory tiles; family 1: the per-point kernels
         if (g_step_variant != 1) {
+            if constexpr (sizeof(T) == 4) {
+                const cudaError_t e = launch_gen2d_f32(MODEL, R, g, s, n_sm);
+                if (e != cudaErrorNotSupported) return e;
+            }
             // Cahn-Hilliard: 288 threads take the (BY + 2R) / 5 x (BX + 8) / 4 mu blocks
             // (up to 272) in one round and the 8 x 32 output blocks; 256 otherwise
             constexpr int BX = 128, BY = 32, NT = MODEL == CH ? 288 : 256;

@@ -585,12 +585,12 @@ __device__ __forceinline__ bool pair_rows(int nx, const void *a, const void *b, 
     return nx % 2 == 0 && (((uintptr_t)a | (uintptr_t)b | (uintptr_t)c | (uintptr_t)d) & 7) == 0;
 }
 
-// A row of LN lanes (lane l holds cells 4 l .. 4 l + 3; the first and the last lane are halo)
+// A row of LN lanes (lane l holds cells 4 l .. 4 l + 3; the first and the last HL lanes are halo)
 // of a grid whose rows are not 16-byte aligned: copied in and written out element by
 // element, or pair by pair where rows are 8-byte aligned (PAIR), consecutive lanes
 // consecutive cells.  left: column of cell 0, a multiple of 4.  Model C 250 x 198 x 301 74.0 us
 // per step by elements, 70.9 by pairs; Cahn-Hilliard 255 x 253 rows of 257 76.5, of 258 64.8.
-template <int LN> struct RaggedRow {
+template <int LN, int HL = 1> struct RaggedRow {
     int left, lane, cw[4];
     bool pair;
     __device__ __forceinline__ RaggedRow(int left_, int lane_, int nx, bool pair_) : left(left_), lane(lane_), pair(pair_) {
@@ -617,14 +617,14 @@ template <int LN> struct RaggedRow {
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
                 const int e = 2 * (lane + LN * q);
-                if (on && e >= 4 && e < 4 * LN - 4 && left + e < nx)
+                if (on && e >= 4 * HL && e < 4 * (LN - HL) && left + e < nx)
                     *reinterpret_cast<float2 *>(row + left + e) = *reinterpret_cast<const float2 *>(stage + e);
             }
         } else {
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int e = lane + LN * q;
-                if (on && e >= 4 && e < 4 * LN - 4 && left + e < nx) row[left + e] = stage[e];
+                if (on && e >= 4 * HL && e < 4 * (LN - HL) && left + e < nx) row[left + e] = stage[e];
             }
         }
     }

@@ -8,25 +8,6 @@
 
 namespace sp {
 
-// Rows per CTA (one warp on grids of few strips, whose last CTA would be half empty, else
-// two on adjacent strips): p rows cost p + halo iterations, each the issue time of the warps that
-// share a scheduler of the fullest SM, at least that of five (a warp's own chain of K steps).
-inline long long warptb_rows(long long total, int halo, int wpc, int occ, int n_sm) {
-    const long long wave = (long long)n_sm * occ, p0 = (total + wave - 1) / wave;
-    long long best = p0;
-    double best_cost = 0;
-    for (long long p = p0; p <= std::min(total, 8 * p0 + 32); ++p) {
-        const long long ctas = (total + p - 1) / p, q = (ctas + n_sm - 1) / n_sm;
-        const double cost = std::max(5.0, q * wpc / 4.0) * (p + halo);
-        if (p == p0 || cost < best_cost * 0.999) {
-            best = p;
-            best_cost = cost;
-        }
-        if (q == 1) break;
-    }
-    return best;
-}
-
 template <int MODEL, int ST, int K, bool AL>
 cudaError_t launch_warptb(const StepArgs &a, cudaStream_t s, int n_sm) {
     typedef Step2dWarpTbShape<MODEL, ST, float, K> Sh;
