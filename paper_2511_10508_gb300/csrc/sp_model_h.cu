@@ -387,7 +387,7 @@ __global__ void __launch_bounds__(MhRows3dShape<ST, T, TY, LN>::NT)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const ConstsC<float> k(a.k, a.kf);
     const int nx = a.nx, ny = a.ny, nz = a.nz;
-    const int lane = threadIdx.x & (LN - 1), w = threadIdx.x / LN;
+    const int lane = threadIdx.x & (LN - 1), w = LN == 32 ? __shfl_sync(0xffffffffu, threadIdx.x / 32, 0) : threadIdx.x / LN;
     const size_t plane = (size_t)nx * (size_t)ny;
     constexpr size_t PL = (size_t)HIN * LN;  // chunks of a plane
     W *const m_own = reinterpret_cast<W *>(smem_raw) + (size_t)w * LN + lane;
