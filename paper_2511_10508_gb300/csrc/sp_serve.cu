@@ -169,6 +169,12 @@ double now_s(std::chrono::steady_clock::time_point t0) {
     return std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
 }
 
+// elements left uninitialised by resize(): a result is written once, by the copy from the device
+struct Uninit : std::allocator<double> {
+    template <typename U> struct rebind { typedef Uninit other; };
+    template <typename U> void construct(U *p) noexcept { ::new ((void *)p) U; }
+};
+
 struct Req {
     uint64_t ticket = 0;
     sp_request r{};
@@ -184,7 +190,7 @@ struct Req {
     int status = SP_PENDING;
     bool done = false;
     double mass = 0;
-    std::vector<double> host;  // FP64 fields, field 0 then field 1
+    std::vector<double, Uninit> host;  // FP64 fields, field 0 then field 1
 };
 
 }  // namespace
