@@ -140,9 +140,11 @@ typedef struct sp_params {
     int gs_patches;        /* Gray-Scott: number of seeded patches */
     int gs_patch;          /* Gray-Scott: patch side (points) */
     int steps_per_launch;  /* time steps fused per kernel launch (temporal blocking:
-                              2D grids 2 or 4; 3D FP32 / BF16 Allen-Cahn and
-                              Gray-Scott with nx a multiple of 4: 2); 0 = the
-                              library's choice, 1 = none */
+                              2D grids 2 or 4; 3D FP32 / BF16 Allen-Cahn,
+                              Gray-Scott and Model C with nx a multiple of 4: 2);
+                              0 = the library's choice (2D FP32: 4 or 2, 1 for
+                              most Cahn-Hilliard grids; small 2D FP64 grids: 2
+                              or 1; else 1), 1 = none */
     int scheme;            /* sp_scheme (default SP_SCHEME_FD) */
     int stencil_order;     /* accuracy order of SP_LAP_GENERATED (even, 2..8; default 2) */
     int flags;             /* SP_FLAG_* bits; other bits must be 0 */

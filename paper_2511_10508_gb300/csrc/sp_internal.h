@@ -28,20 +28,11 @@ struct ReduceGeom {
 
 // Step launchers, one per storage type (sp_step_f64.cu, sp_step_f32.cu,
 // sp_step_bf16.cu).  k forward-Euler steps from a.in* to a.out* in one launch;
-// k must be 1, or the value of steps_per_launch() for this model/stencil/dtype.
+// k: 1, or 2 or 4 (2D) or 2 (3D FP32 / BF16, see steps_per_launch_3d).
 cudaError_t launch_step_f64(int model, int stencil, const StepArgs &a, cudaStream_t s, int n_sm, int k);
 cudaError_t launch_step_f32(int model, int stencil, const StepArgs &a, cudaStream_t s, int n_sm, int k);
 cudaError_t launch_step_bf16(int model, int stencil, const StepArgs &a, cudaStream_t s, int n_sm, int k);
 
-// Steps fused per launch (temporal blocking) for a request of `requested`
-// (0 = the library's choice, 1 = none): 2D grids support 2 and 4 (FP64 on small
-// tiles, where a launch is short enough for its fixed cost to matter); 3D grids
-// see steps_per_launch_3d.  The library's choice follows measurement on GB300:
-// blocking pays where the one-step tile kernel is at the HBM bound (FP32
-// Gray-Scott 32768^2: 1 step 0.99 of the copy bandwidth, 2 steps 1.31
-// effective, 4 steps 1.19); Cahn-Hilliard and BF16 storage are limited by
-// on-chip work and FP64 by the FP64 pipe, so there extra halo work only slows
-// large grids (the autotuner tries it on small FP64 grids).
 // Kernel variant chosen per launch: 0 = the default for the grid, 1 (and 2) =
 // alternative families (2D FP64: small tiles instead of strips, or strips instead
 // of small tiles for grids up to 1024^2, and 2 / 4 = strips of 64 threads / of
@@ -164,6 +155,10 @@ inline int steps_per_launch_3d(int dtype, int model, int nx, int requested) {
     return (ok && requested >= 2) ? 2 : 1;
 }
 
+// Steps fused per launch (temporal blocking) for a request of `requested`
+// (0 = the library's choice, 1 = none): 2D grids support 2 and 4 (FP64 on small
+// tiles, where a launch is short enough for its fixed cost to matter); 3D grids
+// see steps_per_launch_3d.
 // 2D FP32 grids fuse steps by default where warp rows do (sp_w2d.cuh; us per step with 1, 2 and 4):
 // Allen-Cahn, Gray-Scott and Model C four with a radius-1 stencil (Gray-Scott 300 x 301 2.2 / 2.2 /
 // 1.9, 2048^2 10.4 / 6.9 / 5.8, 16384^2 785 / 398 / 216).  A radius-2 stencil leaves room for two; four
