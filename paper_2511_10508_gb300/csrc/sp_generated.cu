@@ -664,14 +664,16 @@ static cudaError_t launch_gen_t(const GenArgs &g, cudaStream_t s, int n_sm) {
         if (al) return launch_gen_rows_model<MODEL, R, T, true>(g, s, n_sm);
         if constexpr (sizeof(T) == 4) return launch_gen_rows_model<MODEL, R, T, false>(g, s, n_sm);
     }
-    const int segs = (g.a.nx + 255) / 256;
-    const long long units = (long long)g.a.ny * g.a.nz * segs;
-    const unsigned blocks = (unsigned)std::min<long long>(units, (long long)n_sm * 8);
-    if constexpr (MODEL == CH) {
-        const cudaError_t e = launch_pdl(gen_mu_kernel<R, DIMS, T>, dim3(blocks), dim3(256), 0, s, g, segs);
-        if (e != cudaSuccess) return e;
+    if constexpr (DIMS == 2 || sizeof(T) != 4) {
+        const int segs = (g.a.nx + 255) / 256;
+        const long long units = (long long)g.a.ny * g.a.nz * segs;
+        const unsigned blocks = (unsigned)std::min<long long>(units, (long long)n_sm * 8);
+        if constexpr (MODEL == CH) {
+            const cudaError_t e = launch_pdl(gen_mu_kernel<R, DIMS, T>, dim3(blocks), dim3(256), 0, s, g, segs);
+            if (e != cudaSuccess) return e;
+        }
+        return launch_pdl(gen_step_kernel<MODEL, R, DIMS, T>, dim3(blocks), dim3(256), 0, s, g, segs);
     }
-    return launch_pdl(gen_step_kernel<MODEL, R, DIMS, T>, dim3(blocks), dim3(256), 0, s, g, segs);
 }
 
 template <int MODEL, typename T>
