@@ -273,11 +273,18 @@ int sp_field_devptr(sp_sim *sim, int field, void **dptr);
  * time each candidate launch configuration for this grid on `stream` (8 steps
  * each, twice; all candidates give bit-identical results, so these are ordinary
  * steps of the run) and keep the fastest.  A choice cached earlier in the
- * process for the same (model, stencil, dtype, dims, grid size class) is taken
- * without timing.  Blocks until the timing events complete.  *steps_taken
+ * process for the same (device, model, stencil, dtype, dims, row alignment, grid
+ * size class) is taken without timing, if it is available for this grid.  Blocks until the timing events complete.  *steps_taken
  * receives the number of time steps advanced (0 to 65).  Captured graphs of
  * another configuration are dropped. */
 int sp_autotune(sp_sim *sim, void *stream, int64_t *steps_taken);
+
+/* The autotuner's table, without device work: sp_tune_record enters a choice (one that
+ * sp_launch_config reported in an earlier run) for the class of a grid of the current
+ * device, SP_EINVAL if it is not a candidate of that grid; sp_tune_lookup gives the choice
+ * that sp_autotune would take for a grid without timing, or SP_ENOTFOUND. */
+int sp_tune_record(int model, int dims, const int64_t shape[3], const sp_params *p, int steps_per_launch, int variant);
+int sp_tune_lookup(int model, int dims, const int64_t shape[3], const sp_params *p, int *steps_per_launch, int *variant);
 
 /* Pin a launch configuration (for instance one that sp_autotune chose in an
  * earlier run): steps fused per launch (1, or 2 / 4 for 2D grids) and kernel

@@ -78,6 +78,9 @@ _SIGS = {
     "sp_field_devptr": (ctypes.c_int, [_vp, ctypes.c_int, _P(_vp)]),
     "sp_steps_taken": (ctypes.c_int, [_vp, _P(_i64)]),
     "sp_autotune": (ctypes.c_int, [_vp, _vp, _P(_i64)]),
+    "sp_tune_record": (ctypes.c_int, [ctypes.c_int, ctypes.c_int, _P(_i64), _P(sp_params), ctypes.c_int, ctypes.c_int]),
+    "sp_tune_lookup": (ctypes.c_int, [ctypes.c_int, ctypes.c_int, _P(_i64), _P(sp_params), _P(ctypes.c_int),
+                                      _P(ctypes.c_int)]),
     "sp_set_launch_config": (ctypes.c_int, [_vp, ctypes.c_int, ctypes.c_int]),
     "sp_stencil_weights": (ctypes.c_int, [ctypes.c_int, ctypes.c_int, _P(ctypes.c_double), _P(ctypes.c_double)]),
     "sp_launch_config": (ctypes.c_int, [_vp, _P(ctypes.c_int), _P(ctypes.c_int)]),

@@ -453,12 +453,20 @@ static cudaError_t launch_one_step_impl(sp_sim *s, cudaStream_t st, int k) {
 //
 // Candidates: (steps per launch, kernel family).  Every candidate computes the
 // same values bit for bit, so the timed steps are ordinary steps of the run.
-// The winner is cached per (model, stencil, dtype, dims, log2 of the grid size).
+// The winner is kept per (device, model, stencil, dtype, dims, row alignment, log2 of the
+// grid size), and another grid of that class takes it only if it is one of its own
+// candidates: two steps per pass and the tensor-map loads exist only for aligned rows.
 
+struct TuneGrid {
+    int device, model, stencil, dtype, dims, nx;
+    uint64_t N;
+    bool fd;  // finite differences
+};
 struct TuneKey {
-    int model, stencil, dtype, dims, size_log2;
+    int device, model, stencil, dtype, dims, align, size_log2;
     bool operator<(const TuneKey &o) const {
-        return std::tie(model, stencil, dtype, dims, size_log2) < std::tie(o.model, o.stencil, o.dtype, o.dims, o.size_log2);
+        return std::tie(device, model, stencil, dtype, dims, align, size_log2) <
+               std::tie(o.device, o.model, o.stencil, o.dtype, o.dims, o.align, o.size_log2);
     }
 };
 struct TuneChoice {
@@ -481,37 +489,41 @@ static void set_launch_config(sp_sim *s, TuneChoice c) {
     s->variant = c.variant;
 }
 
-static TuneKey tune_key(const sp_sim *s) {
-    int lg = 0;
-    while (lg < 62 && (1ull << (lg + 1)) <= s->N) ++lg;
-    return {s->model, s->stencil, s->dtype, s->dims, lg};
+static TuneGrid tune_grid(const sp_sim *s) {
+    return {s->device, s->model, s->stencil, s->dtype, s->dims, s->nx, s->N, s->spec == nullptr};
 }
 
-static std::vector<TuneChoice> tune_candidates(const sp_sim *s) {
+static TuneKey tune_key(const TuneGrid &g) {
+    int lg = 0;
+    while (lg < 62 && (1ull << (lg + 1)) <= g.N) ++lg;
+    return {g.device, g.model, g.stencil, g.dtype, g.dims, std::min(g.nx & -g.nx, 8), lg};
+}
+
+static std::vector<TuneChoice> tune_candidates(const TuneGrid &g) {
     std::vector<TuneChoice> c;
-    if (s->spec || s->model == SP_MODEL_H || s->stencil == SP_LAP_GENERATED) return {{1, 0}};
-    if (s->dims == 2 && s->dtype != SP_F64) {
+    if (!g.fd || g.model == SP_MODEL_H || g.stencil == SP_LAP_GENERATED) return {{1, 0}};
+    if (g.dims == 2 && g.dtype != SP_F64) {
         c.push_back({1, 1});
         for (int spl : {1, 2, 4}) c.push_back({spl, 0});
-    } else if (s->dims == 2 || s->stencil == SP_LAP_27 || s->dtype != SP_F64) {
+    } else if (g.dims == 2 || g.stencil == SP_LAP_27 || g.dtype != SP_F64) {
         c.push_back({1, 0});
         c.push_back({1, 1});
-        if (s->dims == 3 && s->dtype != SP_F64) c.push_back({1, 2});
-        if (s->dims == 3 && s->dtype != SP_F64 && s->model != SP_MODEL_C && s->nx % (int)(16 / s->esize) == 0 &&
+        if (g.dims == 3 && g.dtype != SP_F64) c.push_back({1, 2});
+        if (g.dims == 3 && g.dtype != SP_F64 && g.model != SP_MODEL_C && g.nx % (int)(16 / dtype_size(g.dtype)) == 0 &&
             tma_available())
             c.push_back({1, kTmaFamily});
-        if (planes27_applies(s->dims, s->dtype, s->stencil, s->model) && s->model != SP_MODEL_C)
+        if (planes27_applies(g.dims, g.dtype, g.stencil, g.model) && g.model != SP_MODEL_C)
             c.push_back({1, kZregFamily});
-        if (s->dims == 3 && steps_per_launch_3d(s->dtype, s->model, s->nx, 2) == 2) {
+        if (g.dims == 3 && steps_per_launch_3d(g.dtype, g.model, g.nx, 2) == 2) {
             c.push_back({2, 0});  // two steps per pass, 8 rows
             c.push_back({2, 1});  // 16 rows
-            if (s->model == SP_MODEL_C) {  // one step in the plane rings (else the box kernel)
+            if (g.model == SP_MODEL_C) {  // one step in the plane rings (else the box kernel)
                 c.push_back({1, 4});
                 c.push_back({1, 5});
             }
         }
-        if (s->dims == 2 && s->dtype == SP_F64) {
-            if (s->N <= (size_t)kSmallGrid2d) {  // small grids: steps fused per launch
+        if (g.dims == 2 && g.dtype == SP_F64) {
+            if (g.N <= (size_t)kSmallGrid2d) {  // small grids: steps fused per launch
                 c.push_back({2, 0});
                 c.push_back({4, 0});
             } else {  // two more strip shapes
@@ -521,25 +533,80 @@ static std::vector<TuneChoice> tune_candidates(const sp_sim *s) {
         }
     } else {
         c.push_back({1, 0});
-        if (twopass_applies(s->dims, s->dtype, s->stencil, s->model)) c.push_back({1, kFusedFamily});
+        if (twopass_applies(g.dims, g.dtype, g.stencil, g.model)) c.push_back({1, kFusedFamily});
     }
     return c;
+}
+
+static bool tune_available(const TuneGrid &g, TuneChoice c) {
+    for (const TuneChoice &t : tune_candidates(g))
+        if (t.spl == c.spl && t.variant == c.variant) return true;
+    return false;
+}
+
+// The kept choice of the grid's class, if it is one of this grid's candidates.
+static bool tune_find(const TuneGrid &g, TuneChoice *c) {
+    std::lock_guard<std::mutex> lk(g_tune_mu);
+    const auto it = g_tune_cache.find(tune_key(g));
+    if (it == g_tune_cache.end() || !tune_available(g, it->second)) return false;
+    *c = it->second;
+    return true;
+}
+
+static void tune_keep(const TuneGrid &g, TuneChoice c) {
+    std::lock_guard<std::mutex> lk(g_tune_mu);
+    g_tune_cache[tune_key(g)] = c;
+}
+
+static int tune_grid_of(int model, int dims, const int64_t shape[3], const sp_params *p, TuneGrid *g) {
+    if (!shape || !p) return fail(SP_EINVAL, "NULL argument");
+    int st;
+    if (int rc = validate_params(model, dims, 1.0, 1e-6, *p, &st)) return rc;
+    const int64_t nx = shape[0], ny = shape[1], nz = dims == 2 ? 1 : shape[2];
+    if (nx < 1 || ny < 1 || nz < 1 || nx > INT_MAX || ny > INT_MAX || nz > INT_MAX)
+        return fail(SP_EINVAL, "grid side out of range");
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) {  // no device: a table for a program that will have one
+        cudaGetLastError();
+        dev = 0;
+    }
+    *g = {dev, model, st, p->dtype, dims, (int)nx, (uint64_t)nx * ny * nz, p->scheme == SP_SCHEME_FD};
+    return SP_OK;
+}
+
+extern "C" int sp_tune_record(int model, int dims, const int64_t shape[3], const sp_params *p, int steps_per_launch,
+                              int variant) {
+    TuneGrid g;
+    if (int rc = tune_grid_of(model, dims, shape, p, &g)) return rc;
+    if (!tune_available(g, {steps_per_launch, variant}))
+        return fail(SP_EINVAL, "(%d steps per launch, family %d) is not a candidate of this grid", steps_per_launch, variant);
+    tune_keep(g, {steps_per_launch, variant});
+    return SP_OK;
+}
+
+extern "C" int sp_tune_lookup(int model, int dims, const int64_t shape[3], const sp_params *p, int *steps_per_launch,
+                              int *variant) {
+    if (!steps_per_launch || !variant) return fail(SP_EINVAL, "NULL argument");
+    TuneGrid g;
+    if (int rc = tune_grid_of(model, dims, shape, p, &g)) return rc;
+    TuneChoice c;
+    if (!tune_find(g, &c)) return SP_ENOTFOUND;
+    *steps_per_launch = c.spl;
+    *variant = c.variant;
+    return SP_OK;
 }
 
 // Run the candidates on stream st (kTuneSteps steps each, timed with events);
 // returns the number of steps taken.
 static int64_t autotune(sp_sim *s, cudaStream_t st, int *rc) {
     *rc = SP_OK;
-    const TuneKey key = tune_key(s);
-    {
-        std::lock_guard<std::mutex> lk(g_tune_mu);
-        auto it = g_tune_cache.find(key);
-        if (it != g_tune_cache.end()) {
-            set_launch_config(s, it->second);
-            return 0;
-        }
+    const TuneGrid grid = tune_grid(s);
+    TuneChoice win = {s->spl, s->variant};
+    if (tune_find(grid, &win)) {
+        set_launch_config(s, win);
+        return 0;
     }
-    const std::vector<TuneChoice> cand = tune_candidates(s);
+    const std::vector<TuneChoice> cand = tune_candidates(grid);
     if (cand.size() < 2) return 0;
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
@@ -548,7 +615,6 @@ static int64_t autotune(sp_sim *s, cudaStream_t st, int *rc) {
     }
     int64_t taken = 0;
     float best = 1e30f;
-    TuneChoice win = {s->spl, s->variant};
     for (int pass = 0; pass < 2; ++pass)  // pass 0 warms every candidate up, pass 1 is timed
         for (const TuneChoice &c : cand) {
             set_launch_config(s, c);
@@ -577,8 +643,7 @@ static int64_t autotune(sp_sim *s, cudaStream_t st, int *rc) {
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     set_launch_config(s, win);
-    std::lock_guard<std::mutex> lk(g_tune_mu);
-    g_tune_cache[key] = win;
+    tune_keep(grid, win);
     return taken;
 }
 
@@ -792,12 +857,11 @@ extern "C" int sp_autotune(sp_sim *s, void *stream, int64_t *steps_taken) {
 
 extern "C" int sp_set_launch_config(sp_sim *s, int steps_per_launch, int variant) {
     if (!s) return fail(SP_EINVAL, "sim is NULL");
-    for (const TuneChoice &c : tune_candidates(s))
-        if (c.spl == steps_per_launch && c.variant == variant) {
-            s->tune_pending = false;
-            set_launch_config(s, c);
-            return SP_OK;
-        }
+    if (tune_available(tune_grid(s), {steps_per_launch, variant})) {
+        s->tune_pending = false;
+        set_launch_config(s, {steps_per_launch, variant});
+        return SP_OK;
+    }
     // 2D FP64 finite differences: every strip shape and fused-step count runs on
     // any grid (the autotuner tries only the likely winners of the size class)
     const bool fd2d64 = s->dims == 2 && s->dtype == SP_F64 && !s->spec && s->model != SP_MODEL_H &&

@@ -235,6 +235,11 @@ cudaError_t launch_step_t(const StepArgs &a, cudaStream_t s, int n_sm, int k) {
         }
         if (k == 4) return launch_tb<MODEL, ST, T, 4>(a, s);
         if (k == 2) return launch_tb<MODEL, ST, T, 2>(a, s);
+    } else if (k != 1) {
+        // two steps per pass: 16-byte loads and stores of every row, no other kernel behind them
+        const bool al = a.nx % 4 == 0 &&
+                        ((uintptr_t)a.in0 | (uintptr_t)a.in1 | (uintptr_t)a.out0 | (uintptr_t)a.out1) % 16 == 0;
+        if (k != 2 || MODEL == CH || sizeof(T) == 8 || !al) return cudaErrorInvalidValue;
     }
     if constexpr (StencilInfo<ST>::dims == 2 && std::is_same<T, double>::value) {
         const bool small = (long long)a.nx * a.ny <= kSmallGrid2d;
