@@ -42,6 +42,7 @@ void destroy(Plan *P);
 cudaError_t load(Plan *P, const float *phi, cudaStream_t s);
 cudaError_t step(Plan *P, int model, float *phi, double h, double dt, double c1, double c2, double kappa, cudaStream_t s,
                  bool more);
+float2 *spectrum(Plan *P);  // resident, Z[kx][z][y]
 }  // namespace staged
 
 struct SpectralPlan {
@@ -54,6 +55,9 @@ struct SpectralPlan {
     void *tw;                     // twiddles of every axis length
     void *k2;                     // squared wavenumbers of every axis
     bool nh_valid;                // z holds the transformed cubic term of the current phi
+    // see make_hermitian (sp_spectral.cu)
+    long long done, since;        // steps since the spectrum was computed from phi; since it was made Hermitian
+    long long every, first;       // made Hermitian after `every` steps, from step `first` on
 };
 
 // coefficients of the Fourier update

@@ -1,16 +1,14 @@
 // sp_spectral_staged.cu -- the semi-implicit spectral step (sp_spectral.cu) in single
 // precision where its linear part amplifies modes strongly.
 //
-// A mode with L(k) > 0 grows by G = 1 / (1 - dt L(k)) per step until the cubic term holds
-// it, but nothing holds the rounding noise in the non-Hermitian part of the kx = 0 and
-// Nyquist planes: it grows by G each step and enters phi through the rounding of the
-// inverse transform.  Up to G = 4/3 it stays below the rounding of the result (two runs
-// of 25 steps at G = 1.14 with the two implementations differ by 1e-6 to 1e-5).  At G = 2
-// (Allen-Cahn, dt = 0.5) 50 steps amplify it by 2^50 and every implementation's result
-// is off by 1e-4 to 1e-2 in a way that depends on each rounding.  There this file keeps
-// the operations and their order that such results have always been computed with:
-// Stockham transforms with every stage in shared memory (radices 8, 4, 2, 3, 5, 7;
-// 8192^2 1730 us per step against 853 in registers).
+// The rounding noise in the non-Hermitian part of the kx = 0 and Nyquist planes grows by G per
+// step (make_hermitian, sp_spectral.cu).  In single precision at G = 2 (Allen-Cahn, dt = 0.5) it
+// puts 1e-4 to 1e-2 into phi by step 50, in a way that depends on each rounding.  Results up to
+// G^n = 2^50 have always held that, and stay as they are: this file keeps the operations and
+// their order that they were computed with, Stockham transforms with every stage in shared
+// memory (radices 8, 4, 2, 3, 5, 7; 8192^2 1730 us per step against 853 in registers).  From
+// there on, where the noise used to overwhelm phi within ten steps, the planes are kept
+// Hermitian here too.
 #include <cmath>
 #include <mutex>
 #include <string>
@@ -754,6 +752,8 @@ static cudaError_t spectral_step_t(Plan *P, R *phi, double h, double dt, double 
     P->nh_valid = more && e == cudaSuccess;
     return e;
 }
+
+float2 *spectrum(Plan *P) { return static_cast<float2 *>(P->uh); }
 
 cudaError_t step(Plan *P, int model, float *phi, double h, double dt, double c1, double c2, double kappa, cudaStream_t s,
                  bool more) {
