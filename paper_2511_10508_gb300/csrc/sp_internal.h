@@ -10,6 +10,7 @@
 
 #include "sp.h"
 #include "sp_common.cuh"
+#include "sp_split.h"
 
 namespace sp {
 
@@ -65,57 +66,6 @@ inline cudaError_t launch_w2d(int model, int stencil, const StepArgs &a, cudaStr
            : model == GS ? launch_w2d_gs(stencil, a, s, n_sm, k) : launch_w2d_mc(stencil, a, s, n_sm, k);
 }
 
-// Rows per CTA of the 2D warp-strip kernel, whose CTAs own equal runs of the flattened
-// (strip group, row) space: p rows cost p + halo, q CTAs of `load` (their share of 8
-// warps) on the fullest SM take about q load + latency of them (see planes_per_cta).
-// Runs of at least 32 rows left most SMs idle on small grids: 444 x 568 Cahn-Hilliard 9.2
-// us per step, 3.0 now; 1504 x 1000 4th order 13.2 -> 6.2 (runs of 8 rows; of 4: 7.5).
-inline long long rows_per_cta(long long total, int halo, double load, double latency, int occ, int n_sm) {
-    const long long wave = (long long)n_sm * std::max(occ, 1), p0 = (total + wave - 1) / wave;
-    long long best = p0;
-    double best_cost = 0;
-    for (long long p = p0; p <= std::min(total, 8 * p0 + 32); ++p) {
-        const long long ctas = (total + p - 1) / p, q = (ctas + n_sm - 1) / n_sm;
-        const double cost = (q * load + latency) * (p + halo);
-        if (p == p0 || cost < best_cost * 0.999) {
-            best = p;
-            best_cost = cost;
-        }
-        if (q == 1) break;
-    }
-    return best;
-}
-
-// Warps per CTA of the 2D warp-strip kernels, whose CTAs take that many adjacent strips: the
-// most of at least max / 2 that leave the fewest warps without a strip (13 strips: two CTAs of
-// 7 warps, not of 8).
-inline int warps_per_cta(int strips, int max) {
-    if (strips <= max) return strips;
-    int best = max;
-    for (int w = max - 1; 2 * w >= max; --w)
-        if ((strips + w - 1) / w * w < (strips + best - 1) / best * best) best = w;
-    return best;
-}
-
-// Rows per CTA (one warp on grids of few strips, whose last CTA would be half empty, else
-// two on adjacent strips): p rows cost p + halo iterations, each the issue time of the warps that
-// share a scheduler of the fullest SM, at least that of five (a warp's own chain of K steps).
-inline long long warptb_rows(long long total, int halo, int wpc, int occ, int n_sm) {
-    const long long wave = (long long)n_sm * occ, p0 = (total + wave - 1) / wave;
-    long long best = p0;
-    double best_cost = 0;
-    for (long long p = p0; p <= std::min(total, 8 * p0 + 32); ++p) {
-        const long long ctas = (total + p - 1) / p, q = (ctas + n_sm - 1) / n_sm;
-        const double cost = std::max(5.0, q * wpc / 4.0) * (p + halo);
-        if (p == p0 || cost < best_cost * 0.999) {
-            best = p;
-            best_cost = cost;
-        }
-        if (q == 1) break;
-    }
-    return best;
-}
-
 // Resident CTAs per SM by warps per CTA (1 .. MAXW) of a kernel that takes `smem` bytes per warp.
 template <int MAXW, typename Kern> std::array<int, MAXW + 1> warp_occupancy(Kern kern, size_t smem) {
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem * MAXW));
@@ -125,23 +75,6 @@ template <int MAXW, typename Kern> std::array<int, MAXW + 1> warp_occupancy(Kern
         o[w] = std::max(o[w], 1);
     }
     return o;
-}
-
-// Number of equal z segments for a lockstep schedule of `tiles` x segments work
-// items over `wave` resident CTAs: minimises rounds x (planes per segment +
-// halo planes), the time of the slowest CTA.
-inline int lockstep_segments(long long tiles, int nz, int halo, long long wave) {
-    int best = 1;
-    double best_cost = 0;
-    for (int sgs = 1; sgs <= std::min(nz, 64); ++sgs) {
-        const long long rounds = (tiles * sgs + wave - 1) / wave;
-        const double cost = (double)rounds * ((double)nz / sgs + halo);
-        if (sgs == 1 || cost < best_cost * 0.999) {
-            best = sgs;
-            best_cost = cost;
-        }
-    }
-    return best;
 }
 
 // FP64 2D grids up to 1024^2 use small tiles by default (and may fuse steps).

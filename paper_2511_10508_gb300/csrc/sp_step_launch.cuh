@@ -33,33 +33,6 @@ inline bool small_tile(int nx, int ny, int TX, int TY, double margin) {
 
 constexpr size_t kMaxSmemPerCta = 227 * 1024;  // opt-in maximum of dynamic shared memory per CTA
 
-// Planes per CTA of a persistent 3D kernel whose CTAs own equal contiguous runs of
-// the flattened (tile, z) space; at most one resident wave (n_sm x occ CTAs).  A run
-// of p planes costs p + halo planes, halo standing for the planes it only warms its
-// rings with, once more where runs cross from one tile into the next.  With q CTAs on
-// the fullest SM the kernel takes about q + 1 runs: the FP64 pipe is shared, but the
-// barriers and loads of one run are not hidden.  Grids that fill the wave with long runs keep p =
-// total / wave; small ones are spread over all SMs down to single planes (64^3 FP64
-// Gray-Scott 7-point: 417 us per step with runs of at least 32 planes, 17 us now;
-// 32^3 Cahn-Hilliard 179 -> 11.5 us; 129 x 32 x 208 Cahn-Hilliard 189 -> 47 us, where
-// the balance of q against p decides between runs of 3 (53 us) and 4 planes).
-inline long long planes_per_cta(long long tiles, int nz, double halo, int occ, int n_sm) {
-    const long long total = tiles * nz, wave = (long long)n_sm * std::max(occ, 1);
-    const long long p0 = (total + wave - 1) / wave;
-    long long best = p0;
-    double best_cost = 0;
-    for (long long p = p0; p <= std::min(total, 4 * p0 + 8); ++p) {
-        const long long ctas = (total + p - 1) / p, q = (ctas + n_sm - 1) / n_sm;
-        const double cost = (q + 1.0) * (p + (nz % p ? 2 : 1) * halo);
-        if (p == p0 || cost < best_cost * 0.999) {
-            best = p;
-            best_cost = cost;
-        }
-        if (q == 1) break;  // longer runs on fewer SMs only take longer
-    }
-    return best;
-}
-
 // Batched persistent 2D kernel (FP64): rows per batch and CTAs per SM.
 template <int MODEL> struct Batch2d { static constexpr int NT = 128, RB = (MODEL == CH) ? 8 : (MODEL == AC ? 4 : 2), CPS = 4; };
 
