@@ -12,6 +12,7 @@
 // blocks through shared memory, and each block writes its pair to a scratch
 // array; a single block then combines the block pairs in index order and
 // writes the scaled result.
+#include <cmath>
 #include <type_traits>
 
 #include "sp_internal.h"
@@ -204,6 +205,29 @@ reduce_partial_kernel(const T *__restrict__ f, uint64_t N, double *__restrict__ 
     }
 }
 
+// Energy density of one point, term by term (the definition): for values that the sums below
+// are not made for.
+__device__ __noinline__ double energy_density(int dims, int extra, const double *p, double h, double c1, double c2, double c3) {
+    const double gx = (p[1] - p[0]) / h, gy = (p[2] - p[0]) / h;
+    double g2 = gx * gx + gy * gy;
+    if (dims == 3) {
+        const double gz = (p[3] - p[0]) / h;
+        g2 = g2 + gz * gz;
+    }
+    const double p2 = p[0] * p[0], r = p[4];
+    if (extra == 1) return 0.5 * g2 - 0.5 * c1 * p2 + 0.25 * c2 * p2 * p2 + 0.5 * r * r - c3 * p2 * r;
+    double q = r * r + p[5] * p[5];
+    if (dims == 3) q = q + p[6] * p[6];
+    const double d = 0.5 * g2 - 0.5 * c1 * p2 + 0.25 * c2 * p2 * p2;
+    return extra == 2 ? d + 0.5 * q : d;
+}
+
+// The bits of |x| (FP64: the upper half) and the first value that the energy's sums leave to
+// energy_density: infinities and NaN, in FP64 from 2^200 on, whose fourth power may overflow.
+__device__ __forceinline__ uint32_t size_bits(float x) { return __float_as_uint(x) & 0x7fffffffu; }
+__device__ __forceinline__ uint32_t size_bits(double x) { return (uint32_t)__double2hiint(x) & 0x7fffffffu; }
+template <typename C> constexpr uint32_t kSizeLimit = sizeof(C) == 8 ? 0x4c700000u : 0x7f800000u;
+
 // Free energy: block partials of sum [1/2 sum_axes ((f_{i+e} - f_i)/h)^2 - c1/2 f^2
 // + c2/4 f^4] (forward differences, periodic).  EXTRA 1 (Model C) adds rho^2/2 -
 // c3 f^2 rho, EXTRA 2 (Model H) the currents' |j|^2/2.
@@ -217,20 +241,21 @@ reduce_partial_kernel(const T *__restrict__ f, uint64_t N, double *__restrict__ 
 // the index arithmetic is per chunk.  The sums of 8 points are plain FP64 and then
 // enter the thread's Neumaier pair.  512^3: FP32 14.0 ms and FP64 12.7 ms with a
 // division per difference, one point per thread and a Neumaier update per point;
-// now 2.4 and 2.8 ms, 10.2 operations per point at 515 Gop/s.  A field that holds an infinity gives NaN (f^4 - f^2 of it).
+// now 2.4 and 2.8 ms, 10.2 operations per point at 515 Gop/s.  Chunks with infinities, NaN or huge
+// values, and coefficients or steps beyond 2^+-100 (wild), take energy_density point by point.
 template <typename T, int DIMS, int EXTRA>
 __global__ void __launch_bounds__(kReduceThreads)
 reduce_energy_kernel(const T *__restrict__ f, const T *__restrict__ rho, const T *__restrict__ j0,
                      const T *__restrict__ j1, const T *__restrict__ j2, int nx, int ny, int nz, double half_inv_h2,
-                     double half_c1, double quarter_c2, double c3, double *__restrict__ partials) {
+                     double half_c1, double quarter_c2, double c3, double h, int wild, double *__restrict__ partials) {
     typedef typename Cmp<T>::type C;
     constexpr int V = 16 / sizeof(T);
-    const bool vec = nx % V == 0 && (reinterpret_cast<uintptr_t>(f) & 15u) == 0;
+    const bool vec = nx % V == 0 && ((reinterpret_cast<uintptr_t>(f) | reinterpret_cast<uintptr_t>(rho) | reinterpret_cast<uintptr_t>(j0) |
+                                      reinterpret_cast<uintptr_t>(j1) | reinterpret_cast<uintptr_t>(j2)) & 15u) == 0;
     const uint64_t cpr = (uint64_t)(nx + V - 1) / V, rows = (uint64_t)ny * nz, chunks = cpr * rows;
     const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     double s = 0.0, c = 0.0, g = 0.0, e = 0.0, q = 0.0;  // the pair; gradient, local and current sums of the open block
-    bool inf = false;
     int open = 0;
     auto fold = [&] { neu_add(s, c, FMA(half_inv_h2, g, EXTRA == 2 ? FMA(0.5, q, e) : e)); };
     for (uint64_t u = tid; u < chunks; u += stride) {
@@ -280,6 +305,46 @@ reduce_energy_kernel(const T *__restrict__ f, const T *__restrict__ rho, const T
         }
         const C last = load_one(x0 + n == nx ? p0 - x0 : p0 + n);
         v[V] = last;
+        constexpr int NE = EXTRA == 1 ? 1 : EXTRA == 2 ? DIMS : 0;  // the density, or the currents
+        C ex[NE ? NE : 1][V];
+        (void)ex;
+#pragma unroll
+        for (int a = 0; a < NE; ++a) {
+            const T *p = (EXTRA == 1 ? rho : a == 0 ? j0 : a == 1 ? j1 : j2) + row * (uint64_t)nx + x0;
+            if (vec) {
+                load_vec<T, V>(p, ex[a]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < V; ++j)
+                    if (j < n) ex[a][j] = load_one(p + j);
+            }
+        }
+        uint32_t size = size_bits(last);
+#pragma unroll
+        for (int j = 0; j < V; ++j)
+            if (j < n) {
+                size = max(size, max(size_bits(v[j]), size_bits(vy[j])));
+                if constexpr (DIMS == 3) size = max(size, size_bits(vz[j]));
+#pragma unroll
+                for (int a = 0; a < NE; ++a) size = max(size, size_bits(ex[a][j]));
+            }
+        if (wild || size >= kSizeLimit<C>) {
+            for (int j = 0; j < n; ++j) {
+                double q[7] = {};
+#pragma unroll
+                for (int i = 0; i < V; ++i)
+                    if (i == j) {
+                        q[0] = widen(v[i]);
+                        q[1] = widen(i + 1 < n ? v[i + 1] : last);
+                        q[2] = widen(vy[i]);
+                        if constexpr (DIMS == 3) q[3] = widen(vz[i]);
+#pragma unroll
+                        for (int a = 0; a < NE; ++a) q[4 + a] = widen(ex[a][i]);
+                    }
+                neu_add(s, c, energy_density(DIMS, EXTRA, q, h, 2.0 * half_c1, 4.0 * quarter_c2, c3));
+            }
+            continue;
+        }
 #pragma unroll
         for (int j = 0; j < V; ++j)
             if (j < n) {
@@ -292,20 +357,16 @@ reduce_energy_kernel(const T *__restrict__ f, const T *__restrict__ rho, const T
                     const double dz = widen(vz[j]) - p;
                     g = FMA(dz, dz, g);
                 }
-                inf |= isinf(v[j]);
                 const double p2 = p * p;
                 e = FMA(FMA(quarter_c2, p2, -half_c1), p2, e);
                 if constexpr (EXTRA == 1) {
-                    const double r = widen(to_c(rho[row * (uint64_t)nx + x0 + j]));
+                    const double r = widen(ex[0][j]);
                     e = FMA(FMA(-c3, p2, 0.5 * r), r, e);
                 }
                 if constexpr (EXTRA == 2) {
-                    const uint64_t i = row * (uint64_t)nx + x0 + j;
-                    const double a = widen(to_c(j0[i])), b = widen(to_c(j1[i]));
-                    q = FMA(a, a, q);
-                    q = FMA(b, b, q);
-                    if constexpr (DIMS == 3) {
-                        const double d = widen(to_c(j2[i]));
+#pragma unroll
+                    for (int a = 0; a < NE; ++a) {
+                        const double d = widen(ex[a][j]);
                         q = FMA(d, d, q);
                     }
                 }
@@ -317,7 +378,6 @@ reduce_energy_kernel(const T *__restrict__ f, const T *__restrict__ rho, const T
         }
     }
     fold();
-    if (inf) s = NAN;
     block_combine<SP_SUM_U>(s, c);
     if (threadIdx.x == 0) {
         partials[2 * blockIdx.x] = s;
@@ -342,8 +402,10 @@ static void launch_energy(const T *f, const ReduceGeom &g, double *partials, int
     const T *rho = static_cast<const T *>(g.rho);
     const T *j[3] = {static_cast<const T *>(g.jq[0]), static_cast<const T *>(g.jq[1]), static_cast<const T *>(g.jq[2])};
     const double k = 0.5 / (g.h * g.h), a = 0.5 * g.c1, b = 0.25 * g.c2;
+    auto tame = [](double x) { return std::fabs(x) <= 0x1p100; };
+    const int wild = !(g.h >= 0x1p-100 && tame(g.h) && tame(g.c1) && tame(g.c2) && tame(g.c3));
     auto kern = g.nq > 0 ? reduce_energy_kernel<T, DIMS, 2> : g.rho ? reduce_energy_kernel<T, DIMS, 1> : reduce_energy_kernel<T, DIMS, 0>;
-    kern<<<nblocks, kReduceThreads, 0, s>>>(f, rho, j[0], j[1], j[2], g.nx, g.ny, g.nz, k, a, b, g.c3, partials);
+    kern<<<nblocks, kReduceThreads, 0, s>>>(f, rho, j[0], j[1], j[2], g.nx, g.ny, g.nz, k, a, b, g.c3, g.h, wild, partials);
 }
 
 template <typename T, int WHAT>
