@@ -80,6 +80,13 @@ __device__ __forceinline__ double widen(float x) {
     return __hiloint2double((int)((b & 0x80000000u) | ((mag >> 3) + off)), (int)(b << 29));
 }
 
+// The same of normal values alone.
+__device__ __forceinline__ double widen_normal(double x) { return x; }
+__device__ __forceinline__ double widen_normal(float x) {
+    const int b = __float_as_int(x);
+    return __hiloint2double(((b >> 3) & (int)0x8fffffff) + 0x38000000, b << 29);
+}
+
 // Sum of a block of 32 FP32 values (BF16 values widen to FP32 exactly) in
 // fixed point, with integer arithmetic only.  A value with biased exponent e
 // and 24-bit significand m is m * 2^(max(e,1) - 150).  With E the largest
@@ -227,27 +234,139 @@ __device__ __noinline__ double energy_density(int dims, int extra, const double 
 __device__ __forceinline__ uint32_t size_bits(float x) { return __float_as_uint(x) & 0x7fffffffu; }
 __device__ __forceinline__ uint32_t size_bits(double x) { return (uint32_t)__double2hiint(x) & 0x7fffffffu; }
 template <typename C> constexpr uint32_t kSizeLimit = sizeof(C) == 8 ? 0x4c700000u : 0x7f800000u;
+// below kUsualLimit: values that widen_normal takes, below the limit above
+__device__ __forceinline__ uint32_t usual_bits(float x) { return size_bits(x) - 0x00800000u; }
+__device__ __forceinline__ uint32_t usual_bits(double x) { return size_bits(x); }
+template <typename C> constexpr uint32_t kUsualLimit = sizeof(C) == 8 ? 0x4c700000u : 0x7f000000u;
+
+// a 2^k as an unevaluated sum (x + y)
+__device__ __noinline__ double2 fixed_value(__int128 a, int k) {
+    const bool neg = a < 0;
+    const unsigned __int128 m = neg ? -(unsigned __int128)a : (unsigned __int128)a;
+    auto part = [&](int at) {  // 43 bits from `at` on: below the 2^52 that the upper half adds
+        const uint64_t b = (uint64_t)(m >> at) & ((1ull << 43) - 1);
+        return __hiloint2double((int)(0x43300000u | (uint32_t)(b >> 32)), (int)(uint32_t)b) - 0x1p52;
+    };
+    const double c0 = part(0), c1 = part(43) * 0x1p43, c2 = part(86) * 0x1p86;
+    const double hi = c2 + c1, lo = (c1 - (hi - c2)) + c0;
+    double x, y;
+    if (k > -900 && k < 900) {
+        const double p = __hiloint2double((k + 1023) << 20, 0);
+        x = hi * p, y = lo * p;
+    } else {
+        x = scalbn(hi, k), y = scalbn(lo, k);
+    }
+    return neg ? double2{-x, -y} : double2{x, y};
+}
+
+// A sum of finite doubles in fixed point, with integer instructions only: 96 bits of units of
+// 2^(top - 1097), top the largest biased exponent that they hold (68 at least, so that zeros and
+// denormals count as nothing).  A value keeps its bits down to 2^-74 of 2^(top - 1023), and a million
+// of them fit.  Negative values are added as complements, the ones that these lack in `lack`.
+struct FixedSum {
+    uint32_t w0 = 0, w1 = 0, w2 = 0, lack = 0;
+    int top = 68;
+    double s = 0.0, c = 0.0;  // what was summed in smaller units, a Neumaier pair
+    __device__ __forceinline__ __int128 bits() const {
+        return ((__int128)(int)w2 << 64 | (unsigned __int128)((uint64_t)w1 << 32 | w0)) + lack;
+    }
+    __device__ __forceinline__ int unit() const { return top - 1097; }
+    // before values with the biased exponent e (and some of 2^12 times theirs, so that it happens seldom)
+    __device__ __forceinline__ void hold(int e) {
+        if (e <= top) return;
+        if ((w0 | w1 | w2 | lack) != 0) {
+            const double2 v = fixed_value(bits(), unit());
+            neu_add(s, c, v.x);
+            c += v.y;
+            w0 = w1 = w2 = lack = 0;
+        }
+        top = e + 12;
+    }
+    // adds x (SIGNED false: of at least 0), whose exponent is held: its 53 bits from bit 74 on,
+    // `sh` lower where x is smaller, without branches (the FP64 work of other points goes on beside it)
+    template <bool SIGNED> __device__ __forceinline__ void add(double x) {
+        const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+        const int sh = top + 10 - (int)(SIGNED ? (hi << 1) >> 21 : hi >> 20);
+        const uint32_t m = (hi & 0xfffffu) | 0x100000u;
+        const bool in = sh < 64, low = sh >= 32;
+        const uint32_t x2 = low ? 0u : m, x1 = low ? (in ? m : 0u) : lo, x0 = low && in ? lo : 0u;
+        uint32_t v0 = __funnelshift_r(x0, x1, sh), v1 = __funnelshift_r(x1, x2, sh), v2 = __funnelshift_r(x2, 0u, sh);
+        if constexpr (SIGNED) {
+            const uint32_t neg = (uint32_t)((int)hi >> 31);
+            v0 ^= neg, v1 ^= neg, v2 ^= neg;
+            lack -= neg;
+        }
+        asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
+            : "+r"(w0), "+r"(w1), "+r"(w2) : "r"(v0), "r"(v1), "r"(v2));
+    }
+};
+
+// Sum over a warp, in lane 0, of a 2^k, in the largest of the lanes' units.
+__device__ __forceinline__ void warp_sum(__int128 &a, int &k) {
+    const int km = __reduce_max_sync(0xffffffffu, k);
+    a >>= min(km - k, 127);
+    k = km;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        const uint64_t lo = __shfl_down_sync(0xffffffffu, (uint64_t)a, off);
+        const long long hi = __shfl_down_sync(0xffffffffu, (long long)(a >> 64), off);
+        a += (__int128)hi << 64 | lo;
+    }
+}
+
+// The values of NS FixedSums over a block, one in each of its first NS threads.
+template <int NS> __device__ __forceinline__ double2 block_sums(const FixedSum (&f)[NS]) {
+    constexpr int NW = kReduceThreads / 32;
+    __shared__ uint64_t lo[NS * NW];
+    __shared__ long long hi[NS * NW];
+    __shared__ int ks[NS * NW];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+        __int128 a = f[i].bits();
+        int k = f[i].unit();
+        warp_sum(a, k);
+        if (lane == 0) lo[i * NW + warp] = (uint64_t)a, hi[i * NW + warp] = (long long)(a >> 64), ks[i * NW + warp] = k;
+    }
+    __syncthreads();
+    if (threadIdx.x >= NS) return double2{0.0, 0.0};
+    const int first = threadIdx.x * NW;
+    int k = ks[first];
+#pragma unroll 1
+    for (int w = 1; w < NW; ++w) k = max(k, ks[first + w]);
+    __int128 a = 0;
+#pragma unroll 1
+    for (int w = 0; w < NW; ++w) {
+        const __int128 part = (__int128)hi[first + w] << 64 | lo[first + w];  // (signed: the shift keeps the sign)
+        a += part >> min(k - ks[first + w], 127);
+    }
+    return fixed_value(a, k);
+}
 
 // Free energy: block partials of sum [1/2 sum_axes ((f_{i+e} - f_i)/h)^2 - c1/2 f^2
 // + c2/4 f^4] (forward differences, periodic).  EXTRA 1 (Model C) adds rho^2/2 -
 // c3 f^2 rho, EXTRA 2 (Model H) the currents' |j|^2/2.
 //
 // The FP64 pipe bounds it (2 operations per clock per SM), so the work per point is
-// 9 FP64 operations in 3D: three differences, three multiply-adds into the sum of
-// their squares (1/(2h^2) is applied once per fold, not per point), and f^2,
-// (c2/4) f^2 - c1/2 and their product added by one multiply-add.  Every thread takes
-// chunks of V consecutive points of a row (16-byte loads of the chunk and of its y
-// and z neighbours where alignment allows; the neighbour plane comes from L2), so
-// the index arithmetic is per chunk.  The sums of 8 points are plain FP64 and then
-// enter the thread's Neumaier pair.  512^3: FP32 14.0 ms and FP64 12.7 ms with a
-// division per difference, one point per thread and a Neumaier update per point;
-// now 2.4 and 2.8 ms, 10.2 operations per point at 515 Gop/s.  Chunks with infinities, NaN or huge
-// values, and coefficients or steps beyond 2^+-100 (wild), take energy_density point by point.
+// 8 FP64 operations in 3D: three differences, the sum of their squares by a product and two
+// multiply-adds, f^2 and f^4.  Each of the three (and what the extra fields give) is summed over all
+// points for itself, exactly, in fixed point (FixedSum: the integer units are idle otherwise), and the
+// coefficients, 1/(2h^2) as a sum of two doubles, are applied to the block's sums.  So nothing but a
+// point's own roundings enters the sum, as with one compensated addition per point, which takes 6
+// FP64 operations.  (Plain FP64 sums of 8 points before the compensated one, a rounded 1/(2h^2) and
+// local densities formed per point took 9.6; their error, relative to the sum of 16^3 points of FP32
+// noise at h = 1, was 1.1e-16, now 1.1e-17.)
+// Every thread takes chunks of V consecutive points of a row (16-byte loads of the chunk and of
+// its y and z neighbours where alignment allows; the neighbour plane comes from L2), so
+// the index arithmetic is per chunk.  512^3: FP32 14.0 ms and FP64 12.7 ms with a division per
+// difference, one point per thread and a Neumaier update per point; 2.38 and 2.39 ms with the
+// blocks of 8; now 2.01 and 2.10, 8 operations per point at 535 Gop/s.  Chunks with infinities, NaN or
+// huge values, and coefficients or steps beyond 2^+-100 (wild), take energy_density point by point.
 template <typename T, int DIMS, int EXTRA>
-__global__ void __launch_bounds__(kReduceThreads)
+__global__ void __launch_bounds__(kReduceThreads, kReduceBlocksPerSM)
 reduce_energy_kernel(const T *__restrict__ f, const T *__restrict__ rho, const T *__restrict__ j0,
-                     const T *__restrict__ j1, const T *__restrict__ j2, int nx, int ny, int nz, double half_inv_h2,
-                     double half_c1, double quarter_c2, double c3, double h, int wild, double *__restrict__ partials) {
+                     const T *__restrict__ j1, const T *__restrict__ j2, int nx, int ny, int nz, double2 half_inv_h2,
+                     double c1, double c2, double c3, double h, int wild, double *__restrict__ partials) {
     typedef typename Cmp<T>::type C;
     constexpr int V = 16 / sizeof(T);
     const bool vec = nx % V == 0 && ((reinterpret_cast<uintptr_t>(f) | reinterpret_cast<uintptr_t>(rho) | reinterpret_cast<uintptr_t>(j0) |
@@ -255,9 +374,13 @@ reduce_energy_kernel(const T *__restrict__ f, const T *__restrict__ rho, const T
     const uint64_t cpr = (uint64_t)(nx + V - 1) / V, rows = (uint64_t)ny * nz, chunks = cpr * rows;
     const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    double s = 0.0, c = 0.0, g = 0.0, e = 0.0, q = 0.0;  // the pair; gradient, local and current sums of the open block
-    int open = 0;
-    auto fold = [&] { neu_add(s, c, FMA(half_inv_h2, g, EXTRA == 2 ? FMA(0.5, q, e) : e)); };
+    double s = 0.0, c = 0.0;
+    // sums of the squared differences, of f^2, of f^4, and of rho^2 - 2 c3 f^2 rho or |j|^2
+    constexpr int NS = EXTRA ? 4 : 3;
+    FixedSum sum[NS];
+    const double twice_c3 = 2.0 * c3;
+    (void)twice_c3;
+    const uint32_t limit = wild ? 0u : kUsualLimit<C>;
     for (uint64_t u = tid; u < chunks; u += stride) {
         uint64_t row;
         int x0;
@@ -286,99 +409,124 @@ reduce_energy_kernel(const T *__restrict__ f, const T *__restrict__ rho, const T
         const uint64_t plane = (uint64_t)nx * ny;
         const T *pz = z + 1 == nz ? p0 - (uint64_t)(nz - 1) * plane : p0 + plane;
         const int n = vec ? V : min(V, nx - x0);  // points of this chunk
-        C v[V + 1], vy[V], vz[V];
-        if (vec) {
-            C w[V];
-            load_vec<T, V>(p0, w);
+        // the order parameter here, in y and in z; the density or the currents
+        constexpr int NE = EXTRA == 1 ? 1 : EXTRA == 2 ? DIMS : 0, NX = DIMS + NE;
+        C x[NX][V];
 #pragma unroll
-            for (int j = 0; j < V; ++j) v[j] = w[j];
-            load_vec<T, V>(py, vy);
-            if constexpr (DIMS == 3) load_vec<T, V>(pz, vz);
-        } else {
-#pragma unroll
-            for (int j = 0; j < V; ++j)
-                if (j < n) {
-                    v[j] = load_one(p0 + j);
-                    vy[j] = load_one(py + j);
-                    if constexpr (DIMS == 3) vz[j] = load_one(pz + j);
-                }
-        }
-        const C last = load_one(x0 + n == nx ? p0 - x0 : p0 + n);
-        v[V] = last;
-        constexpr int NE = EXTRA == 1 ? 1 : EXTRA == 2 ? DIMS : 0;  // the density, or the currents
-        C ex[NE ? NE : 1][V];
-        (void)ex;
-#pragma unroll
-        for (int a = 0; a < NE; ++a) {
-            const T *p = (EXTRA == 1 ? rho : a == 0 ? j0 : a == 1 ? j1 : j2) + row * (uint64_t)nx + x0;
+        for (int a = 0; a < NX; ++a) {
+            const int k = a - DIMS;
+            const T *p = a == 0   ? p0
+                         : a == 1 ? py
+                         : k < 0  ? pz
+                                  : (EXTRA == 1 ? rho : k == 0 ? j0 : k == 1 ? j1 : j2) + row * (uint64_t)nx + x0;
             if (vec) {
-                load_vec<T, V>(p, ex[a]);
+                load_vec<T, V>(p, x[a]);
             } else {
 #pragma unroll
-                for (int j = 0; j < V; ++j)
-                    if (j < n) ex[a][j] = load_one(p + j);
+                for (int j = 0; j < V; ++j) x[a][j] = j < n ? load_one(p + j) : C(1);
             }
         }
-        uint32_t size = size_bits(last);
+        const C last = load_one(x0 + n == nx ? p0 - x0 : p0 + n);
+        uint32_t usual = usual_bits(last);
 #pragma unroll
-        for (int j = 0; j < V; ++j)
-            if (j < n) {
-                size = max(size, max(size_bits(v[j]), size_bits(vy[j])));
-                if constexpr (DIMS == 3) size = max(size, size_bits(vz[j]));
+        for (int a = 0; a < NX; ++a)
 #pragma unroll
-                for (int a = 0; a < NE; ++a) size = max(size, size_bits(ex[a][j]));
+            for (int j = 0; j < V; ++j) usual = max(usual, usual_bits(x[a][j]));
+        double w[NX][V], wl;
+        if (usual < limit) {
+            wl = widen_normal(last);
+#pragma unroll
+            for (int a = 0; a < NX; ++a)
+#pragma unroll
+                for (int j = 0; j < V; ++j) w[a][j] = widen_normal(x[a][j]);
+        } else {
+            uint32_t size = size_bits(last);
+            wl = widen(last);
+#pragma unroll
+            for (int a = 0; a < NX; ++a)
+#pragma unroll
+                for (int j = 0; j < V; ++j) {
+                    w[a][j] = widen(x[a][j]);
+                    size = max(size, size_bits(x[a][j]));
+                }
+            if (wild || size >= kSizeLimit<C>) {
+                for (int j = 0; j < n; ++j) {
+                    double q[7] = {};
+#pragma unroll
+                    for (int i = 0; i < V; ++i)
+                        if (i == j) {
+                            q[0] = w[0][i];
+                            q[1] = i + 1 < n ? w[0][i + 1 < V ? i + 1 : 0] : wl;
+                            q[2] = w[1][i];
+                            if constexpr (DIMS == 3) q[3] = w[2][i];
+#pragma unroll
+                            for (int a = 0; a < NE; ++a) q[4 + a] = w[DIMS + a][i];
+                        }
+                    neu_add(s, c, energy_density(DIMS, EXTRA, q, h, c1, c2, c3));
+                }
+                continue;
             }
-        if (wild || size >= kSizeLimit<C>) {
-            for (int j = 0; j < n; ++j) {
-                double q[7] = {};
+        }
+        double t[NS][V];
 #pragma unroll
-                for (int i = 0; i < V; ++i)
-                    if (i == j) {
-                        q[0] = widen(v[i]);
-                        q[1] = widen(i + 1 < n ? v[i + 1] : last);
-                        q[2] = widen(vy[i]);
-                        if constexpr (DIMS == 3) q[3] = widen(vz[i]);
-#pragma unroll
-                        for (int a = 0; a < NE; ++a) q[4 + a] = widen(ex[a][i]);
-                    }
-                neu_add(s, c, energy_density(DIMS, EXTRA, q, h, 2.0 * half_c1, 4.0 * quarter_c2, c3));
+        for (int j = 0; j < V; ++j) {
+            const double p = w[0][j], dx = (j + 1 < n ? w[0][j + 1 < V ? j + 1 : 0] : wl) - p, dy = w[1][j] - p;
+            double g = FMA(dy, dy, dx * dx);
+            if constexpr (DIMS == 3) {
+                const double dz = w[2][j] - p;
+                g = FMA(dz, dz, g);
             }
-            continue;
+            const double p2 = p * p;
+            t[0][j] = g, t[1][j] = p2, t[2][j] = p2 * p2;
+            if constexpr (EXTRA == 1) {
+                const double r = w[DIMS][j];
+                t[NS - 1][j] = FMA(-(twice_c3 * p2), r, r * r);
+            }
+            if constexpr (EXTRA == 2) {
+                double q = w[DIMS][j] * w[DIMS][j];
+#pragma unroll
+                for (int a = 1; a < NE; ++a) q = FMA(w[DIMS + a][j], w[DIMS + a][j], q);
+                t[NS - 1][j] = q;
+            }
+            if (j >= n)
+#pragma unroll
+                for (int i = 0; i < NS; ++i) t[i][j] = 0.0;
         }
 #pragma unroll
-        for (int j = 0; j < V; ++j)
-            if (j < n) {
-                const double p = widen(v[j]);
-                const double dx = widen(j + 1 < n ? v[j + 1] : last) - p;
-                const double dy = widen(vy[j]) - p;
-                g = FMA(dx, dx, g);
-                g = FMA(dy, dy, g);
-                if constexpr (DIMS == 3) {
-                    const double dz = widen(vz[j]) - p;
-                    g = FMA(dz, dz, g);
-                }
-                const double p2 = p * p;
-                e = FMA(FMA(quarter_c2, p2, -half_c1), p2, e);
-                if constexpr (EXTRA == 1) {
-                    const double r = widen(ex[0][j]);
-                    e = FMA(FMA(-c3, p2, 0.5 * r), r, e);
-                }
-                if constexpr (EXTRA == 2) {
+        for (int i = 0; i < NS; ++i) {
+            uint32_t m = 0;
 #pragma unroll
-                    for (int a = 0; a < NE; ++a) {
-                        const double d = widen(ex[a][j]);
-                        q = FMA(d, d, q);
-                    }
-                }
+            for (int j = 0; j < V; ++j) m = max(m, size_bits(t[i][j]));
+            sum[i].hold((int)(m >> 20));
+#pragma unroll
+            for (int j = 0; j < V; ++j) {
+                if (EXTRA == 1 && i == 3) sum[i].template add<true>(t[i][j]);
+                else sum[i].template add<false>(t[i][j]);
             }
-        if (++open == 8 / V) {
-            fold();
-            g = e = q = 0.0;
-            open = 0;
         }
     }
-    fold();
-    block_combine<SP_SUM_U>(s, c);
+    // k (x + y) of sum i, whose coefficient is k, into the pair
+    const double2 coef[4] = {half_inv_h2, {-0.5 * c1, 0.0}, {0.25 * c2, 0.0}, {0.5, 0.0}};
+    auto fold = [&](int i, double x, double y) {
+        const double2 k = coef[i];
+        const double v = k.x * x;
+        neu_add(s, c, v);
+        c += FMA(k.x, x, -v) + FMA(k.x, y, k.y * x);
+    };
+    // (the pairs are in use only after larger units or a chunk summed point by point)
+    bool used = s != 0.0 || c != 0.0;
+#pragma unroll
+    for (int i = 0; i < NS; ++i) used |= sum[i].s != 0.0;
+    if (__syncthreads_or(used)) {
+#pragma unroll
+        for (int i = 0; i < NS; ++i) fold(i, sum[i].s, sum[i].c);
+        block_combine<SP_SUM_U>(s, c);
+    }
+    const double2 mine = block_sums(sum);
+    if (threadIdx.x < 32) {
+#pragma unroll
+        for (int i = 0; i < NS; ++i) fold(i, __shfl_sync(0xffffffffu, mine.x, i), __shfl_sync(0xffffffffu, mine.y, i));
+    }
     if (threadIdx.x == 0) {
         partials[2 * blockIdx.x] = s;
         partials[2 * blockIdx.x + 1] = c;
@@ -401,11 +549,14 @@ template <typename T, int DIMS>
 static void launch_energy(const T *f, const ReduceGeom &g, double *partials, int nblocks, cudaStream_t s) {
     const T *rho = static_cast<const T *>(g.rho);
     const T *j[3] = {static_cast<const T *>(g.jq[0]), static_cast<const T *>(g.jq[1]), static_cast<const T *>(g.jq[2])};
-    const double k = 0.5 / (g.h * g.h), a = 0.5 * g.c1, b = 0.25 * g.c2;
     auto tame = [](double x) { return std::fabs(x) <= 0x1p100; };
     const int wild = !(g.h >= 0x1p-100 && tame(g.h) && tame(g.c1) && tame(g.c2) && tame(g.c3));
+    // 1/(2 h^2) as a sum of two doubles (0 where no sum takes it)
+    const double hh = g.h * g.h, rest = std::fma(g.h, g.h, -hh), k = wild ? 0.0 : 0.5 / hh;
+    const double k2 = wild ? 0.0 : (std::fma(-k, hh, 0.5) - k * rest) / hh;
     auto kern = g.nq > 0 ? reduce_energy_kernel<T, DIMS, 2> : g.rho ? reduce_energy_kernel<T, DIMS, 1> : reduce_energy_kernel<T, DIMS, 0>;
-    kern<<<nblocks, kReduceThreads, 0, s>>>(f, rho, j[0], j[1], j[2], g.nx, g.ny, g.nz, k, a, b, g.c3, g.h, wild, partials);
+    kern<<<nblocks, kReduceThreads, 0, s>>>(f, rho, j[0], j[1], j[2], g.nx, g.ny, g.nz, double2{k, k2}, g.c1, g.c2, g.c3,
+                                            g.h, wild, partials);
 }
 
 template <typename T, int WHAT>

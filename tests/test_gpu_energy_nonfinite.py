@@ -60,3 +60,15 @@ def test_nonfinite_and_huge(sp, model, c1, c3, field, value, phi, dtypes, shape)
             assert abs(got - ref) <= 1e-14 * abs(ref), (dtype, got, ref)  # one value is all of it
         else:
             assert got == ref or (np.isnan(got) and np.isnan(ref)), (dtype, got, ref)
+
+
+@pytest.mark.parametrize("h,c1,dt", [(1.0, 1e40, 1e-41), (1e-40, 1.0, 1e-82)])
+@pytest.mark.parametrize("shape", [(9, 16), (5, 6, 8)])
+def test_coefficients_and_steps_beyond_the_sums(sp, h, c1, dt, shape):
+    for dtype in (0, 1):
+        with sp.Simulation(0, shape, h=h, dt=dt, dtype=dtype, c1=c1, ic_amp=0.5, seed=4) as sim:
+            q = [sim.read(0)]
+            got = sim.reduce(sp.FREE_ENERGY)
+        with np.errstate(all="ignore"):
+            ref = densities(q, h, c1, 1.0, 0.5, 0, sp).sum() * ((h * h) * h if len(shape) == 3 else h * h)
+        assert got == ref or abs(got - ref) <= 1e-13 * abs(ref) or (np.isnan(got) and np.isnan(ref)), (dtype, got, ref)
