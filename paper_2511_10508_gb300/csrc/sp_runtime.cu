@@ -234,6 +234,7 @@ struct sp_sim {
     cudaGraphExec_t graph[2];  // kGraphSteps steps starting from level 0 / level 1
     int spl;                   // steps fused per launch (temporal blocking)
     int variant;               // kernel family (see g_step_variant)
+    bool launched;             // this configuration's kernel has run outside a capture
     void *mu_tmp;              // unfused ablation: mu temporary (allocated on first use)
     bool tune_pending;         // autotune on the next long sp_step
     double genw[kMaxGenRadius + 1];  // generated stencil: kernel weights (d w_0, w_1, ..., w_r)
@@ -487,6 +488,7 @@ static void set_launch_config(sp_sim *s, TuneChoice c) {
         }
     s->spl = c.spl;
     s->variant = c.variant;
+    s->launched = false;
 }
 
 static TuneGrid tune_grid(const sp_sim *s) {
@@ -643,6 +645,7 @@ static int64_t autotune(sp_sim *s, cudaStream_t st, int *rc) {
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     set_launch_config(s, win);
+    s->launched = true;  // as one of the candidates
     tune_keep(grid, win);
     return taken;
 }
@@ -667,9 +670,9 @@ static cudaError_t capture_graph(sp_sim *s) {
 }
 
 // Steps are issued as replays of a captured kGraphSteps-step graph (one per
-// starting level) plus eager launches for the remainder.  The first launches of a
-// handle are eager, so that the kernels' one-time set-up never runs inside a
-// capture.  (They too take spl steps: ten first steps of Gray-Scott 16384^2 with one
+// starting level) plus eager launches for the remainder.  The first launch of a
+// configuration is eager, so that its kernel's one-time set-up never runs inside a
+// capture.  (It too takes spl steps: ten first steps of Gray-Scott 16384^2 with one
 // step in the first launch 3370 us, now 2550.)
 extern "C" int sp_step(sp_sim *s, int64_t nsteps, void *stream) {
     if (!s) return fail(SP_EINVAL, "sim is NULL");
@@ -702,13 +705,14 @@ extern "C" int sp_step(sp_sim *s, int64_t nsteps, void *stream) {
         if (rc != SP_OK) return rc;
     }
     while (nsteps > 0) {
-        if (nsteps >= kGraphSteps && s->steps >= s->spl + 1) {
+        if (nsteps >= kGraphSteps && s->launched) {
             if (!s->graph[s->cur]) SP_CUDA(capture_graph(s));
             SP_CUDA(cudaGraphLaunch(s->graph[s->cur], st));
             s->steps += kGraphSteps;
             nsteps -= kGraphSteps;
         } else if (nsteps >= s->spl && s->spl > 1) {
             SP_CUDA(launch_one_step(s, st, s->spl));
+            s->launched = true;
             s->cur ^= 1;  // one launch swaps the levels, however many steps it fuses
             s->steps += s->spl;
             nsteps -= s->spl;
@@ -719,6 +723,7 @@ extern "C" int sp_step(sp_sim *s, int64_t nsteps, void *stream) {
             nsteps -= 2;
         } else {
             SP_CUDA(launch_one_step(s, st));
+            if (s->spl == 1) s->launched = true;
             s->cur ^= 1;
             s->steps += 1;
             nsteps -= 1;
