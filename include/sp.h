@@ -379,7 +379,8 @@ typedef struct sp_request {
     sp_params params;       /* dtype must be SP_F64 or SP_F32 */
     int64_t nsteps;         /* time steps to run (>= 1) */
     int return_fields;      /* nonzero: keep an FP64 host copy of the final fields */
-    int fault;              /* fault injection for tests: 0 none, 1 the allocation fails */
+    int fault;              /* fault injection for tests: 0 none, 1 the allocation fails,
+                               2 the copy of the result to the host fails */
     int priority;           /* admission priority: higher first (see sp_admission_order) */
 } sp_request;
 

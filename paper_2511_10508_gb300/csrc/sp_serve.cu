@@ -463,8 +463,10 @@ static int retire(sp_server *S, Req *q) {
             }
         }
     }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(S->stream);
-    q->mass = *S->h_scalar;
+    const cudaError_t e2 = cudaStreamSynchronize(S->stream);  // also after an error: copies under way write to host
+    if (e == cudaSuccess) e = q->r.fault == 2 ? cudaErrorUnknown : e2;
+    if (e == cudaSuccess) q->mass = *S->h_scalar;
+    else q->host = decltype(q->host)();  // (resize leaves it unwritten)
     free_buffers(S, q);
     return e == cudaSuccess ? SP_OK : SP_ECUDA;
 }
@@ -694,9 +696,10 @@ static void fill_result(const Req *q, sp_result *out) {
     out->t_submit = q->t_submit;
     out->t_admit = q->t_admit;
     out->t_finish = q->t_finish;
-    out->mass = q->mass;
-    out->fields = q->host.empty() ? nullptr : q->host.data();
-    out->n_values = q->host.size();
+    // (a pending request's result is the scheduler's, which writes it without the lock)
+    out->mass = q->done ? q->mass : 0.0;
+    out->fields = q->done && !q->host.empty() ? q->host.data() : nullptr;
+    out->n_values = q->done ? q->host.size() : 0;
 }
 
 extern "C" int sp_poll(sp_server *S, uint64_t ticket, sp_result *out) {
