@@ -201,9 +201,19 @@ def _copy(src):
         dst[:] = src
         return dst
     cut = [src.size * i // 4 for i in range(5)]
-    ts = [threading.Thread(target=np.copyto, args=(dst[a:b], src[a:b])) for a, b in zip(cut[:-1], cut[1:])]
-    for t in ts:
-        t.start()
+    parts = list(zip(cut[:-1], cut[1:]))
+    ts = []
+    try:
+        while len(parts) > 1:  # the last part is the caller's
+            a, b = parts[0]
+            t = threading.Thread(target=np.copyto, args=(dst[a:b], src[a:b]))
+            t.start()
+            ts.append(t)
+            parts.pop(0)
+    except RuntimeError:  # no thread to be had (a limit, an interpreter that is shutting down)
+        pass
+    for a, b in parts:
+        np.copyto(dst[a:b], src[a:b])
     for t in ts:
         t.join()
     return dst
