@@ -197,8 +197,9 @@ cudaError_t launch_convert_from_f64(int dtype, const double *src, void *dst, uin
 cudaError_t launch_convert_to_f64(int dtype, const void *src, double *dst, uint64_t n, cudaStream_t s);
 
 // Launch with programmatic stream serialisation (the kernel calls pdl_enter() before
-// touching global memory): the next step's CTAs are resident when this one completes,
-// about 0.5 us per launch (444 x 568 Cahn-Hilliard 2.96 -> 2.59 us per step).  Grids of many waves of
+// touching global memory).  No kernel triggers its dependents early, so the next step's CTAs start
+// as this one's exit, before its writes are flushed and its end is reported, and wait for that in
+// pdl_enter(): about 0.5 us per launch (444 x 568 Cahn-Hilliard 2.96 -> 2.59 us per step).  Grids of many waves of
 // CTAs gain nothing and lose a little (16384^2 Gray-Scott, 131072 tiles: 4.84 -> 4.90 ms),
 // so they are launched plainly.
 template <typename... KArgs, typename... Args>

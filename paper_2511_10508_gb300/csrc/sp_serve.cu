@@ -323,7 +323,7 @@ static cudaError_t upload_descriptors(sp_server *S, int Q) {
                            S->stream);
 }
 
-// `from` waits for `to`'s work so far
+// `to` waits for `from`'s work so far
 static cudaError_t chain(cudaStream_t from, cudaStream_t to, cudaEvent_t ev) {
     const cudaError_t e = cudaEventRecord(ev, from);
     return e != cudaSuccess ? e : cudaStreamWaitEvent(to, ev, 0);

@@ -7,7 +7,6 @@
 
 namespace sp {
 
-constexpr int kFftMaxN = 8192;
 constexpr int kFftMaxStages = 16;
 
 // The stages of a register transform with V points per thread: radices 2^lgr[s], the

@@ -1,10 +1,11 @@
 // sp_step_launch.cuh -- host-side launch of the step kernels: tile choices per
 // storage type and stencil radius, and the grid size.
 //
-// Grid sizing: every kernel is persistent.  The work is the flattened space of
-// (column strip or xy tile, row or plane) pairs; the grid is one resident wave
-// and each CTA (2D FP32/BF16: each warp) takes an equal contiguous share, so no
-// SM waits for a tail of long-running CTAs.
+// Grid sizing.  The streaming kernels (strips and warp rows in 2D, plane rings in 3D) are
+// persistent: the work is the flattened space of (column strip or xy tile, row or plane)
+// pairs, the grid at most one resident wave, and each CTA takes an equal contiguous run of it or
+// an equal z segment per tile (sp_split.h).  The tile and box kernels (2D FP64 on small grids, fused
+// steps on tiles, 16-bit storage with unaligned rows) take one CTA per tile or box.
 #pragma once
 
 #include <algorithm>
@@ -76,10 +77,10 @@ cudaError_t launch_tb(const StepArgs &a, cudaStream_t s) {
     return launch_pdl(kern, grid, dim3(NT), Sh::smem_bytes, s, a);
 }
 
-// 3D FP32 / BF16 Allen-Cahn and Gray-Scott with a plane ring per time level: K
-// steps per pass (temporal blocking for K = 2) on warp-row tiles of 120 x TY
-// outputs; lockstep z segments.  Needs nx a multiple of 4 and 16-byte aligned
-// fields (the runtime offers these families only then).
+// 3D FP32 / BF16 Allen-Cahn, Gray-Scott and Model C with a plane ring per time level: K
+// steps per pass (temporal blocking for K = 2) on tiles of 4 (LN - 2) x TY
+// outputs; lockstep z segments.  AL: nx a multiple of 4 and 16-byte aligned fields, which K = 2 and
+// 16-bit storage need; one step of FP32 takes any row (AL = false).
 template <int MODEL, int ST, typename T, int TY, int K, bool AL, int LN = 32>
 cudaError_t launch_tbs(const StepArgs &a, cudaStream_t s, int n_sm) {
     typedef Step3dTbsShape<MODEL, ST, T, TY, K, LN> Sh;
